@@ -140,7 +140,7 @@ struct louvain_ctx {
   int32_t* hmoved = nullptr;   // local moving: iteration + 1 of a hub's last move (by hub-list position)
   int32_t* d_gcat = nullptr;   // per graph: its class-schedule category (kCatSmall, kCatLarge, kCatSparse)
   std::vector<int32_t> hgcat;   // the same on the host
-  LMThresholds thr = {{kLMCap[0], kLMCap[1], kLMCap[2], kLMCap[3], kLMCap[4]}};   // degree mapping
+  LMThresholds thr = {{kLMCap[0], kLMCap[1], kLMCap[2], kLMCap[3], kLMCap[4]}, kBigDegree};   // degree mapping
   bool warm = false;           // this run's pass 0 starts from the membership in memb
   int64_t lm_cands = 0;        // candidate communities evaluated by this run's local moving
   louvain_ctx* sub = nullptr;  // louvain_run_partitioned: the parts' context (same device and stream)
@@ -430,6 +430,8 @@ template <typename W>
 int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool wide, int* iters_out,
                  int64_t* edges_out, int64_t* visited_out) {
   const bool async = c->opt.mode == LOUVAIN_ASYNC;
+  LMThresholds thr = c->thr;
+  thr.big = async ? kBigDegreeAsync : kBigDegree;
   // Colour classes (option): the classes are a greedy colouring of the pass
   // graph, the same for every iteration of the pass.
   const bool colour = c->opt.colour_classes != 0;
@@ -481,7 +483,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   auto reclassify_small = [&]() {
     int32_t* idx = (int32_t*)c->moves;   // free in asynchronous mode
     lm_keys_sub(g.off, c->level, sub_m, P, c->key, multi ? c->gid : nullptr, multi ? c->vo : nullptr, c->d_gcat,
-                cs, c->d_iter, c->thr, nullptr, nullptr, s);
+                cs, c->d_iter, thr, nullptr, nullptr, s);
     stable_partition(c->key, sub_m, nkeys, idx, c->key_off, c->tmp, s);
     gather_ids(idx, c->level, sub_m, c->list, s);
   };
@@ -501,12 +503,12 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   auto classify = [&](int iter, bool filter) -> int {
     if (edge_m > 0) {
       lm_keys_sub(g.off, c->level, edge_m, P, c->key, multi ? c->gid : nullptr, multi ? c->vo : nullptr, c->d_gcat,
-                  cs, c->d_iter, c->thr, filter ? c->stamp[iter & 1] : nullptr, multi ? c->d_gon : nullptr, s);
+                  cs, c->d_iter, thr, filter ? c->stamp[iter & 1] : nullptr, multi ? c->d_gon : nullptr, s);
       stable_partition(c->key, edge_m, nkeys, c->newid, c->key_off, c->tmp, s);
       gather_ids(c->newid, c->level, edge_m, c->list, s);
     } else {
       lm_keys(g.off, g.n, P, c->key, multi ? c->gid : nullptr, multi ? c->vo : nullptr, c->d_gcat, cs, c->d_iter,
-              c->thr, filter ? c->stamp[iter & 1] : nullptr, multi ? c->d_gon : nullptr, s);
+              thr, filter ? c->stamp[iter & 1] : nullptr, multi ? c->d_gon : nullptr, s);
       stable_partition(c->key, g.n, nkeys, c->list, c->key_off, c->tmp, s);
     }
     CKLAUNCH();
@@ -1846,7 +1848,7 @@ int louvain_load_parts(louvain_ctx* c, int64_t num_graphs, const int64_t* ns, co
 
 int louvain_set_mapping(louvain_ctx* c, const int32_t* thresholds) {
   if (!c) return LOUVAIN_ERR_INVALID_ARG;
-  LMThresholds th = {{kLMCap[0], kLMCap[1], kLMCap[2], kLMCap[3], kLMCap[4]}};
+  LMThresholds th = {{kLMCap[0], kLMCap[1], kLMCap[2], kLMCap[3], kLMCap[4]}, kBigDegree};
   if (thresholds) {
     for (int b = 0; b < 5; ++b) {
       if (thresholds[b] < 1 || thresholds[b] > kLMCap[b] || (b > 0 && thresholds[b] <= thresholds[b - 1]))

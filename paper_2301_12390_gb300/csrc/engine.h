@@ -10,26 +10,37 @@
 namespace gbl {
 
 // Degree classes of the local-moving phase (see local_move.cu).
-constexpr int kBuckets = 6;          // 0 thread, 1 warp/64, 2 warp/256, 3 block/2k, 4 block/8k, 5 hub
-constexpr int kHubBucket = 5;
+constexpr int kBuckets = 7;          // 0 thread, 1 warp/64, 2 warp/256, 3 block/2k, 4 block/8k, 5 block/18k, 6 hub
+constexpr int kBigBucket = 5;
+constexpr int kHubBucket = 6;
 // Degree thresholds of the local-moving mapping: bucket b < 5 takes the
-// degrees in (t[b - 1], t[b]], degrees above t[4] are hubs.  Each t[b] stays
+// degrees in (t[b - 1], t[b]]; of the degrees above t[4], those in
+// (kBlockDegree, big] go to bucket 5, the others are hubs.  Each t[b] stays
 // within its kernel's capacity kLMCap[b] (register table of 8 entries; shared
 // tables of 64, 256, 2048 and 8192 slots at most half full), so lowering one
 // moves vertices to a wider mapping with a sparser table.  The defaults are
 // the capacities; louvain_autotune picks others by timing.
 struct LMThresholds {
   int32_t t[5];
+  int32_t big;
 };
 constexpr int32_t kLMCap[5] = {8, 32, 128, 1024, 4096};
+// Bucket 5 takes the degrees its 1024 threads can hold in registers (12 each)
+// and its table of 18432 slots keeps at most two thirds full; a hub's chunks
+// go through a global table in two launches, 2.5 times the time per entry.
+// In asynchronous mode the buckets' speeds also decide which vertices commit
+// first: with everything up to 12288 taken out of the hub chain R-MAT s22's Q
+// rises by 2-4% (0.0750 -> 0.0780), with 8192 by 0-1%; up to 6144 it stays and
+// the run still gains (155 -> 148 ms over eight tolerances).
+constexpr int32_t kBlockDegree = kLMCap[4], kBigDegree = 12288, kBigDegreeAsync = 6144;
 __host__ __device__ inline int lm_bucket_of(int64_t deg, const LMThresholds& th) {
   if (deg <= 0) return -1;
 #pragma unroll
   for (int b = 0; b < 5; ++b)
     if (deg <= th.t[b]) return b;
-  return 5;
+  return deg > kBlockDegree && deg <= th.big ? kBigBucket : kHubBucket;
 }
-constexpr int64_t kHubChunkEntries = 1024;   // entries per insert block of a hub
+constexpr int64_t kHubChunkEntries = 4096;   // entries per insert block of a hub
 constexpr int64_t kSlotChunk = 4096;         // table slots per scan block (hubs and large communities)
 
 // Community classes of the aggregation phase by total member degree.

@@ -11,7 +11,8 @@
 //   bucket 2  degree 33..128    one warp per vertex, 256-slot shared table
 //   bucket 3  degree 129..1024  one block per vertex, 2048-slot shared table
 //   bucket 4  degree 1025..4096 one block per vertex, 8192-slot shared table
-//   bucket 5  degree > 4096     hub: several blocks insert into a global
+//   bucket 5  degree 4097..12288  one block per vertex, 18432-slot shared table
+//   bucket 6  larger degrees    hub: several blocks insert into a global
 //                               table of 2*degree slots, one block decides
 //
 // Synchronous mode (Jacobi): decisions read the state at the start of the
@@ -196,37 +197,56 @@ __device__ __forceinline__ bool is_active(const LMArgs<W>& a, const IterView& iv
   return !a.prune || iv.iter == 0 || iv.sr[i] == iv.iter;
 }
 
-// What a per-vertex kernel needs of list entry vi before its row: loaded one
-// vertex ahead so that these loads overlap the previous vertex.
-struct VertexInfo {
-  int32_t i, d, szd;
-  bool on;        // in range, active and its graph still iterating
-  int graph;
-  int64_t b, e;
-  long long Ki, M, sd;
+// What a warp or block needs of a vertex before its row.
+struct VertexRow {
+  int32_t i, d;   // the vertex and its community
+  int deg;
+  int64_t b;      // first entry of its row
+  long long Ki;
+  int graph;      // set by window_row
+  long long M;
 };
 
-template <typename W, bool ASYNC, int LD = (ASYNC ? 1 : 0)>
-__device__ __forceinline__ VertexInfo vertex_info(const LMArgs<W>& a, const IterView& iv,
-                                                  const int32_t* __restrict__ verts, int nverts, int vi) {
-  VertexInfo v;
-  v.on = false;
-  v.i = 0;
-  v.d = 0;
-  v.szd = 0;
+// A window of 32 list entries first, first + stride, ...: lane l loads entry
+// first + l * stride, so one chain of dependent loads (list entry, stamp, row
+// bounds, community, degree) serves 32 vertices and inactive vertices cost
+// nothing more.  Returns the lanes whose vertex is visited in this iteration.
+// A vertex's own community only changes by its own commit, so it may be read
+// ahead; its community's total and size are read when its row is.
+template <typename W, int LD>
+__device__ __forceinline__ unsigned vertex_window(const LMArgs<W>& a, const IterView& iv,
+                                                  const int32_t* __restrict__ verts, int64_t nverts, int64_t first,
+                                                  int64_t stride, int lane, VertexRow& r) {
+  bool on = false;
+  const int64_t at = first + lane * stride;
+  r = VertexRow{0, 0, 0, 0, 0, 0, 0};
+  if (at < nverts) {
+    r.i = verts[at];
+    if (is_active(a, iv, r.i) && (!a.gid || a.g_on[a.gid[r.i]])) {
+      on = true;
+      r.b = a.off[r.i];
+      r.deg = (int)(a.off[r.i + 1] - r.b);
+      r.d = ld_state<LD == 2 ? 2 : 1>(a.memb + r.i);
+      r.Ki = a.K[r.i];
+    }
+  }
+  return __ballot_sync(0xffffffffu, on);
+}
+
+// Lane src's vertex of a window, to every lane.
+template <typename W>
+__device__ __forceinline__ VertexRow window_row(const LMArgs<W>& a, const VertexRow& r, int src) {
+  VertexRow v;
+  v.i = __shfl_sync(0xffffffffu, r.i, src);
+  v.d = __shfl_sync(0xffffffffu, r.d, src);
+  v.deg = __shfl_sync(0xffffffffu, r.deg, src);
+  v.b = __shfl_sync(0xffffffffu, r.b, src);
+  v.Ki = __shfl_sync(0xffffffffu, r.Ki, src);
   v.graph = 0;
-  v.b = v.e = 0;
-  v.Ki = v.M = v.sd = 0;
-  if (vi >= nverts) return v;
-  v.i = verts[vi];
-  v.b = a.off[v.i];
-  v.e = a.off[v.i + 1];
-  v.d = ld_state<LD == 2 ? 2 : 1>(a.memb + v.i);
-  v.Ki = a.K[v.i];
-  v.on = is_active(a, iv, v.i) && graph_of(a, v.i, &v.M, &v.graph);
-  if (v.on) {   // the loads that depend on d, only for a vertex that is visited
-    v.sd = ld_state<LD>(a.sig + v.d);
-    v.szd = ld_state<LD>(a.csize + v.d);
+  v.M = a.M;
+  if (a.gid) {
+    v.graph = a.gid[v.i];
+    v.M = a.Mg[v.graph];
   }
   return v;
 }
@@ -490,112 +510,120 @@ __global__ void __launch_bounds__(128) lm_thread_sorted(LMArgs<W> a, const int32
 
 // ------------------------------------------ buckets 1-2: warp per vertex
 
+// Tallies a warp keeps in registers while it walks its vertices, added to the
+// block's accumulator once at the end (all 32 lanes call add).
+struct WarpTally {
+  unsigned long long edges = 0;
+  unsigned visited = 0, cands = 0;   // per thread, of one launch
+  __device__ __forceinline__ void add(BlockAcc& acc) {
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) edges += __shfl_xor_sync(0xffffffffu, edges, m);
+    unsigned long long c = cands;
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) c += __shfl_xor_sync(0xffffffffu, c, m);
+    visited = __reduce_add_sync(0xffffffffu, visited);
+    if ((threadIdx.x & 31) == 0) {
+      if (edges) atomicAdd(&acc.edges, edges);
+      if (visited) atomicAdd(&acc.visited, (unsigned long long)visited);
+      if (c) atomicAdd(&acc.cands, c);
+    }
+  }
+};
+
+// The U entries of row v that this thread holds (entry u * step + lane0),
+// their communities gathered with all loads in flight; kEmpty for none and
+// for a self-loop.  Rounds from nu on hold nothing for any lane of the warp.
+template <int U, int LD, typename W, typename V>
+__device__ __forceinline__ void row_communities(const LMArgs<W>& a, const VertexRow& v, int lane0, int step, int nu,
+                                                int32_t (&cc)[U], V (&ww)[U]) {
+  const int32_t* __restrict__ col = a.col + v.b;
+  const W* __restrict__ wt = a.wt + v.b;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    cc[u] = v.i;
+    ww[u] = 0;
+    if (u < nu) {
+      const int x = u * step + lane0;
+      if (x < v.deg) {
+        cc[u] = col[x];
+        ww[u] = (V)wt[x];
+      }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) cc[u] = u < nu && cc[u] != v.i ? ld_state<LD>(a.memb + cc[u]) : kEmpty;
+}
+
 // One vertex of degree <= U * 32 by one warp: its neighbour communities summed
 // in the warp's shared table (CAP slots, left empty again), the best score
 // against its own community's, the move committed and its neighbours marked.
-// SIZES: a singleton under the guard loads its candidates' sizes with their
-// totals (one dependent load less before the decision; off where the
+// The lane whose entry claims a slot keeps the community and the slot in
+// registers: it asks for the community's total at once, and after the sums
+// are complete it alone evaluates and clears the slot, so nothing scans the
+// table.  SIZES: a singleton under the guard loads its candidates' sizes with
+// their totals (one dependent load less before the decision; off where the
 // registers would spill).
 template <typename W, bool WIDE, bool ASYNC, int CAP, int U, int LD, bool SIZES>
 __device__ __forceinline__ void warp_vertex(const LMArgs<W>& a, const IterView& iv, BlockAcc& acc, int32_t* keys,
-                                            typename TableVal<WIDE>::T* vals, const VertexInfo& cur, int lane,
-                                            bool& ok) {
+                                            typename TableVal<WIDE>::T* vals, const VertexRow& v, int lane, bool& ok,
+                                            unsigned& cands) {
   typedef typename Arith<WIDE>::S S;
   typedef typename TableVal<WIDE>::T V;
-  const int32_t i = cur.i, d = cur.d;
-  const int64_t b = cur.b, e = cur.e;
-  const long long Ki = cur.Ki, M = cur.M;
-  const int graph = cur.graph;
-  for (int64_t x0 = b; x0 < e; x0 += U * kWarp) {
-    // rounds of 32 entries that hold at least one (the rest are skipped)
-    const int nu = (int)min((int64_t)U, (e - x0 + kWarp - 1) / kWarp);
-    int32_t cc[U];
-    unsigned long long ww[U];
+  const long long sd = ld_state<LD>(a.sig + v.d);
+  const int32_t szd = ld_state<LD>(a.csize + v.d);
+  // rounds of 32 entries that hold at least one (the rest are skipped)
+  const int nu = (v.deg + kWarp - 1) / kWarp;
+  int32_t cc[U];
+  V ww[U];
+  int hs[U];
+  row_communities<U, LD>(a, v, lane, kWarp, nu, cc, ww);
+  const unsigned fresh = table_add_row<CAP, U, V>(keys, vals, cc, ww, nu, hs, &ok);
+  const bool want_size = SIZES && a.guard && szd == 1;
+  long long sg[U];
+  bool one[U];   // the candidate is a singleton (asked only for the guard)
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      cc[u] = i;
-      ww[u] = 0ull;
-      if (u < nu) {
-        const int64_t x = x0 + u * kWarp + lane;
-        if (x < e) {
-          cc[u] = a.col[x];
-          ww[u] = (unsigned long long)a.wt[x];
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) cc[u] = cc[u] != i ? ld_state<LD>(a.memb + cc[u]) : kEmpty;
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (cc[u] != kEmpty) ok &= table_add_pow2<CAP, V>(keys, vals, cc[u], ww[u]);
+  for (int u = 0; u < U; ++u) {
+    const bool cand = ((fresh >> u) & 1u) && cc[u] != v.d;
+    sg[u] = cand ? ld_state<LD>(a.sig + cc[u]) : 0;
+    one[u] = cand && want_size && cc[u] > v.d && ld_state<LD>(a.csize + cc[u]) == 1;
   }
-  __syncwarp();
-  // a singleton under the guard loads its candidates' sizes with their
-  // totals and carries the best one's through the reduction
-  const bool want_size = SIZES && a.guard && cur.szd == 1;
-  unsigned long long kid = 0;
+  __syncwarp();   // the sums are complete
+  V kid = 0;
   S bg = Arith<WIDE>::lowest();
   int32_t bc = -1, bsz = 0;
-  unsigned ncand = 0;
 #pragma unroll
-  for (int t0 = 0; t0 < CAP; t0 += kWarp * 4) {
-    int32_t cs[4];
-    long long sg[4];
-    unsigned long long vs[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int t = t0 + u * kWarp + lane;
-      cs[u] = t < CAP ? keys[t] : kEmpty;
-      vs[u] = t < CAP ? vals[t] : 0ull;
+  for (int u = 0; u < U; ++u) {
+    if (!((fresh >> u) & 1u)) continue;
+    const V sum = vals[hs[u]];
+    if (cc[u] != v.d) {
+      ++cands;
+      const S g = Arith<WIDE>::score(v.M, (long long)sum, v.Ki, sg[u]);
+      if (better(g, cc[u], bg, bc)) { bg = g; bc = cc[u]; bsz = one[u] ? 1 : 0; }
+    } else {
+      kid = sum;
     }
-    bool one[4];   // the candidate is a singleton (asked only for the guard)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const bool cand = cs[u] != kEmpty && cs[u] != d;
-      sg[u] = cand ? ld_state<LD>(a.sig + cs[u]) : 0;
-      one[u] = cand && want_size && cs[u] > d && ld_state<LD>(a.csize + cs[u]) == 1;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int t = t0 + u * kWarp + lane;
-      if (cs[u] != kEmpty) {
-        if (cs[u] != d) {
-          ++ncand;
-          S g = Arith<WIDE>::score(M, (long long)vs[u], Ki, sg[u]);
-          if (better(g, cs[u], bg, bc)) { bg = g; bc = cs[u]; bsz = one[u] ? 1 : 0; }
-        } else {
-          kid = vs[u];
-        }
-        keys[t] = kEmpty;
-        vals[t] = 0;
-      }
-    }
+    keys[hs[u]] = kEmpty;
+    vals[hs[u]] = 0;
   }
   if (want_size) warp_argmax_carry(bg, bc, bsz);
   else warp_argmax(bg, bc);
-  ncand = __reduce_add_sync(0xffffffffu, ncand);
   {
     const unsigned has = __ballot_sync(0xffffffffu, kid != 0);
-    kid = has ? __shfl_sync(0xffffffffu, kid, __ffs(has) - 1) : 0ull;
+    kid = has ? __shfl_sync(0xffffffffu, kid, __ffs(has) - 1) : (V)0;
   }
   bool moved = false;
-  if (lane == 0) {
-    atomicAdd(&acc.cands, (unsigned long long)ncand);
-    atomicAdd(&acc.edges, (unsigned long long)(e - b));
-    atomicAdd(&acc.visited, 1ull);
-    moved = commit_choice<W, WIDE, ASYNC, LD>(a, acc, i, d, Ki, cur.sd, cur.szd, bg, bc, kid, M, graph, nullptr,
+  if (lane == 0)
+    moved = commit_choice<W, WIDE, ASYNC, LD>(a, acc, v.i, v.d, v.Ki, sd, szd, bg, bc, kid, v.M, v.graph, nullptr,
                                               want_size ? bsz : -1);
-  }
   moved = __shfl_sync(0xffffffffu, moved, 0);
-  if (moved && a.prune) mark_row<U>(a, iv, i, b, e, lane, kWarp);
+  if (moved && a.prune) mark_row<U>(a, iv, v.i, v.b, v.b + v.deg, lane, kWarp);
 }
 
-// U entries per lane are loaded and gathered before any insert (U * 32 covers
-// the bucket's largest degree), so their memory latencies overlap.
+// U entries per lane cover the bucket's largest degree: the row is loaded and
+// gathered before any insert, so its memory latencies overlap.
 template <typename W, bool WIDE, bool ASYNC, int CAP, int U>
 __global__ void __launch_bounds__(256, 4) lm_warp(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
   const IterView iv = iter_view(a);
-  typedef typename Arith<WIDE>::S S;
   typedef typename TableVal<WIDE>::T V;
   constexpr int WPB = 8;
   __shared__ int32_t skeys[WPB][CAP];
@@ -608,16 +636,23 @@ __global__ void __launch_bounds__(256, 4) lm_warp(LMArgs<W> a, const int32_t* __
   for (int t = lane; t < CAP; t += kWarp) { keys[t] = kEmpty; vals[t] = 0; }
   __syncthreads();
   bool ok = true;
-  const int stride = gridDim.x * WPB;
-  VertexInfo nx = vertex_info<W, ASYNC>(a, iv, verts, nverts, blockIdx.x * WPB + wib);
-  for (int vi = blockIdx.x * WPB + wib; vi < nverts; vi += stride) {
-    const VertexInfo cur = nx;
-    nx = vertex_info<W, ASYNC>(a, iv, verts, nverts, vi + stride);
-    if (!cur.on) continue;
-    warp_vertex<W, WIDE, ASYNC, CAP, U, (ASYNC ? 1 : 0), (CAP <= 64 && !WIDE)>(a, iv, acc, keys, vals, cur, lane,
-                                                                                 ok);
-    __syncwarp();
+  WarpTally tally;
+  const int64_t stride = (int64_t)gridDim.x * WPB;
+  for (int64_t w0 = (int64_t)blockIdx.x * WPB + wib; w0 < nverts; w0 += kWarp * stride) {
+    VertexRow r;
+    unsigned live = vertex_window<W, (ASYNC ? 1 : 0)>(a, iv, verts, nverts, w0, stride, lane, r);
+    if ((live >> lane) & 1u) {
+      tally.edges += (unsigned)r.deg;
+      ++tally.visited;
+    }
+    for (; live; live &= live - 1) {
+      const VertexRow v = window_row(a, r, __ffs(live) - 1);
+      warp_vertex<W, WIDE, ASYNC, CAP, U, (ASYNC ? 1 : 0), (CAP <= 64 && !WIDE)>(a, iv, acc, keys, vals, v, lane, ok,
+                                                                                   tally.cands);
+      __syncwarp();
+    }
   }
+  tally.add(acc);
   if (!__all_sync(0xffffffffu, ok) && lane == 0) atomicOr(&acc.error, kErrProbe);
   __syncthreads();
   acc_flush(acc, a.ctr);
@@ -647,6 +682,7 @@ __global__ void __launch_bounds__(256, 3) lm_class(LMArgs<W> a, const int32_t* _
   for (int t = lane; t < CAP; t += kWarp) { keys[t] = kEmpty; vals[t] = 0; }
   __syncthreads();
   bool ok = true;
+  WarpTally tally;
   const int64_t r0 = ko[ch], n0 = ko[ch + 1] - r0;
   const int64_t r1 = ko[P + ch], n1 = ko[P + ch + 1] - r1;
   const int64_t r2 = ko[2 * P + ch], n2 = ko[2 * P + ch + 1] - r2;
@@ -661,17 +697,23 @@ __global__ void __launch_bounds__(256, 3) lm_class(LMArgs<W> a, const int32_t* _
     }
     const int64_t u = t - m0;
     const int64_t idx = u < n1 ? r1 + u : r2 + (u - n1);
-    const VertexInfo cur = vertex_info<W, ASYNC>(a, iv, list + idx, 1, 0);
-    if (!cur.on) continue;
-    warp_vertex<W, WIDE, ASYNC, CAP, U, (ASYNC ? 1 : 0), !WIDE>(a, iv, acc, keys, vals, cur, lane, ok);
+    VertexRow r;
+    if (!vertex_window<W, (ASYNC ? 1 : 0)>(a, iv, list + idx, 1, 0, 1, lane, r)) continue;
+    if (lane == 0) {
+      tally.edges += (unsigned)r.deg;
+      ++tally.visited;
+    }
+    const VertexRow v = window_row(a, r, 0);
+    warp_vertex<W, WIDE, ASYNC, CAP, U, (ASYNC ? 1 : 0), !WIDE>(a, iv, acc, keys, vals, v, lane, ok, tally.cands);
     __syncwarp();
   }
+  tally.add(acc);
   if (!__all_sync(0xffffffffu, ok) && lane == 0) atomicOr(&acc.error, kErrProbe);
   __syncthreads();
   acc_flush(acc, a.ctr);
 }
 
-// ----------------------------------------- buckets 3-4: block per vertex
+// ----------------------------------------- buckets 3-5: block per vertex
 
 // A decided move waiting for the block to commit it, with its row bounds
 // (for the pruning marks).
@@ -698,8 +740,12 @@ __device__ __forceinline__ void flush_moves(const LMArgs<W>& a, const IterView& 
       a.moves[pos] = make_int2(m.i, m.c);
     }
   }
-  if (a.prune)   // one warp per move, the warps' moves in parallel
+  if (!a.prune) return;
+  if (nthr >= 512) {   // long rows: the whole block marks one after the other
+    for (int t = 0; t < n; ++t) mark_row<8>(a, iv, q[t].i, q[t].b, q[t].e, tid, nthr);
+  } else {             // one warp per move, the warps' moves in parallel
     for (int t = tid >> 5; t < n; t += nthr >> 5) mark_row<8>(a, iv, q[t].i, q[t].b, q[t].e, tid & 31, kWarp);
+  }
 }
 
 // Decide (no commit yet): the exact gain of the best candidate against the
@@ -727,143 +773,130 @@ __device__ __forceinline__ bool decide_move(const LMArgs<W>& a, BlockAcc& acc, i
   return true;
 }
 
+// One vertex at a time by a block of THREADS threads holding U entries each
+// (U * THREADS covers the bucket's largest degree).  As in warp_vertex the
+// thread whose entry claims a table slot evaluates and clears it from its own
+// registers, so no list of touched slots and no scan of the table is needed.
 // Two barriers per vertex: the small shared values alternate between two
 // copies by vertex parity, so the next vertex can start while warp 0 still
-// reduces and decides; moves queue in shared memory and are committed by the
-// whole block when the queue fills and at the end.
-template <typename W, bool WIDE, bool ASYNC, int CAP, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : 2)
+// decides; moves queue in shared memory and are committed by the whole block
+// when the queue fills and at the end.
+// Bound by the latency of row, community and total loads and by issue slots
+// (R-MAT of 2M vertices, degrees 129-1024: 340 thread instructions an entry
+// with the touched-slot list and its scan, 48% of the issue slots).  R-MAT of
+// 4.2M vertices, synchronous: 143.4 -> 117.8 ms a run with this kernel, its
+// 12288-degree instance in place of the hub chain and 4096-entry hub chunks.
+template <typename W, bool WIDE, bool ASYNC, int CAP, int THREADS, int U>
+__global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ? 2 : 1)
     lm_block(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
   const IterView iv = iter_view(a);
   typedef typename Arith<WIDE>::S S;
   typedef typename TableVal<WIDE>::T V;
   constexpr int NW = THREADS / kWarp;
-  constexpr int U = 4;
+  constexpr int LD = ASYNC ? 1 : 0;
   constexpr int QCAP = 64;
-  // dynamic shared memory: values (CAP V), keys (CAP i32), touched slots (CAP/2 u16)
+  // dynamic shared memory: values (CAP V), keys (CAP i32)
   extern __shared__ unsigned long long dyn[];
   V* vals = (V*)dyn;
   int32_t* keys = (int32_t*)(vals + CAP);
-  uint16_t* touched = (uint16_t*)(keys + CAP);
   __shared__ BlockAcc acc;
   __shared__ S red_g[2][NW];
   __shared__ int32_t red_c[2][NW];
   __shared__ unsigned long long s_kid[2];
-  __shared__ int s_nt[2];
   __shared__ PendingMove queue[QCAP];
   __shared__ int q_n;
+  __shared__ VertexRow win[kWarp];
+  __shared__ unsigned s_live[2];   // by window parity: an empty window has no other barrier
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   acc_init(acc);
-  if (threadIdx.x == 0) { s_nt[0] = s_nt[1] = 0; s_kid[0] = s_kid[1] = 0; q_n = 0; }
+  if (threadIdx.x == 0) { s_kid[0] = s_kid[1] = 0; q_n = 0; }
   for (int t = threadIdx.x; t < CAP; t += THREADS) { keys[t] = kEmpty; vals[t] = 0; }
   __syncthreads();
   bool ok = true;
-  int p = 0;
-  // The next vertex's list entry, activity, row bounds, community and degree
-  // are loaded while the current one is processed.
-  VertexInfo nx = vertex_info<W, ASYNC>(a, iv, verts, nverts, blockIdx.x);
-  for (int vi = blockIdx.x; vi < nverts; vi += gridDim.x) {
-    const VertexInfo cur = nx;
-    if (!cur.on) {   // uniform across the block
-      nx = vertex_info<W, ASYNC>(a, iv, verts, nverts, vi + gridDim.x);
-      continue;
-    }
-    const int32_t i = cur.i, d = cur.d;
-    const int64_t b = cur.b, e = cur.e;
-    const long long Ki = cur.Ki, M = cur.M;
-    const int graph = cur.graph;
-    for (int64_t x0 = b; x0 < e; x0 += U * THREADS) {
-      // this warp's rounds that hold at least one entry (the rest skipped)
-      const int64_t rem = e - x0 - wid * kWarp;
-      const int nu = rem <= 0 ? 0 : (int)min((int64_t)U, (rem + THREADS - 1) / THREADS);
-      int32_t cc[U];
-      unsigned long long ww[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        cc[u] = i;
-        ww[u] = 0ull;
-        if (u < nu) {
-          const int64_t x = x0 + u * THREADS + threadIdx.x;
-          if (x < e) {
-            cc[u] = a.col[x];
-            ww[u] = (unsigned long long)a.wt[x];
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) cc[u] = cc[u] != i ? ld_memb<ASYNC>(a.memb + cc[u]) : kEmpty;
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (u >= nu) break;
-        bool fresh = false;
-        int h = -1;
-        if (cc[u] != kEmpty) {
-          h = table_add_pow2_slot<CAP, V>(keys, vals, cc[u], ww[u], &fresh);
-          if (h < 0) ok = false;
-        }
-        // one append per warp for the new keys of its lanes
-        const unsigned m = __ballot_sync(0xffffffffu, fresh);
-        int base = 0;
-        if (lane == 0 && m) base = atomicAdd(&s_nt[p], __popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (fresh) touched[base + __popc(m & lanemask_lt_lm())] = (uint16_t)h;
-      }
-    }
-    nx = vertex_info<W, ASYNC>(a, iv, verts, nverts, vi + gridDim.x);
-    __syncthreads();   // B1: table complete; warp 0 has finished the previous vertex
-    if (q_n >= QCAP) {   // uniform: q_n was last written before this barrier
-      flush_moves<W, ASYNC>(a, iv, queue, q_n, threadIdx.x, THREADS);
-      __syncthreads();
-      if (threadIdx.x == 0) q_n = 0;
-    }
-    if (threadIdx.x == 0) { s_nt[p ^ 1] = 0; s_kid[p ^ 1] = 0; }   // the next vertex's copies
-    const int nt = s_nt[p];
-    S bg = Arith<WIDE>::lowest();
-    int32_t bc = -1;
-    for (int t0 = 0; t0 < nt; t0 += U * THREADS) {
-      const int rem = nt - t0 - wid * kWarp;
-      const int nu = rem <= 0 ? 0 : min(U, (rem + THREADS - 1) / THREADS);
-      int hs[U];
-      int32_t cs[U];
-      long long sg[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int t = t0 + u * THREADS + threadIdx.x;
-        hs[u] = u < nu && t < nt ? (int)touched[t] : -1;
-        cs[u] = hs[u] >= 0 ? keys[hs[u]] : kEmpty;
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) sg[u] = (cs[u] != kEmpty && cs[u] != d) ? ld_sig<ASYNC>(a.sig + cs[u]) : 0;
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (hs[u] < 0) continue;
-        if (cs[u] != d) {
-          S g = Arith<WIDE>::score(M, (long long)vals[hs[u]], Ki, sg[u]);
-          if (better(g, cs[u], bg, bc)) { bg = g; bc = cs[u]; }
-        } else {
-          s_kid[p] = vals[hs[u]];
-        }
-        keys[hs[u]] = kEmpty;
-        vals[hs[u]] = 0;
-      }
-    }
-    warp_argmax(bg, bc);
-    if (lane == 0) { red_g[p][wid] = bg; red_c[p][wid] = bc; }
-    __syncthreads();   // B2: candidates evaluated, table clear
+  int p = 0, wp = 0;
+  WarpTally tally;
+  // the next 32 vertices, loaded by warp 0 (in shared memory: a row's bounds,
+  // community and degree are read where they are used instead of held)
+  for (int64_t w0 = blockIdx.x; w0 < nverts; w0 += (int64_t)kWarp * gridDim.x, wp ^= 1) {
     if (wid == 0) {
-      bg = lane < NW ? red_g[p][lane] : Arith<WIDE>::lowest();
-      bc = lane < NW ? red_c[p][lane] : -1;
-      warp_argmax(bg, bc);
-      if (lane == 0) {
-        atomicAdd(&acc.edges, (unsigned long long)(e - b));
-        atomicAdd(&acc.visited, 1ull);
-        atomicAdd(&acc.cands, (unsigned long long)(s_nt[p] - (s_kid[p] != 0 ? 1 : 0)));
-        if (decide_move<W, WIDE, ASYNC>(a, acc, d, Ki, cur.sd, cur.szd, bg, bc, s_kid[p], M, graph))
-          queue[q_n++] = PendingMove{i, bc, d, 0, b, e};
+      VertexRow r;
+      const unsigned on = vertex_window<W, LD>(a, iv, verts, nverts, w0, gridDim.x, lane, r);
+      if ((on >> lane) & 1u) {
+        tally.edges += (unsigned)r.deg;
+        ++tally.visited;
       }
+      win[lane] = r;
+      if (lane == 0) s_live[wp] = on;
     }
-    p ^= 1;
+    __syncthreads();
+    for (unsigned live = s_live[wp]; live; live &= live - 1) {   // uniform across the block
+      const VertexRow& v = win[__ffs(live) - 1];
+      long long sd = 0;
+      int32_t szd = 0;
+      if (wid == 0) {   // for the decision
+        sd = ld_state<LD>(a.sig + v.d);
+        szd = ld_state<LD>(a.csize + v.d);
+      }
+      // this warp's rounds that hold at least one entry (the rest skipped)
+      const int rem = v.deg - wid * kWarp;
+      const int nu = rem <= 0 ? 0 : (rem + THREADS - 1) / THREADS;
+      int32_t cc[U];
+      int hs[U];
+      unsigned fresh;
+      {
+        V ww[U];
+        row_communities<U, LD>(a, v, (int)threadIdx.x, THREADS, nu, cc, ww);
+        fresh = table_add_row<CAP, U, V>(keys, vals, cc, ww, nu, hs, &ok);
+      }
+      __syncthreads();   // B1: table complete; warp 0 has finished the previous vertex
+      if (q_n >= QCAP) {   // uniform: q_n was last written before this barrier
+        flush_moves<W, ASYNC>(a, iv, queue, q_n, threadIdx.x, THREADS);
+        __syncthreads();
+        if (threadIdx.x == 0) q_n = 0;
+      }
+      if (threadIdx.x == 0) s_kid[p ^ 1] = 0;   // the next vertex's copy
+      const long long M = a.gid ? a.Mg[a.gid[v.i]] : a.M, Ki = v.Ki;
+      const int32_t d = v.d;
+      S bg = Arith<WIDE>::lowest();
+      int32_t bc = -1;
+#pragma unroll
+      for (int u0 = 0; u0 < U; u0 += 4) {
+        if (u0 >= nu) break;
+        long long sg[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          sg[j] = ((fresh >> (u0 + j)) & 1u) && cc[u0 + j] != d ? ld_state<LD>(a.sig + cc[u0 + j]) : 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int u = u0 + j;
+          if (!((fresh >> u) & 1u)) continue;
+          const V sum = vals[hs[u]];
+          if (cc[u] != d) {
+            ++tally.cands;
+            const S g = Arith<WIDE>::score(M, (long long)sum, Ki, sg[j]);
+            if (better(g, cc[u], bg, bc)) { bg = g; bc = cc[u]; }
+          } else {
+            s_kid[p] = sum;
+          }
+          keys[hs[u]] = kEmpty;
+          vals[hs[u]] = 0;
+        }
+      }
+      warp_argmax(bg, bc);
+      if (lane == 0) { red_g[p][wid] = bg; red_c[p][wid] = bc; }
+      __syncthreads();   // B2: candidates evaluated, table clear
+      if (wid == 0) {
+        bg = lane < NW ? red_g[p][lane] : Arith<WIDE>::lowest();
+        bc = lane < NW ? red_c[p][lane] : -1;
+        warp_argmax(bg, bc);
+        if (lane == 0 &&
+            decide_move<W, WIDE, ASYNC>(a, acc, d, Ki, sd, szd, bg, bc, s_kid[p], M, a.gid ? a.gid[v.i] : 0))
+          queue[q_n++] = PendingMove{v.i, bc, d, 0, v.b, v.b + v.deg};
+      }
+      p ^= 1;
+    }
   }
+  tally.add(acc);
   __syncthreads();
   flush_moves<W, ASYNC>(a, iv, queue, q_n, threadIdx.x, THREADS);
   if (!ok) atomicOr(&acc.error, kErrProbe);
@@ -871,12 +904,12 @@ __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : 2)
   acc_flush(acc, a.ctr);
 }
 
-// ------------------------------------------------- bucket 5: hub vertices
+// ------------------------------------------------- bucket 6: hub vertices
 //
 // Hub h of a class owns global table slots [hbase[h] - hbase[0], + 2 deg):
 // every class's tables start at slot 0, so a class reuses the slots the
 // previous class's scan just cleared, which are still in L2.
-// 1. insert: blocks are (hub, 2048-entry chunk) pairs; each sums its chunk
+// 1. insert: blocks are (hub, kHubChunkEntries-entry chunk) pairs; each sums its chunk
 //    per community in shared memory, then adds each distinct community once
 //    to the hub's global table;
 // 2. scan: blocks are (hub, 4096-slot chunk) pairs; each evaluates the gain
@@ -889,65 +922,49 @@ constexpr int kHubChunk = (int)kHubChunkEntries;
 
 constexpr int kItemCache = 512;   // hub prefix entries a block copies to shared memory
 
+constexpr int kHubThreads = 512;
+
 template <typename W, bool WIDE, bool ASYNC>
-__global__ void __launch_bounds__(256) lm_hub_insert(LMArgs<W> a, const int32_t* __restrict__ hubs, int nhubs,
-                                                     const int64_t* __restrict__ chunk_pre) {
+__global__ void __launch_bounds__(kHubThreads) lm_hub_insert(LMArgs<W> a, const int32_t* __restrict__ hubs, int nhubs,
+                                                             const int64_t* __restrict__ chunk_pre) {
   typedef typename TableVal<WIDE>::T V;
   const IterView iv = iter_view(a);
   constexpr int CAP = 2 * kHubChunk;
+  constexpr int U = kHubChunk / kHubThreads;
+  static_assert(U >= 1 && kHubChunk % kHubThreads == 0, "a chunk covers whole rounds of the block");
   extern __shared__ unsigned long long hdyn[];
   V* svals = (V*)hdyn;
   int32_t* skeys = (int32_t*)(svals + CAP);
   __shared__ int64_t s_pre[kItemCache + 1];
   const int h = block_item<kItemCache>(chunk_pre, nhubs, blockIdx.x, s_pre);
-  const int32_t i = hubs[h];
-  if (!is_active(a, iv, i)) return;   // uniform across the block
-  {
-    long long M;
-    int graph;
-    if (!graph_of(a, i, &M, &graph)) return;
-  }
+  VertexRow v;
+  v.i = hubs[h];
+  if (!is_active(a, iv, v.i)) return;   // uniform across the block
+  if (!graph_of(a, v.i, &v.M, &v.graph)) return;
   const int64_t q = (int64_t)blockIdx.x - (chunk_pre[h] - chunk_pre[0]);
-  for (int t = threadIdx.x; t < CAP; t += blockDim.x) { skeys[t] = kEmpty; svals[t] = 0; }
+  for (int t = threadIdx.x; t < CAP; t += kHubThreads) { skeys[t] = kEmpty; svals[t] = 0; }
   __syncthreads();
-  const int64_t b = a.off[i], e = a.off[i + 1];
+  const int64_t b = a.off[v.i], e = a.off[v.i + 1];
   const int64_t base = a.hbase[h] - a.hbase[0];   // the class's tables start at slot 0
   const uint32_t cap = (uint32_t)(2 * (e - b));
-  const int64_t x0 = b + q * kHubChunk, x1 = min(e, x0 + kHubChunk);
+  v.b = b + q * kHubChunk;
+  v.deg = (int)min((int64_t)kHubChunk, e - v.b);
   bool ok = true;
-  constexpr int U = kHubChunk / 256;
-  static_assert(U >= 1 && kHubChunk % 256 == 0, "a chunk covers whole rounds of 256 threads");
-  for (int64_t y = x0; y < x1; y += U * 256) {
-    int32_t cc[U];
-    unsigned long long ww[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int64_t x = y + u * 256 + threadIdx.x;
-      const bool v = x < x1;
-      cc[u] = v ? a.col[x] : i;
-      ww[u] = v ? (unsigned long long)a.wt[x] : 0ull;
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) cc[u] = cc[u] != i ? ld_memb<ASYNC>(a.memb + cc[u]) : kEmpty;
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (cc[u] != kEmpty) ok &= table_add_pow2<CAP, V>(skeys, svals, cc[u], ww[u]);
-  }
+  int32_t cc[U];
+  V ww[U];
+  int hs[U];
+  row_communities<U, (ASYNC ? 1 : 0)>(a, v, (int)threadIdx.x, kHubThreads, U, cc, ww);
+  const unsigned fresh = table_add_row<CAP, U, V>(skeys, svals, cc, ww, U, hs, &ok);
   __syncthreads();
-  int32_t* keys = a.hkeys + base;
-  unsigned long long* vals = a.hvals + base;
-  constexpr int J = 8;
-  for (int t0 = 0; t0 < CAP; t0 += J * 256) {
-    int32_t kk[J];
-    unsigned long long vv[J];
+  // the thread that claimed a slot adds its sum to the hub's table
+  unsigned long long vv[U];
 #pragma unroll
-    for (int j = 0; j < J; ++j) {   // slots past CAP (a table smaller than J * 256) read as empty
-      const int t = t0 + j * 256 + (int)threadIdx.x;
-      kk[j] = t < CAP ? skeys[t] : kEmpty;
-      vv[j] = t < CAP ? (unsigned long long)svals[t] : 0ull;
-    }
-    ok &= gtable_add_many<J>(keys, vals, cap, kk, vv);
+  for (int u = 0; u < U; ++u) {
+    const bool mine = (fresh >> u) & 1u;
+    vv[u] = mine ? (unsigned long long)svals[hs[u]] : 0ull;
+    if (!mine) cc[u] = kEmpty;
   }
+  ok &= gtable_add_many<U>(a.hkeys + base, a.hvals + base, cap, cc, vv);
   if (!ok) atomicOr(&a.ctr->error, kErrProbe);
 }
 
@@ -1117,6 +1134,15 @@ int grid_for(K kernel, int threads, size_t smem, int work_blocks) {
   return g < 1 ? 1 : g;
 }
 
+template <typename W, bool WIDE, bool ASYNC, int CAP, int THREADS, int U>
+void launch_block_t(const LMArgs<W>& a, const int32_t* verts, int nverts, cudaStream_t s) {
+  const size_t smem = (size_t)CAP * (sizeof(typename TableVal<WIDE>::T) + 4);
+  auto k = lm_block<W, WIDE, ASYNC, CAP, THREADS, U>;
+  static std::atomic<unsigned long long> attr{0};
+  smem_limit_once(attr, k, smem);
+  (count_launch(), k<<<grid_for(k, THREADS, smem, nverts), THREADS, smem, s>>>(a, verts, nverts));
+}
+
 template <typename W, bool WIDE, bool ASYNC>
 void launch_bucket_t(const LMArgs<W>& a, int bucket, const int32_t* verts, int nverts, cudaStream_t s) {
   if (nverts <= 0) return;
@@ -1141,22 +1167,9 @@ void launch_bucket_t(const LMArgs<W>& a, int bucket, const int32_t* verts, int n
       (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 7) / 8), 256, 0, s>>>(a, verts, nverts));
       break;
     }
-    case 3: {
-      constexpr int CAP = 2048;
-      size_t smem = (size_t)CAP * (sizeof(typename TableVal<WIDE>::T) + 4 + 1);
-      auto k = lm_block<W, WIDE, ASYNC, CAP, 128>;
-      (count_launch(), k<<<grid_for(k, 128, smem, nverts), 128, smem, s>>>(a, verts, nverts));
-      break;
-    }
-    case 4: {
-      constexpr int CAP = 8192;
-      size_t smem = (size_t)CAP * (sizeof(typename TableVal<WIDE>::T) + 4 + 1);
-      auto k = lm_block<W, WIDE, ASYNC, CAP, 512>;
-      static std::atomic<unsigned long long> attr{0};
-      smem_limit_once(attr, k, smem);
-      (count_launch(), k<<<grid_for(k, 512, smem, nverts), 512, smem, s>>>(a, verts, nverts));
-      break;
-    }
+    case 3: launch_block_t<W, WIDE, ASYNC, 2048, 128, 8>(a, verts, nverts, s); break;
+    case 4: launch_block_t<W, WIDE, ASYNC, 8192, 512, 8>(a, verts, nverts, s); break;
+    case 5: launch_block_t<W, WIDE, ASYNC, 18432, 1024, 12>(a, verts, nverts, s); break;
     default: break;
   }
 }
@@ -1175,18 +1188,27 @@ void lm_launch_bucket(const LMArgs<W>& a, bool wide, bool async, int bucket, con
   }
 }
 
+template <typename W, bool WIDE, bool ASYNC>
+static void launch_hub_insert(const LMArgs<W>& a, const int32_t* hubs, int nhubs, const int64_t* chunk_pre,
+                              int64_t nchunks, cudaStream_t s) {
+  const size_t smem = (size_t)(2 * kHubChunk) * (sizeof(typename TableVal<WIDE>::T) + 4);
+  auto k = lm_hub_insert<W, WIDE, ASYNC>;
+  static std::atomic<unsigned long long> attr{0};
+  smem_limit_once(attr, k, smem);
+  (count_launch(), k<<<(unsigned)nchunks, kHubThreads, smem, s>>>(a, hubs, nhubs, chunk_pre));
+}
+
 template <typename W>
 void lm_launch_hubs(const LMArgs<W>& a, bool wide, bool async, const int32_t* hubs, int nhubs,
                     const int64_t* chunk_pre, int64_t nchunks, const int64_t* spre, int64_t nslotchunks,
                     cudaStream_t s) {
   if (nhubs <= 0 || nchunks <= 0) return;
-  const size_t smem = (size_t)(2 * kHubChunk) * (wide ? 12 : 8);
   if (wide) {
-    if (async) (count_launch(), lm_hub_insert<W, true, true><<<(unsigned)nchunks, 256, smem, s>>>(a, hubs, nhubs, chunk_pre));
-    else (count_launch(), lm_hub_insert<W, true, false><<<(unsigned)nchunks, 256, smem, s>>>(a, hubs, nhubs, chunk_pre));
+    if (async) launch_hub_insert<W, true, true>(a, hubs, nhubs, chunk_pre, nchunks, s);
+    else launch_hub_insert<W, true, false>(a, hubs, nhubs, chunk_pre, nchunks, s);
   } else {
-    if (async) (count_launch(), lm_hub_insert<W, false, true><<<(unsigned)nchunks, 256, smem, s>>>(a, hubs, nhubs, chunk_pre));
-    else (count_launch(), lm_hub_insert<W, false, false><<<(unsigned)nchunks, 256, smem, s>>>(a, hubs, nhubs, chunk_pre));
+    if (async) launch_hub_insert<W, false, true>(a, hubs, nhubs, chunk_pre, nchunks, s);
+    else launch_hub_insert<W, false, false>(a, hubs, nhubs, chunk_pre, nchunks, s);
   }
   if (wide) {
     if (async) (count_launch(), lm_hub_scan<W, true, true><<<(unsigned)nslotchunks, 256, 0, s>>>(a, hubs, nhubs));
