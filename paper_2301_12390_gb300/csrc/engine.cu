@@ -472,7 +472,17 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   cs.mode_b = mode_b;
   // Bucket lists: key = bucket * P + class, hubs of all classes contiguous,
   // and the hubs' table layout.
-  std::vector<int64_t> ko(nkeys + 1);
+  std::vector<int64_t> ko(nkeys + 2);
+  // With M >= 2^31 (wide) a bucket still takes 64-bit gains and 32-bit sums
+  // when every vertex in it has K_i <= klimit = 2^61 / M: then |M K_{i->c}| and
+  // |K_i Sigma_c| stay at or below 2^61, a gain at or below 2^62 and every
+  // K_{i->c} below 2^31.  ko[nkeys + 1] receives the buckets that do not (found
+  // by the pass's first classification; degrees do not change within a pass).
+  // Road grid of 16.8M vertices (M = 3e9): degrees 1-8 913 -> 560 us an
+  // iteration.  Only vertices holding more than 2^61 / M^2 of all weight stay wide.
+  const long long klimit = wide ? (long long)((1ull << 61) / (unsigned long long)c->M) : 0;
+  unsigned long long wmask = 0;
+  auto wide_bucket = [&](int b) { return ((wmask >> b) & 1ull) != 0; };
   int64_t hub0 = 0, hub1 = 0, nhubs = 0;
   std::vector<int64_t> hchunks, hschunks;
   // sub_m > 0: the classes are drawn anew over the sub_m vertices with edges
@@ -501,6 +511,8 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // takes the partition's positions.
   int64_t edge_m = 0;
   auto classify = [&](int iter, bool filter) -> int {
+    const bool first = wide && iter == 0;
+    if (first) CK(cudaMemsetAsync(c->key_off + nkeys + 1, 0, sizeof(int64_t), s));
     if (edge_m > 0) {
       lm_keys_sub(g.off, c->level, edge_m, P, c->key, multi ? c->gid : nullptr, multi ? c->vo : nullptr, c->d_gcat,
                   cs, c->d_iter, thr, filter ? c->stamp[iter & 1] : nullptr, multi ? c->d_gon : nullptr, s);
@@ -508,11 +520,13 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
       gather_ids(c->newid, c->level, edge_m, c->list, s);
     } else {
       lm_keys(g.off, g.n, P, c->key, multi ? c->gid : nullptr, multi ? c->vo : nullptr, c->d_gcat, cs, c->d_iter,
-              thr, filter ? c->stamp[iter & 1] : nullptr, multi ? c->d_gon : nullptr, s);
+              thr, filter ? c->stamp[iter & 1] : nullptr, multi ? c->d_gon : nullptr, first ? c->K : nullptr, klimit,
+              (unsigned long long*)(c->key_off + nkeys + 1), s);
       stable_partition(c->key, g.n, nkeys, c->list, c->key_off, c->tmp, s);
     }
     CKLAUNCH();
     if (int r = fetch(c, ko.data(), c->key_off, ko.size() * sizeof(int64_t))) return r;
+    if (first) wmask = (unsigned long long)ko[nkeys + 1];
     hub0 = ko[kHubBucket * P];
     hub1 = ko[kHubBucket * P + P];
     nhubs = hub1 - hub0;
@@ -612,7 +626,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
     if (small_pass && sub_m > 0 && !drawn) reclassify_small();
     drawn = false;
     for (int ch = 0; ch < P && small_pass; ++ch) {
-      lm_launch_class<W>(a, wide, async, c->list, c->key_off, P, ch, class_grid_verts, s);
+      lm_launch_class<W>(a, wide_bucket(0) || wide_bucket(1) || wide_bucket(2), async, c->list, c->key_off, P, ch, class_grid_verts, s);
       if (!async) lm_launch_commit<W>(a, ko[3 * P], s);
       CKLAUNCH();
     }
@@ -629,7 +643,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
           int64_t s0 = ko[b * P + ch], s1 = ko[b * P + ch + 1];
           if (s1 <= s0) continue;
           sused[b] = true;
-          lm_launch_bucket<W>(a, wide, async, b, c->list + s0, (int)(s1 - s0), c->aux[b]);
+          lm_launch_bucket<W>(a, wide_bucket(b), async, b, c->list + s0, (int)(s1 - s0), c->aux[b]);
         }
         // hubs go in groups of consecutive classes (one launch sequence each)
         const int hstep = P / kHubGroups > 1 ? P / kHubGroups : 1;
@@ -644,7 +658,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
           ah.hkid = c->hkid + h0;
           ah.hdone = c->hdone + h0;
           ah.hmoved = c->hmoved + h0;
-          lm_launch_hubs<W>(ah, wide, async, c->list + hub0 + h0, (int)(h1 - h0), c->chunk_pre + h0,
+          lm_launch_hubs<W>(ah, wide_bucket(kHubBucket), async, c->list + hub0 + h0, (int)(h1 - h0), c->chunk_pre + h0,
                             hchunks[h1] - hchunks[h0], c->spre + h0, hschunks[h1] - hschunks[h0], c->aux[kHubBucket]);
         }
         CKLAUNCH();
@@ -664,7 +678,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
         if (s1 <= s0) continue;
         used[b] = true;
         CK(cudaStreamWaitEvent(c->aux[b], c->ev_fork, 0));
-        lm_launch_bucket<W>(a, wide, async, b, c->list + s0, (int)(s1 - s0), c->aux[b]);
+        lm_launch_bucket<W>(a, wide_bucket(b), async, b, c->list + s0, (int)(s1 - s0), c->aux[b]);
       }
       int64_t h0 = ko[kHubBucket * P + ch] - hub0, h1 = ko[kHubBucket * P + ch + 1] - hub0;
       if (h1 > h0) {
@@ -676,7 +690,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
         ah.hkid = c->hkid + h0;
         ah.hdone = c->hdone + h0;
         ah.hmoved = c->hmoved + h0;
-        lm_launch_hubs<W>(ah, wide, async, c->list + hub0 + h0, (int)(h1 - h0), c->chunk_pre + h0,
+        lm_launch_hubs<W>(ah, wide_bucket(kHubBucket), async, c->list + hub0 + h0, (int)(h1 - h0), c->chunk_pre + h0,
                           hchunks[h1] - hchunks[h0], c->spre + h0, hschunks[h1] - hschunks[h0], c->aux[kHubBucket]);
       }
       // join
@@ -1443,7 +1457,7 @@ int alloc_arena(louvain_ctx* c, int64_t n, int64_t nnz) {
   ALLOC(c->level, n);
   ALLOC(c->top, n);
   ALLOC(c->moves, n);
-  ALLOC(c->key_off, kBuckets * 64 + 8);
+  ALLOC(c->key_off, kBuckets * 64 + 8);   // offsets (nkeys + 1), then the wide buckets
   ALLOC(c->cnt, N1);
   ALLOC(c->cstart, N1);
   ALLOC(c->fill, N1);

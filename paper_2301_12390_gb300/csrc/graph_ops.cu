@@ -334,10 +334,15 @@ void stable_partition(const int32_t* key, int64_t n, int nkeys, int32_t* out, in
 __global__ void lm_keys_k(const int64_t* __restrict__ off, int64_t n, int P, int32_t* key,
                           const int32_t* __restrict__ gid, const int64_t* __restrict__ vo,
                           const int32_t* __restrict__ gcat, ClassSpec cs, const int* __restrict__ d_iter,
-                          LMThresholds th, const int32_t* __restrict__ active, const int32_t* __restrict__ g_on) {
+                          LMThresholds th, const int32_t* __restrict__ active, const int32_t* __restrict__ g_on,
+                          const long long* __restrict__ K, long long klimit, unsigned long long* wmask) {
   const int iter = *d_iter;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     int b = lm_bucket_of(off[i + 1] - off[i], th);
+    if (K && b >= 0 && K[i] > klimit) {
+      const unsigned long long bit = 1ull << b;
+      if (!(*(volatile unsigned long long*)wmask & bit)) atomicOr(wmask, bit);
+    }
     if (active && (active[i] != iter || (gid && !g_on[gid[i]]))) b = -1;
     key[i] = b < 0 ? kBuckets * P : b * P + (P > 1 ? vertex_class(i, gid, vo, gcat, cs, iter) : 0);
   }
@@ -373,9 +378,10 @@ static unsigned grid1d(int64_t n, int per = kT) {
 
 void lm_keys(const int64_t* off, int64_t n, int P, int32_t* key, const int32_t* gid, const int64_t* vo,
              const int32_t* gcat, ClassSpec cs, const int* d_iter, LMThresholds th, const int32_t* active,
-             const int32_t* g_on, cudaStream_t s) {
+             const int32_t* g_on, const long long* K, long long klimit, unsigned long long* wmask, cudaStream_t s) {
   if (n > 0)
-    (count_launch(), lm_keys_k<<<grid1d(n), kT, 0, s>>>(off, n, P, key, gid, vo, gcat, cs, d_iter, th, active, g_on));
+    (count_launch(), lm_keys_k<<<grid1d(n), kT, 0, s>>>(off, n, P, key, gid, vo, gcat, cs, d_iter, th, active, g_on,
+                                                        K, klimit, wmask));
 }
 
 __global__ void hub_sizes_k(const int64_t* off, const int32_t* hubs, int64_t nhubs, int64_t* cap, int64_t* chunks,
