@@ -128,7 +128,9 @@ __device__ __forceinline__ void warp_move_totals(const LMArgs<W>& a, BlockAcc& a
 // within a synchronous class; an asynchronous decision may use any recent
 // value).  size_c: the size of c when the caller loaded it with the
 // candidates (the guard's test), else -1 and it is loaded here.
-template <typename W, bool WIDE, bool ASYNC, int LD = (ASYNC ? 1 : 0)>
+// LIST false: a synchronous move is not appended here (the caller does it for
+// the whole warp).
+template <typename W, bool WIDE, bool ASYNC, int LD = (ASYNC ? 1 : 0), bool LIST = true>
 __device__ __forceinline__ bool commit_choice(const LMArgs<W>& a, BlockAcc& acc, int32_t i, int32_t d, long long Ki,
                                               long long sd, int32_t szd, typename Arith<WIDE>::S best, int32_t c,
                                               unsigned long long kid, long long M, int graph,
@@ -144,7 +146,7 @@ __device__ __forceinline__ bool commit_choice(const LMArgs<W>& a, BlockAcc& acc,
     atomicAdd((unsigned long long*)(a.sig + c), (unsigned long long)Ki);
     atomicSub(a.csize + d, 1);
     atomicAdd(a.csize + c, 1);
-  } else {
+  } else if (LIST) {
     unsigned long long pos = atomicAdd(&a.ctr->nmoves_list, 1ull);
     a.moves[pos] = make_int2(i, c);
   }
@@ -275,104 +277,179 @@ __device__ __forceinline__ void mark_row(const LMArgs<W>& a, const IterView& iv,
 
 // --------------------------------------------- bucket 0: thread per vertex
 
-// The row (<= 8 entries) is loaded first and its neighbours' communities
-// gathered with all loads in flight; duplicates are then merged in registers.
-// Lane l of the calling warp takes list entry vi (none if vi >= nverts); all
-// 32 lanes call it.  Whole warps sum their counters, moves and gains over the
-// warp: per-lane atomics on the block's counters serialise (measured: a third
-// of the thread kernel's time).
+// Synchronous moves of a warp's lanes (all 32 call it), appended to the move
+// list with one atomic: neighbouring records come from neighbouring vertices,
+// so the commit's loads coalesce.
+template <typename W>
+__device__ __forceinline__ void append_moves(const LMArgs<W>& a, bool moved, int32_t i, int32_t c) {
+  const unsigned m = __ballot_sync(0xffffffffu, moved);
+  if (!m) return;
+  const int leader = __ffs(m) - 1;
+  unsigned long long base = 0;
+  if ((int)(threadIdx.x & 31) == leader) base = atomicAdd(&a.ctr->nmoves_list, (unsigned long long)__popc(m));
+  base = __shfl_sync(0xffffffffu, base, leader);
+  if (moved) a.moves[base + __popc(m & lanemask_lt_lm())] = make_int2(i, c);
+}
+
+// Vertex i (on: it is visited) of degree deg <= D by one lane, row at b: the
+// row is loaded first and its neighbours' communities gathered with all loads
+// in flight; duplicates are then merged in registers.  gv: the gain of a move.
+// A synchronous move is left to the caller's append (to: its target).
+template <typename W, bool WIDE, bool ASYNC, int D>
+__device__ __forceinline__ bool thread_decide(const LMArgs<W>& a, const IterView& iv, BlockAcc& acc, int32_t i,
+                                              int64_t b, int deg, int32_t d, long long Ki, long long M, int graph,
+                                              int32_t* to, u128* gv, unsigned* n_cand) {
+  typedef typename Arith<WIDE>::S S;
+  typedef typename TableVal<WIDE>::T V;
+  const long long sd = ld_sig<ASYNC>(a.sig + d);
+  const int32_t szd = ld_size<ASYNC>(a.csize + d);
+  int32_t cc[D];
+  V ww[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const bool v = k < deg;
+    cc[k] = v ? a.col[b + k] : i;
+    ww[k] = v ? (V)a.wt[b + k] : (V)0;
+  }
+#pragma unroll
+  for (int k = 0; k < D; ++k) cc[k] = cc[k] != i ? ld_memb<ASYNC>(a.memb + cc[k]) : kEmpty;
+#pragma unroll
+  for (int k = 1; k < D; ++k) {
+    bool merged = false;
+#pragma unroll
+    for (int l = 0; l < k; ++l)
+      if (!merged && cc[k] != kEmpty && cc[l] == cc[k]) { ww[l] += ww[k]; merged = true; }
+    if (merged) cc[k] = kEmpty;
+  }
+  V kid = 0;
+#pragma unroll
+  for (int k = 0; k < D; ++k)
+    if (cc[k] == d) kid = ww[k];
+  // the candidates' totals, and for a singleton under the guard their
+  // sizes too (loaded with the totals instead of after the choice)
+  const bool want_size = a.guard && szd == 1;
+  long long sg[D];
+  int32_t sz[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const bool cand = cc[k] != kEmpty && cc[k] != d;
+    sg[k] = cand ? ld_sig<ASYNC>(a.sig + cc[k]) : 0;
+    sz[k] = cand && want_size && cc[k] > d ? ld_size<ASYNC>(a.csize + cc[k]) : 0;
+  }
+  S bg = Arith<WIDE>::lowest();
+  int32_t bc = -1, bsz = 0;
+  unsigned ncand = 0;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    if (cc[k] != kEmpty && cc[k] != d) {
+      ++ncand;
+      S g = Arith<WIDE>::score(M, (long long)ww[k], Ki, sg[k]);
+      if (better(g, cc[k], bg, bc)) { bg = g; bc = cc[k]; bsz = sz[k]; }
+    }
+  }
+  *n_cand = ncand;
+  *to = bc;
+  return commit_choice<W, WIDE, ASYNC, (ASYNC ? 1 : 0), false>(a, acc, i, d, Ki, sd, szd, bg, bc, kid, M, graph, gv,
+                                                              bsz);
+}
+
+// Up to 32 visited vertices, a lane each (i < 0: none); all 32 lanes call it.
+// A warp whose rows all have at most four entries (a road grid's nearly all
+// do) takes the instance that compares six pairs instead of 28.  Whole warps
+// sum their counters, moves and gains over the warp: per-lane atomics on the
+// block's counters serialise (measured: a third of the kernel's time).
+template <typename W, bool WIDE, bool ASYNC>
+__device__ __forceinline__ void thread_vertices(const LMArgs<W>& a, const IterView& iv, BlockAcc& acc, int32_t i) {
+  int64_t b = 0;
+  int deg = 0, graph = 0;
+  int32_t d = 0, to = -1;
+  long long Ki = 0, M = 0;
+  if (i >= 0) {
+    b = a.off[i];
+    deg = (int)(a.off[i + 1] - b);
+    d = a.memb[i];
+    Ki = a.K[i];
+    M = a.M;
+    if (a.gid) {
+      graph = a.gid[i];
+      M = a.Mg[graph];
+    }
+  }
+  bool moved = false;
+  u128 gv = 0;
+  unsigned n_cand = 0;
+  const unsigned longest = __reduce_max_sync(0xffffffffu, (unsigned)deg);
+  if (longest <= 4) {
+    if (i >= 0)
+      moved = thread_decide<W, WIDE, ASYNC, 4>(a, iv, acc, i, b, deg, d, Ki, M, graph, &to, &gv, &n_cand);
+  } else {
+    if (i >= 0)
+      moved = thread_decide<W, WIDE, ASYNC, 8>(a, iv, acc, i, b, deg, d, Ki, M, graph, &to, &gv, &n_cand);
+  }
+  if (moved && a.prune) mark_row<8>(a, iv, i, b, b + deg);
+  if (!ASYNC) append_moves(a, moved, i, to);
+  const unsigned n_edges = __reduce_add_sync(0xffffffffu, (unsigned)deg);
+  const unsigned n_visited = (unsigned)__popc(__ballot_sync(0xffffffffu, i >= 0));
+  n_cand = __reduce_add_sync(0xffffffffu, n_cand);
+  if ((threadIdx.x & 31) == 0 && n_visited) {
+    atomicAdd(&acc.edges, (unsigned long long)n_edges);
+    atomicAdd(&acc.visited, (unsigned long long)n_visited);
+    atomicAdd(&acc.cands, (unsigned long long)n_cand);
+  }
+  warp_move_totals(a, acc, moved, graph, gv);
+}
+
+// Lane l takes list entry base + l (none past nverts or inactive).
 template <typename W, bool WIDE, bool ASYNC>
 __device__ __forceinline__ void thread_vertex(const LMArgs<W>& a, const IterView& iv, BlockAcc& acc,
                                               const int32_t* __restrict__ verts, int64_t nverts, int64_t vi) {
-  typedef typename Arith<WIDE>::S S;
-  {
-    bool moved = false;
-    u128 gv = 0;
-    int graph = 0;
-    unsigned n_edges = 0, n_visited = 0, n_cand = 0;
-    do {
-      if (vi >= nverts) break;
-      int32_t i = verts[vi];
-      // the vertex's row bounds, community and degree are loaded together
-      // with its stamp, before the activity test
-      const int64_t b = a.off[i], e = a.off[i + 1];
-      const int32_t d = a.memb[i];
-      const long long Ki = a.K[i];
-      if (!is_active(a, iv, i)) break;
-      long long M;
-      if (!graph_of(a, i, &M, &graph)) break;
-      const long long sd = ld_sig<ASYNC>(a.sig + d);
-      const int32_t szd = ld_size<ASYNC>(a.csize + d);
-      int32_t cc[8];
-      unsigned long long ww[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const bool v = b + k < e;
-        cc[k] = v ? a.col[b + k] : i;
-        ww[k] = v ? (unsigned long long)a.wt[b + k] : 0ull;
-      }
-#pragma unroll
-      for (int k = 0; k < 8; ++k) cc[k] = cc[k] != i ? ld_memb<ASYNC>(a.memb + cc[k]) : kEmpty;
-#pragma unroll
-      for (int k = 1; k < 8; ++k) {
-        bool merged = false;
-#pragma unroll
-        for (int l = 0; l < k; ++l)
-          if (!merged && cc[k] != kEmpty && cc[l] == cc[k]) { ww[l] += ww[k]; merged = true; }
-        if (merged) cc[k] = kEmpty;
-      }
-      unsigned long long kid = 0;
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (cc[k] == d) kid = ww[k];
-      // the candidates' totals, and for a singleton under the guard their
-      // sizes too (loaded with the totals instead of after the choice)
-      const bool want_size = a.guard && szd == 1;
-      long long sg[8];
-      int32_t sz[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const bool cand = cc[k] != kEmpty && cc[k] != d;
-        sg[k] = cand ? ld_sig<ASYNC>(a.sig + cc[k]) : 0;
-        sz[k] = cand && want_size && cc[k] > d ? ld_size<ASYNC>(a.csize + cc[k]) : 0;
-      }
-      S bg = Arith<WIDE>::lowest();
-      int32_t bc = -1, bsz = 0;
-      unsigned ncand = 0;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        if (cc[k] != kEmpty && cc[k] != d) {
-          ++ncand;
-          S g = Arith<WIDE>::score(M, (long long)ww[k], Ki, sg[k]);
-          if (better(g, cc[k], bg, bc)) { bg = g; bc = cc[k]; bsz = sz[k]; }
-        }
-      }
-      n_cand = ncand;
-      n_edges = (unsigned)(e - b);
-      n_visited = 1;
-      moved = commit_choice<W, WIDE, ASYNC>(a, acc, i, d, Ki, sd, szd, bg, bc, kid, M, graph, &gv, bsz);
-      if (moved && a.prune) mark_row<8>(a, iv, i, b, e);
-    } while (false);
-    n_edges = __reduce_add_sync(0xffffffffu, n_edges);
-    n_visited = __reduce_add_sync(0xffffffffu, n_visited);
-    n_cand = __reduce_add_sync(0xffffffffu, n_cand);
-    if ((threadIdx.x & 31) == 0 && n_visited) {
-      atomicAdd(&acc.edges, (unsigned long long)n_edges);
-      atomicAdd(&acc.visited, (unsigned long long)n_visited);
-      atomicAdd(&acc.cands, (unsigned long long)n_cand);
-    }
-    warp_move_totals(a, acc, moved, graph, gv);
+  int32_t i = -1;
+  if (vi < nverts) {
+    i = verts[vi];
+    if (!is_active(a, iv, i) || (a.gid && !a.g_on[a.gid[i]])) i = -1;
   }
+  if (__any_sync(0xffffffffu, i >= 0)) thread_vertices<W, WIDE, ASYNC>(a, iv, acc, i);
 }
 
+// The warp walks its list entries 32 at a time and queues the visited ones in
+// shared memory until 32 are there: with pruning most lanes of a warp would
+// otherwise idle through the others' rows.
 template <typename W, bool WIDE, bool ASYNC>
 __global__ void __launch_bounds__(256, 3) lm_thread(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
   const IterView iv = iter_view(a);
   __shared__ BlockAcc acc;
+  __shared__ int32_t queue[8][2 * kWarp];
   acc_init(acc);
   __syncthreads();
-  for (int base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < nverts; base += gridDim.x * blockDim.x)
-    thread_vertex<W, WIDE, ASYNC>(a, iv, acc, verts, nverts, base + (int)(threadIdx.x & 31));
+  const int lane = threadIdx.x & 31;
+  int32_t* q = queue[threadIdx.x >> 5];
+  int have = 0;
+  for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < nverts;
+       base += (int64_t)gridDim.x * blockDim.x) {
+    int32_t i = -1;
+    if (base + lane < nverts) {
+      i = verts[base + lane];
+      if (!is_active(a, iv, i) || (a.gid && !a.g_on[a.gid[i]])) i = -1;
+    }
+    const unsigned on = __ballot_sync(0xffffffffu, i >= 0);
+    if (have == 0 && on == 0xffffffffu) {   // nothing to gather
+      thread_vertices<W, WIDE, ASYNC>(a, iv, acc, i);
+      continue;
+    }
+    if (i >= 0) q[have + __popc(on & lanemask_lt_lm())] = i;
+    have += __popc(on);
+    __syncwarp();
+    if (have >= kWarp) {
+      const int32_t j = q[lane];
+      const int32_t rest = q[kWarp + lane];
+      __syncwarp();
+      q[lane] = rest;
+      have -= kWarp;
+      __syncwarp();
+      thread_vertices<W, WIDE, ASYNC>(a, iv, acc, j);
+    }
+  }
+  if (have > 0) thread_vertices<W, WIDE, ASYNC>(a, iv, acc, lane < have ? q[lane] : -1);
   __syncthreads();
   acc_flush(acc, a.ctr);
 }
@@ -396,6 +473,7 @@ __device__ __forceinline__ void thread_vertex_sorted(const LMArgs<W>& a, const I
   bool moved = false;
   u128 gv = 0;
   int graph = 0;
+  int32_t vert = 0, to = -1;
   unsigned n_edges = 0, n_visited = 0, n_cand = 0;
   do {
     if (vi >= nverts) break;
@@ -482,9 +560,13 @@ __device__ __forceinline__ void thread_vertex_sorted(const LMArgs<W>& a, const I
     n_cand = ncand;
     n_edges = (unsigned)(e - b);
     n_visited = 1;
-    moved = commit_choice<W, false, ASYNC>(a, acc, i, d, Ki, sd, szd, bg, bc, kid, M, graph, &gv, bsz);
+    moved = commit_choice<W, false, ASYNC, (ASYNC ? 1 : 0), false>(a, acc, i, d, Ki, sd, szd, bg, bc, kid, M, graph,
+                                                                   &gv, bsz);
+    vert = i;
+    to = bc;
     if (moved && a.prune) mark_row<8>(a, iv, i, b, e);
   } while (false);
+  if (!ASYNC) append_moves(a, moved, vert, to);
   n_edges = __reduce_add_sync(0xffffffffu, n_edges);
   n_visited = __reduce_add_sync(0xffffffffu, n_visited);
   n_cand = __reduce_add_sync(0xffffffffu, n_cand);

@@ -42,7 +42,7 @@ EDGES = [[1, 8, 9, 31, 32, 33, 64, 127, 128, 129], [256, 1000, 1024, 1025, 2048,
          [4097, 6144, 6145, 8191, 12287], [12288, 12289, 16384, 16385]]
 
 
-@pytest.mark.parametrize("wmax", [1, 8, 200000])   # the last: 128-bit gains
+@pytest.mark.parametrize("wmax", [1, 8, 200000, 1 << 30])   # 128-bit gains: of some vertices, of all
 @pytest.mark.parametrize("degrees", EDGES, ids=["-%d" % max(d) for d in EDGES])
 def test_degrees_at_bucket_edges(degrees, wmax):
     assert_sync_parity(_stars(degrees, wmax, 11), prune=1, max_iterations=6, max_passes=3)
