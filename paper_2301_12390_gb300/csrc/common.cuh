@@ -69,6 +69,23 @@ __device__ __forceinline__ void atomic_add_u128(unsigned long long* lo, unsigned
   if (vhi) atomicAdd(hi, vhi);
 }
 
+// The double nearest to v (ties to even): the same value as the host's
+// conversion of a 128-bit integer.  The top 64 bits keep a sticky bit for the
+// rest, so the one rounding is that of the 64-bit conversion.
+__host__ __device__ inline double u128_to_double(u128 v) {
+  unsigned long long hi = (unsigned long long)(v >> 64), lo = (unsigned long long)v;
+  if (!hi) return (double)lo;
+  int up = 0;   // leading zeros of hi
+  while (!(hi >> 63)) {
+    hi = (hi << 1) | (lo >> 63);
+    lo <<= 1;
+    ++up;
+  }
+  double scale = 1.0;
+  for (int k = up; k < 64; ++k) scale *= 2.0;
+  return (double)(hi | (lo ? 1ull : 0ull)) * scale;
+}
+
 // ------------------------------------------------------------- the gain
 
 // score(x) = M * K_{i->x} - K_i * Sigma'_x, Sigma'_x the total of community x

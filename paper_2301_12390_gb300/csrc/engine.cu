@@ -141,6 +141,7 @@ struct louvain_ctx {
   int32_t* d_gcat = nullptr;   // per graph: its class-schedule category (kCatSmall, kCatLarge, kCatSparse)
   std::vector<int32_t> hgcat;   // the same on the host
   LMThresholds thr = {{kLMCap[0], kLMCap[1], kLMCap[2], kLMCap[3], kLMCap[4]}, kBigDegree};   // degree mapping
+  bool tuning = false;         // a trial of louvain_autotune: every vertex through the mapping
   bool warm = false;           // this run's pass 0 starts from the membership in memb
   int64_t lm_cands = 0;        // candidate communities evaluated by this run's local moving
   louvain_ctx* sub = nullptr;  // louvain_run_partitioned: the parts' context (same device and stream)
@@ -174,6 +175,9 @@ struct louvain_ctx {
   int64_t G = 1;
   std::vector<GraphState> gst;
   std::vector<int64_t> gM0, gn0;       // per graph: M and vertices of the loaded graph
+  std::vector<int64_t> ge0;            // ... and its entries
+  // several graphs: the pass graph's vo and each graph's entries, and the next one's
+  std::vector<int64_t> vo_host, ent_host, vo_host_next, ent_host_next;
   std::vector<i128> gqnum0;            // per graph: singleton Q numerator of the loaded graph
   int32_t* gid0 = nullptr;             // graph of every input vertex
   int32_t* gid_a = nullptr;
@@ -206,6 +210,7 @@ struct louvain_ctx {
   unsigned long long* d_gSS = nullptr;
   int64_t hcap = 0;                    // pinned per-graph host buffers below hold hcap graphs
   int32_t* h_gon = nullptr;
+  int32_t* h_ids = nullptr;
   unsigned long long* h_gmoves = nullptr;
   unsigned long long* h_gs = nullptr;
   unsigned long long* h_gL = nullptr;
@@ -225,6 +230,9 @@ struct louvain_ctx {
   static constexpr int kAux = kBuckets;
   cudaStream_t aux[kAux] = {};
   cudaEvent_t ev_fork = nullptr;
+  // the launches of a batch's small graphs run beside those of the others
+  cudaStream_t side = nullptr;
+  cudaEvent_t ev_side = nullptr;
   cudaEvent_t ev_join[kAux] = {};
 };
 
@@ -470,6 +478,147 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   const bool reclass = (any_small && mode_s == 1) || (any_big && mode_b == 1);   // every iteration
   cs.mode_s = mode_s;
   cs.mode_b = mode_b;
+  LMArgs<W> a;
+  memset(&a, 0, sizeof(a));
+  a.off = g.off;
+  a.col = g.col;
+  a.wt = (const W*)g.w;
+  a.K = c->K;
+  a.memb = c->memb;
+  a.sig = c->sig;
+  a.csize = c->csize;
+  a.moves = c->moves;
+  a.ctr = c->ctr;
+  a.M = c->M;
+  a.prune = c->opt.prune;
+  a.guard = c->opt.singleton_guard;
+  a.hkeys = c->gkeys;
+  a.hvals = c->gvals;
+  a.hpart = c->hpart;
+  a.hpart_c = c->hpart_c;
+  a.hdone = c->hdone;
+  a.d_iter = c->d_iter;
+  a.stamps[0] = c->stamp[0];
+  a.stamps[1] = c->stamp[1];
+  if (multi) {
+    a.gid = c->gid;
+    a.Mg = c->d_Mg;
+    a.g_on = c->d_gon;
+    a.g_moves = c->d_gmoves;
+    a.g_s = c->d_gs;
+  }
+  // the graphs that iterate in this pass
+  for (int64_t q = 0; q < G; ++q) {
+    c->gst[q].pass_moves = 0;
+    c->gst[q].pass_iters = 0;
+    c->h_gon[q] = c->gst[q].stopped ? 0 : 1;
+  }
+  if (multi) CK(cudaMemcpyAsync(c->d_gon, c->h_gon, G * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+  int64_t edges_total = 0, visited_total = 0, cands_total = 0;
+  // Small graphs: the whole phase in one launch, a block per graph, beside the
+  // other graphs' launches (on the side stream).  Custom mappings and the
+  // recomputed stop rule take the kernels below for every graph.
+  std::vector<int32_t> tiny, small;   // the graphs done in one launch
+  bool any_left = true;
+  {
+    bool on = c->opt.stop_rule == 0 && c->opt.max_iterations <= kSmallIters && !c->tuning &&
+              G * kSmallRec <= c->cap_nnz;
+    for (int b = 0; b < 5; ++b) on = on && c->thr.t[b] == kLMCap[b];
+    if (on) any_left = false;
+    for (int64_t q = 0; q < G && on; ++q) {
+      if (!c->h_gon[q]) continue;
+      const int cat = multi ? c->hgcat[q] : cs.single_cat;
+      const int Pg = cat == kCatSmall ? cs.Ps : cat == kCatSparse ? cs.Pl : cs.Pb;
+      const int64_t nq = multi ? c->vo_host[q + 1] - c->vo_host[q] : g.n, eq = multi ? c->ent_host[q] : g.nnz;
+      // of several graphs only those whose every degree suits 64-bit gains
+      // (the launch finds out for a single one)
+      if (nq <= kSmallVerts && eq <= small_entries(Pg) && (!multi || c->gst[q].M < (1ll << 31)))
+        (nq <= kTinyVerts ? tiny : small).push_back((int32_t)q);
+      else
+        any_left = true;
+    }
+  }
+  SmallArgs sa{multi ? c->vo : nullptr, nullptr, c->d_gcat, g.n, 0, false, cs, tol, c->opt.max_iterations,
+               (unsigned long long*)c->tw};   // c->tw: free until the pass aggregates
+  const bool any_block = !tiny.empty() || !small.empty();   // some graph is done in one launch
+  const bool beside = any_block && any_left;
+  if (any_block) {
+    cudaStream_t ss = beside ? c->side : s;
+    if (multi) {
+      int32_t* ids = (int32_t*)c->kcount;   // free until the pass renumbers
+      int64_t at = 0;
+      for (const std::vector<int32_t>* v : {&tiny, &small})
+        for (int32_t q : *v) {
+          c->h_ids[at++] = q;
+          c->h_gon[q] = 0;   // the launches below leave it out
+        }
+      CK(cudaMemcpyAsync(ids, c->h_ids, at * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+      CK(cudaMemcpyAsync(c->d_gon, c->h_gon, G * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+      sa.ids = ids;
+    }
+    if (beside) {
+      CK(cudaEventRecord(c->ev_fork, s));
+      CK(cudaStreamWaitEvent(ss, c->ev_fork, 0));
+    }
+    sa.count = (int64_t)small.size();   // the long ones first
+    const int32_t* ids = sa.ids;
+    if (multi) sa.ids = ids + tiny.size();
+    lm_launch_small<W>(a, sa, async, ss);
+    sa.count = (int64_t)tiny.size();
+    sa.tiny = true;
+    sa.ids = ids;
+    lm_launch_small<W>(a, sa, async, ss);
+    CKLAUNCH();
+    if (beside) CK(cudaEventRecord(c->ev_side, ss));
+  }
+  // Their records, once the launch is done (waits for the stream); *left: a
+  // single graph did not fit after all.
+  std::vector<IterRec> small_iters;   // per iteration, summed over these graphs
+  auto small_results = [&](bool* left) -> int {
+    std::vector<unsigned long long> rec(G * kSmallRec);
+    if (int r = fetch_many(c, {{rec.data(), c->tw, rec.size() * sizeof(unsigned long long)}})) return r;
+    for (const std::vector<int32_t>* v : {&tiny, &small})
+      for (int32_t q : *v) {
+        const unsigned long long* r = rec.data() + q * kSmallRec;
+        if (r[0] == kSmallNot && !multi) {
+          *left = true;
+          return 0;
+        }
+        if (r[0] > (unsigned long long)kSmallIters)
+          return fail(c, LOUVAIN_ERR_INTERNAL, "local-moving: a small graph's launch failed");
+        GraphState& st = c->gst[q];
+        edges_total += (int64_t)r[1];
+        visited_total += (int64_t)r[2];
+        cands_total += (int64_t)r[3];
+        for (int64_t t = 0; t < (int64_t)r[0]; ++t) {
+          const IterRec x{pass, (int64_t)r[4 + 3 * t], ((u128)r[6 + 3 * t] << 64) | (u128)r[5 + 3 * t]};
+          if (multi) st.iters.push_back(x);
+          st.pass_moves += x.moves;
+          st.pass_iters++;
+          if (t == (int64_t)small_iters.size()) small_iters.push_back(IterRec{pass, 0, 0});
+          small_iters[t].moves += x.moves;
+          small_iters[t].S += x.S;
+        }
+      }
+    return 0;
+  };
+  if (any_block && !any_left) {
+    if (int r = small_results(&any_left)) return r;
+    if (!any_left) {
+      c->iters.insert(c->iters.end(), small_iters.begin(), small_iters.end());
+      *iters_out = (int)small_iters.size();
+      *edges_out = edges_total;
+      *visited_out = visited_total;
+      c->lm_cands += cands_total;
+      return 0;
+    }
+  }
+  // an early return below must not leave the side stream's launch running
+  struct Join {
+    cudaStream_t st;
+    ~Join() { if (st) cudaStreamSynchronize(st); }
+  } join_side{beside ? c->side : nullptr};
+  const size_t iters0 = c->iters.size();
   // Bucket lists: key = bucket * P + class, hubs of all classes contiguous,
   // and the hubs' table layout.
   std::vector<int64_t> ko(nkeys + 2);
@@ -567,43 +716,6 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // hub move stamps are iteration numbers of this pass (by position in the
   // first hub list; later lists are subsets of it)
   if (nhubs > 0) CK(cudaMemsetAsync(c->hmoved, 0, (size_t)nhubs * sizeof(int32_t), s));
-  LMArgs<W> a;
-  memset(&a, 0, sizeof(a));
-  a.off = g.off;
-  a.col = g.col;
-  a.wt = (const W*)g.w;
-  a.K = c->K;
-  a.memb = c->memb;
-  a.sig = c->sig;
-  a.csize = c->csize;
-  a.moves = c->moves;
-  a.ctr = c->ctr;
-  a.M = c->M;
-  a.prune = c->opt.prune;
-  a.guard = c->opt.singleton_guard;
-  a.hkeys = c->gkeys;
-  a.hvals = c->gvals;
-  a.hpart = c->hpart;
-  a.hpart_c = c->hpart_c;
-  a.hdone = c->hdone;
-  a.d_iter = c->d_iter;
-  a.stamps[0] = c->stamp[0];
-  a.stamps[1] = c->stamp[1];
-  if (multi) {
-    a.gid = c->gid;
-    a.Mg = c->d_Mg;
-    a.g_on = c->d_gon;
-    a.g_moves = c->d_gmoves;
-    a.g_s = c->d_gs;
-  }
-  // the graphs that iterate in this pass
-  for (int64_t q = 0; q < G; ++q) {
-    c->gst[q].pass_moves = 0;
-    c->gst[q].pass_iters = 0;
-    c->h_gon[q] = c->gst[q].stopped ? 0 : 1;
-  }
-  if (multi) CK(cudaMemcpyAsync(c->d_gon, c->h_gon, G * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-  int64_t edges_total = 0, visited_total = 0, cands_total = 0;
 
   // One iteration's launch sequence: counters cleared, every class's buckets
   // forked onto their streams and joined (synchronous: then committed), and
@@ -852,6 +964,19 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   if (gexec) cudaGraphExecDestroy(gexec);
   if (graph) cudaGraphDestroy(graph);
   if (rc) return rc;
+  if (beside) {
+    CK(cudaStreamWaitEvent(s, c->ev_side, 0));
+    bool left = false;
+    if (int r = small_results(&left)) return r;
+    join_side.st = nullptr;
+  }
+  // the iterations of the graphs done in one launch join those of the others
+  for (size_t t = 0; t < small_iters.size(); ++t) {
+    if (iters0 + t == c->iters.size()) c->iters.push_back(IterRec{pass, 0, 0});
+    c->iters[iters0 + t].moves += small_iters[t].moves;
+    c->iters[iters0 + t].S += small_iters[t].S;
+  }
+  if ((int)small_iters.size() > it) it = (int)small_iters.size();
   *iters_out = it;
   *edges_out = edges_total;
   *visited_out = visited_total;
@@ -964,7 +1089,11 @@ int aggregate(louvain_ctx* c, const PassState& g, int64_t k, PassState* next, st
                                {c->h_acc, c->acc, 8 * sizeof(unsigned long long)}}))
       return r;
   } else {
+    graph_entries(c->offX[dst], c->vo_next, G, (int64_t*)c->d_gs, s);
+    CKLAUNCH();
+    c->ent_host_next.resize(G);
     if (int r = fetch_many(c, {{&nnz2, c->offX[dst] + k, sizeof(int64_t)}, {&flag, c->flags, sizeof(int)},
+                               {c->ent_host_next.data(), c->d_gs, G * sizeof(int64_t)},
                                {c->h_gL, c->d_gL, 2 * G * sizeof(unsigned long long)},
                                {c->h_gSS, c->d_gSS, 2 * G * sizeof(unsigned long long)}}))
       return r;
@@ -1045,6 +1174,7 @@ int compact_coarse(louvain_ctx* c, PassState* next, int64_t k, const std::vector
     std::vector<int64_t> vo_c(G + 1), zpre(G + 1);
     if (int r = fetch(c, vo_c.data(), c->vo, (G + 1) * sizeof(int64_t))) return r;
     for (int64_t q = 0; q <= G; ++q) zpre[q] = vo_full[q] - vo_c[q];
+    c->vo_host_next = vo_c;
     for (int64_t q = 0; q < G; ++q) c->h_zg[q] = zpre[q + 1] - zpre[q];
     CK(cudaMemcpyAsync(c->d_zpre, zpre.data(), (G + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(c->vo_next, c->vo, (G + 1) * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
@@ -1214,6 +1344,7 @@ int run_pass(louvain_ctx* c, const PassState& g, int pass, double* tol, bool wid
     if (int r = fetch(c, &k, c->scal, sizeof(int64_t))) return r;
   }
   if (c->compacted) c->kc_top = k;
+  c->vo_host_next = vo_next;
   // If another pass may follow, aggregate first: the coarse self-loops give
   // sum_C L_C, so the pass's Q numerators cost no extra scan of the graph; a
   // coarse graph built for a pass after which every graph stops is dropped.
@@ -1264,6 +1395,8 @@ int run_pass(louvain_ctx* c, const PassState& g, int pass, double* tol, bool wid
     if (multi) {
       std::swap(c->gid, c->gid_next);
       std::swap(c->vo, c->vo_next);
+      std::swap(c->vo_host, c->vo_host_next);
+      std::swap(c->ent_host, c->ent_host_next);
     }
   }
   if (c->opt.record_levels && iso > 0)
@@ -1298,6 +1431,9 @@ int init_run_state(louvain_ctx* c) {
     st.iters.clear();
   }
   if (G > 1) {
+    c->vo_host.assign(G + 1, 0);
+    for (int64_t q = 0; q < G; ++q) c->vo_host[q + 1] = c->vo_host[q] + c->gn0[q];
+    c->ent_host = c->ge0;
     c->gid = c->gid_a;
     c->gid_next = c->gid_b;
     c->vo = c->vo_a;
@@ -1380,7 +1516,10 @@ int tune_trial(louvain_ctx* c, const LMThresholds& th, float* ms) {
   int iters = 0;
   int64_t edges = 0, visited = 0;
   CK(cudaEventRecord(c->ev[0], s));
-  if (int r = local_moving<int32_t>(c, g, 0, c->opt.tolerance, wide, &iters, &edges, &visited)) return r;
+  c->tuning = true;
+  const int rl = local_moving<int32_t>(c, g, 0, c->opt.tolerance, wide, &iters, &edges, &visited);
+  c->tuning = false;
+  if (rl) return rl;
   CK(cudaEventRecord(c->ev[1], s));
   CK(cudaEventSynchronize(c->ev[1]));
   cudaEventElapsedTime(ms, c->ev[0], c->ev[1]);
@@ -1520,6 +1659,8 @@ int alloc_arena(louvain_ctx* c, int64_t n, int64_t nnz) {
 
 void free_host_graph_buffers(louvain_ctx* c) {
   if (c->h_gon) cudaFreeHost(c->h_gon);
+  if (c->h_ids) cudaFreeHost(c->h_ids);
+  c->h_ids = nullptr;
   if (c->h_gmoves) cudaFreeHost(c->h_gmoves);
   if (c->h_gs) cudaFreeHost(c->h_gs);
   if (c->h_gL) cudaFreeHost(c->h_gL);
@@ -1533,6 +1674,7 @@ int host_graph_buffers(louvain_ctx* c, int64_t G) {
   if (c->hcap >= G) return 0;
   free_host_graph_buffers(c);
   if (cudaMallocHost(&c->h_gon, G * sizeof(int32_t)) != cudaSuccess ||
+      cudaMallocHost(&c->h_ids, G * sizeof(int32_t)) != cudaSuccess ||
       cudaMallocHost(&c->h_gmoves, G * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMallocHost(&c->h_gs, 2 * G * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMallocHost(&c->h_gL, 2 * G * sizeof(unsigned long long)) != cudaSuccess ||
@@ -1612,7 +1754,12 @@ int louvain_create(louvain_ctx** out, const louvain_options* opt, int device, vo
       delete c;
       return LOUVAIN_ERR_CUDA;
     }
-  if (cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess) { delete c; return LOUVAIN_ERR_CUDA; }
+  if (cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_side, cudaEventDisableTiming) != cudaSuccess ||
+      cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, prio_least) != cudaSuccess) {
+    delete c;
+    return LOUVAIN_ERR_CUDA;
+  }
   if (cudaMallocHost(&c->h_ctr, sizeof(DevCounters)) != cudaSuccess ||
       cudaMallocHost(&c->h_acc, 8 * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMallocHost(&c->h_scal, 8 * sizeof(int64_t)) != cudaSuccess ||
@@ -1763,6 +1910,7 @@ int load_graphs(louvain_ctx* c, int64_t G, const int64_t* vo, int64_t n, int64_t
       CKLAUNCH();
       if (int r = fetch(c, ge.data(), c->d_gs, G * sizeof(int64_t))) return r;
     }
+    c->ge0 = ge;
     c->hgcat.assign(G, kCatLarge);
     for (int64_t q = 0; q < G; ++q)
       c->hgcat[q] = c->gn0[q] < kSmallGraph ? kCatSmall
@@ -2189,6 +2337,8 @@ void louvain_destroy(louvain_ctx* c) {
     if (c->ev_join[i]) cudaEventDestroy(c->ev_join[i]);
   }
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+  if (c->side) { cudaStreamSynchronize(c->side); cudaStreamDestroy(c->side); }
+  if (c->ev_side) cudaEventDestroy(c->ev_side);
   if (c->h_ctr) cudaFreeHost(c->h_ctr);
   if (c->h_acc) cudaFreeHost(c->h_acc);
   if (c->h_scal) cudaFreeHost(c->h_scal);

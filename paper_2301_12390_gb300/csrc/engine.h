@@ -117,6 +117,37 @@ template <typename W>
 void lm_launch_class(const LMArgs<W>& a, bool wide, bool async, const int32_t* list, const int64_t* ko, int P,
                      int ch, int64_t nverts, cudaStream_t s);
 constexpr int64_t kSmallPassEntries = 1 << 21;   // CSR entries up to which a pass takes one launch per class
+// Small graphs: the whole local-moving phase of a graph by one block, its
+// state in shared memory.  One graph (vo null: vertices [0, n)) or the `count`
+// graphs ids[0..count) of several (graph g: vertices [vo[g], vo[g + 1])); tiny:
+// all of them have at most kTinyVerts vertices.  rec: per graph kSmallRec
+// words: iterations run (kSmallNot: the graph does not fit and nothing was
+// done; kSmallErr: a table overflowed), entries scanned, vertices visited,
+// candidates, then per iteration its moves and the sum of their gains (lo, hi).
+constexpr int kSmallIters = 32;   // a larger max_iterations takes the launches
+constexpr int kSmallRec = 4 + 3 * kSmallIters;
+constexpr unsigned long long kSmallNot = ~0ull, kSmallErr = ~1ull;
+constexpr int64_t kSmallVerts = 8192, kTinyVerts = 1024;   // vertices whose state fits a block's shared memory
+// Entries up to which one block beats the launches of an iteration: a block
+// takes about 1 ns an entry and 1 us a class, the launches about 6 us a class
+// and 15 us an iteration whatever the size.
+__host__ __device__ inline int64_t small_entries(int classes) {
+  const int64_t e = 16384 + 4096 * (int64_t)classes;
+  return e < 131072 ? e : 131072;
+}
+struct SmallArgs {
+  const int64_t* vo;
+  const int32_t* ids;
+  const int32_t* gcat;
+  int64_t n, count;
+  bool tiny;
+  ClassSpec cs;
+  double tol;
+  int max_iterations;
+  unsigned long long* rec;
+};
+template <typename W>
+void lm_launch_small(const LMArgs<W>& a, const SmallArgs& sa, bool async, cudaStream_t s);
 // Pruning marks of every hub of the pass's hub list that moved in this iteration.
 template <typename W>
 void lm_launch_hub_mark(const LMArgs<W>& a, const int32_t* hubs, int nhubs, const int64_t* chunk_pre, int64_t nchunks,
@@ -143,7 +174,8 @@ void stable_partition(const int32_t* key, int64_t n, int nkeys, int32_t* out, in
 // of vertex i (P >= Ps, Pb); vertices of degree 0 get the trailing key
 // kBuckets * P.
 // active (may be null): the stamps of this iteration; with it, vertices not
-// active in it, or of a stopped graph (g_on), get the trailing key.
+// active in it get the trailing key, and so do those of a graph that does not
+// iterate (g_on, may be null).
 // K (may be null): bit b of *wmask is set when a vertex of bucket b has a
 // degree above klimit.
 void lm_keys(const int64_t* off, int64_t n, int P, int32_t* key, const int32_t* gid, const int64_t* vo,

@@ -329,8 +329,8 @@ void stable_partition(const int32_t* key, int64_t n, int nkeys, int32_t* out, in
 // --------------------------------------------------- local-moving lists
 
 // With `active` (the stamps read in this iteration), vertices that are not
-// active, or whose graph has stopped (g_on), get the trailing key too, so the
-// lists hold only the vertices the iteration visits.
+// active get the trailing key too, and so do those of a graph that does not
+// iterate (g_on), so the lists hold only the vertices the iteration visits.
 __global__ void lm_keys_k(const int64_t* __restrict__ off, int64_t n, int P, int32_t* key,
                           const int32_t* __restrict__ gid, const int64_t* __restrict__ vo,
                           const int32_t* __restrict__ gcat, ClassSpec cs, const int* __restrict__ d_iter,
@@ -343,7 +343,7 @@ __global__ void lm_keys_k(const int64_t* __restrict__ off, int64_t n, int P, int
       const unsigned long long bit = 1ull << b;
       if (!(*(volatile unsigned long long*)wmask & bit)) atomicOr(wmask, bit);
     }
-    if (active && (active[i] != iter || (gid && !g_on[gid[i]]))) b = -1;
+    if ((active && active[i] != iter) || (gid && g_on && !g_on[gid[i]])) b = -1;
     key[i] = b < 0 ? kBuckets * P : b * P + (P > 1 ? vertex_class(i, gid, vo, gcat, cs, iter) : 0);
   }
 }
@@ -359,7 +359,7 @@ __global__ void lm_keys_sub_k(const int64_t* __restrict__ off, const int32_t* __
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
     const int32_t i = sub[j];
     int b = lm_bucket_of(off[i + 1] - off[i], th);
-    if (active && (active[i] != iter || (gid && !g_on[gid[i]]))) b = -1;
+    if ((active && active[i] != iter) || (gid && g_on && !g_on[gid[i]])) b = -1;
     key[j] = b < 0 ? kBuckets * P : b * P + (P > 1 ? vertex_class(i, gid, vo, gcat, cs, iter) : 0);
   }
 }

@@ -795,6 +795,461 @@ __global__ void __launch_bounds__(256, 3) lm_class(LMArgs<W> a, const int32_t* _
   acc_flush(acc, a.ctr);
 }
 
+// ------------------------- small graphs: one block per graph, whole phase
+//
+// A graph of few thousand vertices leaves most of the chip idle whatever the
+// mapping, and a launch per class (5-7 us each, 8 to 32 classes an iteration)
+// costs more than its work.  One block then runs every iteration of the phase:
+// memberships, totals, sizes and activity bits live in shared memory, a class
+// ends at a block barrier, and the iteration's stop test is taken here, on the
+// same exact sums and roundings as on the host.  The graphs of a batch run
+// side by side, each its own number of iterations.  Class, order and commit
+// rules are those of the kernels above: asynchronous moves apply at once,
+// synchronous ones when the class is done.  A vertex of degree <= 8 takes a
+// lane, a larger one a warp.  With at most kTinyVerts vertices every warp has an
+// array of sums indexed by community; with more, a table of 256 slots for
+// degrees up to 128, and the block together takes larger ones, its warps'
+// values forming one such array.
+
+// One vertex's best candidate so far.
+struct SmallBest {
+  long long g;
+  int32_t c;
+};
+
+template <typename W, bool ASYNC, int NMAX, int THREADS>
+struct SmallGraph {
+  static constexpr int NW = THREADS / kWarp;
+  static constexpr bool kDense = NMAX <= kTinyVerts;   // sums indexed by community for every warp
+  static constexpr int CAP = kDense ? NMAX : 256;      // values of a warp (kDense) or slots of its table
+  static constexpr uint16_t kNone = 0xffff;  // no target
+  static_assert(NW * CAP >= NMAX, "the values of all tables are one array indexed by community");
+  // dynamic shared memory
+  long long* sig;      // NMAX
+  int32_t* size;       // NMAX
+  int32_t* keys;       // NW * CAP, empty between vertices (not with kDense)
+  unsigned* vals;      // NW * CAP, zero between vertices
+  unsigned* act;       // 2 * NMAX / 32: active in this / the next iteration
+  uint16_t* memb;      // NMAX
+  uint16_t* list;      // NMAX: vertices with entries by class
+  uint16_t* to;        // NMAX: synchronous targets of the class
+  static constexpr size_t kBytes = (size_t)NMAX * (8 + 4 + 3 * 2) + (size_t)NW * CAP * (kDense ? 4 : 8) + 2 * NMAX / 8;
+
+  __device__ __forceinline__ explicit SmallGraph(void* mem) {
+    sig = (long long*)mem;
+    size = (int32_t*)(sig + NMAX);
+    keys = size + NMAX;
+    vals = (unsigned*)(kDense ? keys : keys + NW * CAP);
+    act = vals + NW * CAP;
+    memb = (uint16_t*)(act + 2 * NMAX / 32);
+    list = memb + NMAX;
+    to = list + NMAX;
+  }
+  __device__ __forceinline__ void mark(unsigned* next, int v) const {
+    const unsigned bit = 1u << (v & 31);
+    if (!(next[v >> 5] & bit)) atomicOr(next + (v >> 5), bit);
+  }
+  // Vertex v moves from d to c now (asynchronous) or at the class's end.
+  __device__ __forceinline__ void move(int v, int d, int c, long long Ki) const {
+    if (ASYNC) {
+      memb[v] = (uint16_t)c;
+      atomicAdd((unsigned long long*)(sig + d), (unsigned long long)(-Ki));
+      atomicAdd((unsigned long long*)(sig + c), (unsigned long long)Ki);
+      atomicSub(size + d, 1);
+      atomicAdd(size + c, 1);
+    } else {
+      to[v] = (uint16_t)c;
+    }
+  }
+  // The gain of moving to the best candidate if the move is taken, else 0.
+  __device__ __forceinline__ long long gain(const SmallBest& best, int d, long long Ki, long long M, unsigned kid,
+                                            int guard) const {
+    if (best.c < 0) return 0;
+    const long long g = best.g - Arith<false>::score(M, (long long)kid, Ki, ((volatile long long*)sig)[d] - Ki);
+    if (g <= 0) return 0;
+    if (guard && best.c > d && ((volatile int32_t*)size)[d] == 1 && ((volatile int32_t*)size)[best.c] == 1) return 0;
+    return g;
+  }
+};
+
+template <typename W, bool ASYNC, int NMAX, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMArgs<W> a, SmallArgs sa) {
+  typedef SmallGraph<W, ASYNC, NMAX, THREADS> SG;
+  constexpr int NW = SG::NW;
+  extern __shared__ unsigned long long sdyn[];
+  const SG s(sdyn);
+  __shared__ int s_start[66], s_fill[64];
+  __shared__ int s_stop, s_moved;
+  __shared__ unsigned s_kid;
+  __shared__ long long r_g[NW];
+  __shared__ int32_t r_c[NW];
+  __shared__ unsigned long long r_lo[NW], r_hi[NW], r_moves[NW];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const bool single = sa.vo == nullptr;
+  const int64_t g = single ? 0 : sa.ids[blockIdx.x];
+  const int64_t v0 = single ? 0 : sa.vo[g];
+  const int64_t ng = (single ? sa.n : sa.vo[g + 1]) - v0;
+  const int64_t nnz = a.off[v0 + ng] - a.off[v0];
+  unsigned long long* rec = sa.rec + g * kSmallRec;
+  const int cat = single ? sa.cs.single_cat : sa.gcat[g];
+  const int P = cat == kCatSmall ? sa.cs.Ps : cat == kCatSparse ? sa.cs.Pl : sa.cs.Pb;
+  const int mode = cat == kCatSmall ? sa.cs.mode_s : sa.cs.mode_b;
+  const long long M = single ? a.M : a.Mg[g];
+  // 64-bit gains and 32-bit sums must hold every vertex (as for the buckets)
+  const long long klimit = M < (1ll << 31) ? M : (long long)((1ull << 61) / (unsigned long long)M);
+  int unfit = ng > NMAX || nnz > small_entries(P);
+  if (!unfit)
+    for (int v = tid; v < ng; v += THREADS) unfit |= a.K[v0 + v] > klimit;
+  if (__syncthreads_or(unfit)) {
+    if (tid == 0) rec[0] = kSmallNot;
+    return;
+  }
+  const int n = (int)ng;
+  const int64_t* __restrict__ off = a.off + v0;
+  for (int v = tid; v < n; v += THREADS) {
+    s.memb[v] = (uint16_t)(a.memb[v0 + v] - v0);
+    s.sig[v] = a.sig[v0 + v];
+    s.size[v] = a.csize[v0 + v];
+    s.to[v] = SG::kNone;
+  }
+  for (int t = tid; t < NW * SG::CAP; t += THREADS) {
+    if (!SG::kDense) s.keys[t] = kEmpty;
+    s.vals[t] = 0;
+  }
+  for (int t = tid; t < 2 * NMAX / 32; t += THREADS) s.act[t] = 0;
+  const double MM = u128_to_double((u128)M * (u128)M);
+  int32_t* keys = s.keys + wid * SG::CAP;
+  unsigned* vals = s.vals + wid * SG::CAP;
+  unsigned long long edges = 0;
+  unsigned visited = 0, cands = 0;
+  bool ok = true;
+  int it = 0;
+  for (; it < sa.max_iterations; ++it) {
+    __syncthreads();
+    if (it == 0 || mode == 1) {   // the class lists of this iteration
+      for (int c = tid; c < P; c += THREADS) s_fill[c] = 0;
+      __syncthreads();
+      for (int v = tid; v < n; v += THREADS)
+        if (off[v + 1] > off[v])
+          atomicAdd(&s_fill[P > 1 ? vertex_class(v0 + v, single ? nullptr : a.gid, sa.vo, sa.gcat, sa.cs, it) : 0], 1);
+      __syncthreads();
+      if (tid == 0) {
+        int sum = 0;
+        for (int c = 0; c < P; ++c) {
+          const int k = s_fill[c];
+          s_start[c] = s_fill[c] = sum;
+          sum += k;
+        }
+        s_start[P] = sum;
+      }
+      __syncthreads();
+      for (int v = tid; v < n; v += THREADS)
+        if (off[v + 1] > off[v])
+          s.list[atomicAdd(
+              &s_fill[P > 1 ? vertex_class(v0 + v, single ? nullptr : a.gid, sa.vo, sa.gcat, sa.cs, it) : 0], 1)] =
+              (uint16_t)v;
+    }
+    const unsigned* cur = s.act + (it & 1) * (NMAX / 32);
+    unsigned* next = s.act + ((it + 1) & 1) * (NMAX / 32);
+    for (int t = tid; t < NMAX / 32; t += THREADS) next[t] = 0;
+    __syncthreads();
+    unsigned moves = 0;
+    u128 S = 0;
+    for (int ch = 0; ch < P; ++ch) {
+      const int l0 = s_start[ch], m = s_start[ch + 1] - l0;
+      if (m == 0) continue;   // uniform
+      bool left = false;
+      // warp w takes entries w, w + NW, ...: 32 of them at a time, a lane each
+      for (int j0 = wid; j0 < m; j0 += kWarp * NW) {
+        const int j = j0 + lane * NW;
+        int v = -1, deg = 0, d = 0;
+        int64_t b = 0;
+        long long Ki = 0;
+        if (j < m) {
+          v = s.list[l0 + j];
+          if (a.prune && it > 0 && !((cur[v >> 5] >> (v & 31)) & 1u)) v = -1;
+        }
+        if (v >= 0) {
+          b = off[v];
+          deg = (int)(off[v + 1] - b);
+          Ki = a.K[v0 + v];
+          d = s.memb[v];
+          edges += (unsigned)deg;
+          ++visited;
+        }
+        if (v >= 0 && deg <= 8) {   // the lane alone
+          int cl[8], cc[8];
+          unsigned ww[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            cl[k] = k < deg ? (int)(__ldg(a.col + b + k) - v0) : v;
+            ww[k] = k < deg ? (unsigned)__ldg(a.wt + b + k) : 0u;
+          }
+#pragma unroll
+          for (int k = 0; k < 8; ++k) cc[k] = cl[k] != v ? (int)((volatile uint16_t*)s.memb)[cl[k]] : kEmpty;
+#pragma unroll
+          for (int k = 1; k < 8; ++k) {
+            bool merged = false;
+#pragma unroll
+            for (int l = 0; l < k; ++l)
+              if (!merged && cc[k] != kEmpty && cc[l] == cc[k]) { ww[l] += ww[k]; merged = true; }
+            if (merged) cc[k] = kEmpty;
+          }
+          unsigned kid = 0;
+          SmallBest best{Arith<false>::lowest(), -1};
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            if (cc[k] == kEmpty) continue;
+            if (cc[k] == d) {
+              kid = ww[k];
+            } else {
+              ++cands;
+              const long long sc =
+                  Arith<false>::score(M, (long long)ww[k], Ki, ((volatile long long*)s.sig)[cc[k]]);
+              if (better(sc, cc[k], best.g, best.c)) best = SmallBest{sc, cc[k]};
+            }
+          }
+          const long long gn = s.gain(best, d, Ki, M, kid, a.guard);
+          if (gn) {
+            s.move(v, d, best.c, Ki);
+            ++moves;
+            S += (u128)(unsigned long long)gn;
+            if (a.prune) {
+              s.mark(next, v);
+#pragma unroll
+              for (int k = 0; k < 8; ++k) s.mark(next, cl[k]);   // cl = v past the row
+            }
+          }
+        }
+        for (unsigned big = __ballot_sync(0xffffffffu, v >= 0 && deg > 8); big; big &= big - 1) {
+          const int src = __ffs(big) - 1;
+          const int vv = __shfl_sync(0xffffffffu, v, src), dg = __shfl_sync(0xffffffffu, deg, src);
+          const int dd = __shfl_sync(0xffffffffu, d, src);
+          const int64_t bb = __shfl_sync(0xffffffffu, b, src);
+          const long long kk = __shfl_sync(0xffffffffu, Ki, src);
+          if (dg > 128 && !SG::kDense) {   // for the block, after the class's other vertices
+            left = true;
+            continue;
+          }
+          int cl[4], cc[4];
+          unsigned ww[4];
+          auto load = [&](int x0) {   // entries x0 + 32 u + lane of the row
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int x = x0 + u * kWarp + lane;
+              cl[u] = vv;
+              ww[u] = 0;
+              if (x < dg) {
+                cl[u] = (int)(__ldg(a.col + bb + x) - v0);
+                ww[u] = (unsigned)__ldg(a.wt + bb + x);
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) cc[u] = cl[u] != vv ? (int)((volatile uint16_t*)s.memb)[cl[u]] : kEmpty;
+          };
+          unsigned kid = 0;
+          SmallBest best{Arith<false>::lowest(), -1};
+          auto candidate = [&](int c, unsigned sum) {
+            if (c == dd) {
+              kid = sum;
+            } else {
+              ++cands;
+              const long long sc = Arith<false>::score(M, (long long)sum, kk, ((volatile long long*)s.sig)[c]);
+              if (better(sc, c, best.g, best.c)) best = SmallBest{sc, c};
+            }
+          };
+          load(0);
+          if constexpr (SG::kDense) {
+            for (int x0 = 0;;) {
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (cc[u] != kEmpty) atomicAdd(vals + cc[u], ww[u]);
+              if ((x0 += 4 * kWarp) >= dg) break;
+              load(x0);
+            }
+            __syncwarp();
+            if (dg <= 4 * kWarp) {   // the first lane to take a sum evaluates it
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const unsigned sum = cc[u] != kEmpty ? atomicExch(vals + cc[u], 0u) : 0u;
+                if (sum) candidate(cc[u], sum);
+              }
+            } else {   // a long row: every community of the graph
+              for (int c = lane; c < n; c += kWarp) {
+                const unsigned sum = vals[c];
+                if (!sum) continue;
+                vals[c] = 0;
+                candidate(c, sum);
+              }
+            }
+          } else {
+            int hs[4];
+            const int nu = (dg + kWarp - 1) / kWarp;
+            const unsigned fresh = table_add_row<SG::CAP, 4, unsigned>(keys, vals, cc, ww, nu, hs, &ok);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              if (!((fresh >> u) & 1u)) continue;
+              candidate(cc[u], vals[hs[u]]);
+              keys[hs[u]] = kEmpty;
+              vals[hs[u]] = 0;
+            }
+          }
+          warp_argmax(best.g, best.c);
+          kid = __reduce_max_sync(0xffffffffu, kid);
+          long long gn = 0;
+          if (lane == 0) {
+            gn = s.gain(best, dd, kk, M, kid, a.guard);
+            if (gn) {
+              s.move(vv, dd, best.c, kk);
+              ++moves;
+              S += (u128)(unsigned long long)gn;
+            }
+          }
+          if (a.prune && __shfl_sync(0xffffffffu, gn != 0, 0)) {
+            if (lane == 0) s.mark(next, vv);
+            if (dg > 4 * kWarp) {
+              for (int x = lane; x < dg; x += kWarp) s.mark(next, (int)(__ldg(a.col + bb + x) - v0));
+            } else {
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (cl[u] != vv) s.mark(next, cl[u]);
+            }
+          }
+          __syncwarp();
+        }
+      }
+      const bool nbig = __syncthreads_or(left);
+      if (nbig) {   // uniform: vertices of degree above 128, the block together
+        unsigned* dense = s.vals;
+        for (int j = 0; j < m; ++j) {
+          const int v = s.list[l0 + j];
+          const int64_t b = off[v];
+          const int deg = (int)(off[v + 1] - b);
+          if (deg <= 128 || (a.prune && it > 0 && !((cur[v >> 5] >> (v & 31)) & 1u))) continue;   // uniform
+          const int d = s.memb[v];
+          const long long Ki = a.K[v0 + v];
+          if (tid == 0) s_kid = 0;
+          for (int x = tid; x < deg; x += THREADS) {
+            const int u = (int)(__ldg(a.col + b + x) - v0);
+            if (u != v) atomicAdd(dense + s.memb[u], (unsigned)__ldg(a.wt + b + x));
+          }
+          __syncthreads();
+          SmallBest best{Arith<false>::lowest(), -1};
+          for (int x = tid; x < deg; x += THREADS) {   // the first thread to take a sum evaluates it
+            const int u = (int)(__ldg(a.col + b + x) - v0);
+            if (u == v) continue;
+            const int c = s.memb[u];
+            const unsigned sum = dense[c] ? atomicExch(dense + c, 0u) : 0u;
+            if (!sum) continue;
+            if (c == d) {
+              s_kid = sum;
+            } else {
+              ++cands;
+              const long long sc = Arith<false>::score(M, (long long)sum, Ki, s.sig[c]);
+              if (better(sc, c, best.g, best.c)) best = SmallBest{sc, c};
+            }
+          }
+          warp_argmax(best.g, best.c);
+          if (lane == 0) { r_g[wid] = best.g; r_c[wid] = best.c; }
+          __syncthreads();
+          if (wid == 0) {
+            best = lane < NW ? SmallBest{r_g[lane], r_c[lane]} : SmallBest{Arith<false>::lowest(), -1};
+            warp_argmax(best.g, best.c);
+            if (lane == 0) {
+              const long long gn = s.gain(best, d, Ki, M, s_kid, a.guard);
+              s_moved = gn != 0;
+              if (gn) {
+                s.move(v, d, best.c, Ki);
+                ++moves;
+                S += (u128)(unsigned long long)gn;
+              }
+            }
+          }
+          __syncthreads();
+          if (a.prune && s_moved) {
+            if (tid == 0) s.mark(next, v);
+            for (int x = tid; x < deg; x += THREADS) s.mark(next, (int)(__ldg(a.col + b + x) - v0));
+          }
+        }
+        __syncthreads();
+      }
+      if (!ASYNC) {   // the class's moves
+        for (int j = tid; j < m; j += THREADS) {
+          const int v = s.list[l0 + j];
+          const uint16_t c = s.to[v];
+          if (c == SG::kNone) continue;
+          s.to[v] = SG::kNone;
+          const int d = s.memb[v];
+          const long long Ki = a.K[v0 + v];
+          s.memb[v] = c;
+          atomicAdd((unsigned long long*)(s.sig + d), (unsigned long long)(-Ki));
+          atomicAdd((unsigned long long*)(s.sig + c), (unsigned long long)Ki);
+          atomicSub(s.size + d, 1);
+          atomicAdd(s.size + c, 1);
+        }
+        __syncthreads();
+      }
+    }
+    // the iteration's totals and its stop test
+    S = warp_sum_u128(S);
+    const unsigned wm = __reduce_add_sync(0xffffffffu, moves);
+    if (lane == 0) {
+      r_lo[wid] = (unsigned long long)S;
+      r_hi[wid] = (unsigned long long)(S >> 64);
+      r_moves[wid] = wm;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      u128 tot = 0;
+      unsigned long long mv = 0;
+      for (int w = 0; w < NW; ++w) {
+        tot += ((u128)r_hi[w] << 64) | (u128)r_lo[w];
+        mv += r_moves[w];
+      }
+      rec[4 + 3 * it] = mv;
+      rec[5 + 3 * it] = (unsigned long long)tot;
+      rec[6 + 3 * it] = (unsigned long long)(tot >> 64);
+      s_stop = (2.0 * u128_to_double(tot)) / MM <= sa.tol;
+    }
+    __syncthreads();
+    if (s_stop) {
+      ++it;
+      break;
+    }
+  }
+  for (int v = tid; v < n; v += THREADS) {
+    a.memb[v0 + v] = (int32_t)(v0 + s.memb[v]);
+    a.sig[v0 + v] = s.sig[v];
+    a.csize[v0 + v] = s.size[v];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) edges += __shfl_xor_sync(0xffffffffu, edges, o);
+  visited = __reduce_add_sync(0xffffffffu, visited);
+  unsigned long long cd = cands;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) cd += __shfl_xor_sync(0xffffffffu, cd, o);
+  const bool failed = __syncthreads_or(!ok);
+  if (lane == 0) {
+    r_lo[wid] = edges;
+    r_hi[wid] = visited;
+    r_moves[wid] = cd;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    unsigned long long e = 0, vs = 0, c = 0;
+    for (int w = 0; w < NW; ++w) {
+      e += r_lo[w];
+      vs += r_hi[w];
+      c += r_moves[w];
+    }
+    rec[0] = failed ? kSmallErr : (unsigned long long)it;
+    rec[1] = e;
+    rec[2] = vs;
+    rec[3] = c;
+  }
+}
+
 // ----------------------------------------- buckets 3-5: block per vertex
 
 // A decided move waiting for the block to commit it, with its row bounds
@@ -1317,6 +1772,34 @@ void lm_launch_class(const LMArgs<W>& a, bool wide, bool async, const int32_t* l
   }
 }
 
+namespace {
+
+template <typename W, bool ASYNC, int NMAX, int THREADS>
+void launch_small_t(const LMArgs<W>& a, const SmallArgs& sa, cudaStream_t s) {
+  auto k = lm_small<W, ASYNC, NMAX, THREADS>;
+  const size_t smem = SmallGraph<W, ASYNC, NMAX, THREADS>::kBytes;
+  static std::atomic<unsigned long long> attr{0};
+  smem_limit_once(attr, k, smem);
+  (count_launch(), k<<<(unsigned)sa.count, THREADS, smem, s>>>(a, sa));
+}
+
+// Graphs of at most kTinyVerts vertices take 256 threads and 51 KB (four
+// blocks on an SM), larger ones a whole SM.
+template <typename W, bool ASYNC>
+void launch_small_by_size(const LMArgs<W>& a, const SmallArgs& sa, cudaStream_t s) {
+  if (sa.tiny) launch_small_t<W, ASYNC, kTinyVerts, 256>(a, sa, s);
+  else launch_small_t<W, ASYNC, kSmallVerts, 1024>(a, sa, s);
+}
+
+}  // namespace
+
+template <typename W>
+void lm_launch_small(const LMArgs<W>& a, const SmallArgs& sa, bool async, cudaStream_t s) {
+  if (sa.count <= 0) return;
+  if (async) launch_small_by_size<W, true>(a, sa, s);
+  else launch_small_by_size<W, false>(a, sa, s);
+}
+
 template <typename W>
 void lm_launch_hub_mark(const LMArgs<W>& a, const int32_t* hubs, int nhubs, const int64_t* chunk_pre, int64_t nchunks,
                         cudaStream_t s) {
@@ -1343,6 +1826,8 @@ template void lm_launch_class<int32_t>(const LMArgs<int32_t>&, bool, bool, const
                                        int, int64_t, cudaStream_t);
 template void lm_launch_class<int64_t>(const LMArgs<int64_t>&, bool, bool, const int32_t*, const int64_t*, int,
                                        int, int64_t, cudaStream_t);
+template void lm_launch_small<int32_t>(const LMArgs<int32_t>&, const SmallArgs&, bool, cudaStream_t);
+template void lm_launch_small<int64_t>(const LMArgs<int64_t>&, const SmallArgs&, bool, cudaStream_t);
 template void lm_launch_hub_mark<int32_t>(const LMArgs<int32_t>&, const int32_t*, int, const int64_t*, int64_t,
                                           cudaStream_t);
 template void lm_launch_hub_mark<int64_t>(const LMArgs<int64_t>&, const int32_t*, int, const int64_t*, int64_t,
