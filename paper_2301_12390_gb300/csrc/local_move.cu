@@ -660,7 +660,9 @@ __device__ __forceinline__ void warp_vertex(const LMArgs<W>& a, const IterView& 
   int hs[U];
   row_communities<U, LD>(a, v, lane, kWarp, nu, cc, ww);
   const unsigned fresh = table_add_row<CAP, U, V>(keys, vals, cc, ww, nu, hs, &ok);
-  const bool want_size = SIZES && a.guard && szd == 1;
+  // one lane's reading for the whole warp: it decides which reduction below the
+  // lanes take together, and an asynchronous size may change between two loads
+  const bool want_size = __shfl_sync(0xffffffffu, (int)(SIZES && a.guard && szd == 1), 0) != 0;
   long long sg[U];
   bool one[U];   // the candidate is a singleton (asked only for the guard)
 #pragma unroll
