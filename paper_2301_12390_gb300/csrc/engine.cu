@@ -155,7 +155,8 @@ struct louvain_ctx {
   size_t tmp_bytes = 0;
   int64_t M0 = 0;                      // total weight of the loaded graph
   int64_t cap_n = 0, cap_nnz = 0;      // arena capacity
-  bool dry_run = false;                // alloc_arena only adds up the bytes
+  bool dry_run = false;                // arena_pieces only adds up the bytes
+  unsigned char* arena_base = nullptr; // the arena, one allocation
   bool tables_dirty = true;            // global tables need clearing (new arena or a failed run)
   i128 qnum0 = 0;                      // exact Q numerator of the singleton partition of the loaded graph
   DevCounters* ctr = nullptr;
@@ -265,32 +266,20 @@ void free_all(louvain_ctx* c) {
   c->cap_nnz = 0;
 }
 
+// A buffer of the arena: the next piece of c->arena_base, or with dry_run only
+// its bytes (the arena is one allocation: the 71 cudaMalloc and cudaFree calls
+// of a buffer each took 8 ms whenever a server slot's arena grew, and every
+// cudaFree waits for the device).
 template <typename T>
 int dalloc(louvain_ctx* c, T** p, int64_t count) {
   size_t b = (size_t)(count > 0 ? count : 1) * sizeof(T);
   b = (b + 255) & ~(size_t)255;
-  if (c->dry_run) {   // size the arena only
-    c->bytes += (int64_t)b;
-    *p = nullptr;
-    return 0;
-  }
-  void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, b);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(c, LOUVAIN_ERR_OOM, "cudaMalloc of " + std::to_string(b) + " bytes failed");
-  }
-  c->allocs.push_back(q);
+  *p = c->dry_run ? nullptr : (T*)(c->arena_base + c->bytes);
   c->bytes += (int64_t)b;
-  *p = (T*)q;
   return 0;
 }
 
-#define ALLOC(ptr, count)                          \
-  do {                                             \
-    int r_ = dalloc(c, &(ptr), (int64_t)(count));  \
-    if (r_) { free_all(c); return r_; }            \
-  } while (0)
+#define ALLOC(ptr, count) dalloc(c, &(ptr), (int64_t)(count))
 
 int check_options(const louvain_options* o) {
   if (o->mode != LOUVAIN_SYNC && o->mode != LOUVAIN_ASYNC) return 1;
@@ -1570,9 +1559,9 @@ int autotune(louvain_ctx* c, float* best_ms) {
 
 // Device arena for graphs of up to n vertices and nnz entries (every buffer
 // is sized by one of the two); reused by later loads that fit.
-int alloc_arena(louvain_ctx* c, int64_t n, int64_t nnz) {
-  free_all(c);
+static int arena_pieces(louvain_ctx* c, int64_t n, int64_t nnz) {
   const int64_t N1 = n + 1;
+  c->bytes = 0;
   ALLOC(c->off0, N1);
   ALLOC(c->col0, nnz);
   ALLOC(c->w0, nnz);
@@ -1651,11 +1640,47 @@ int alloc_arena(louvain_ctx* c, int64_t n, int64_t nnz) {
   ALLOC(c->d_gs, 2 * N1);
   ALLOC(c->d_gL, 2 * N1);
   ALLOC(c->d_gSS, 2 * N1);
+  return 0;
+}
+
+static int64_t arena_size(int64_t n, int64_t nnz) {
+  louvain_ctx c;
+  c.dry_run = true;
+  arena_pieces(&c, n, nnz);
+  return c.bytes;
+}
+
+int alloc_arena(louvain_ctx* c, int64_t n, int64_t nnz) {
+  free_all(c);
+  const int64_t total = arena_size(n, nnz);
+  void* q = nullptr;
+  if (cudaMalloc(&q, (size_t)total) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(c, LOUVAIN_ERR_OOM, "cudaMalloc of " + std::to_string(total) + " bytes failed");
+  }
+  c->allocs.push_back(q);
+  c->arena_base = (unsigned char*)q;
+  arena_pieces(c, n, nnz);
   c->cap_n = n;
   c->cap_nnz = nnz;
   c->tables_dirty = true;
   return 0;
 }
+
+// An arena for graphs of up to n vertices and nnz entries before the load that
+// needs it (the server, which knows what its slot held before).
+namespace gbl {
+int reserve_arena(louvain_ctx* c, int64_t n, int64_t nnz) {
+  if (!c) return LOUVAIN_ERR_INVALID_ARG;
+  if (c->cap_n >= n && c->cap_nnz >= nnz && !c->allocs.empty()) return 0;
+  if (cudaSetDevice(c->device) != cudaSuccess) return LOUVAIN_ERR_CUDA;
+  return alloc_arena(c, n, nnz);
+}
+void arena_capacity(const louvain_ctx* c, int64_t* n, int64_t* nnz) {
+  *n = c ? c->cap_n : 0;
+  *nnz = c ? c->cap_nnz : 0;
+}
+}  // namespace gbl
 
 void free_host_graph_buffers(louvain_ctx* c) {
   if (c->h_gon) cudaFreeHost(c->h_gon);
@@ -2305,11 +2330,8 @@ int louvain_batch_get_iterations(louvain_ctx* c, int64_t g, int64_t* out, int64_
 
 int louvain_arena_bytes(int64_t n, int64_t nnz, int64_t* bytes) {
   if (n < 0 || nnz < 0 || !bytes) return LOUVAIN_ERR_INVALID_ARG;
-  louvain_ctx c;
-  c.dry_run = true;
-  int r = alloc_arena(&c, n, nnz);
-  *bytes = c.bytes;
-  return r;
+  *bytes = arena_size(n, nnz);
+  return 0;
 }
 
 int louvain_get_num_graphs(louvain_ctx* c, int64_t* num_graphs) {

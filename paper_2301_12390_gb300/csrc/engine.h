@@ -380,3 +380,11 @@ int blocks_per_sm(K kernel, int threads, size_t smem) {
 }
 
 }  // namespace gbl
+
+struct louvain_ctx;
+namespace gbl {
+// engine.cu, for the server: an arena for n vertices and nnz entries ahead of
+// the load, and what a context's arena holds.
+int reserve_arena(louvain_ctx* c, int64_t n, int64_t nnz);
+void arena_capacity(const louvain_ctx* c, int64_t* n, int64_t* nnz);
+}  // namespace gbl

@@ -11,6 +11,7 @@
 // keeps the arenas of all slots within the device-memory budget, a slot that
 // cannot grow waits for memory that other slots release, and a request that
 // cannot fit even alone is answered with LOUVAIN_ERR_OOM.
+#include <algorithm>
 #include <chrono>
 #include <condition_variable>
 #include <cstdint>
@@ -25,6 +26,7 @@
 #include <vector>
 #include <cuda_runtime.h>
 #include "../../include/louvain.h"
+#include "engine.h"
 
 namespace {
 
@@ -261,6 +263,20 @@ void worker(louvain_server* S, int k) {
       S->cv_work.notify_all();
       continue;
     }
+    // A slot whose arena must grow keeps what it held in the other dimension
+    // (vertices or entries), so that batches of differing shapes do not trade
+    // one for the other run after run; without room for both, just the batch.
+    int64_t cap_n = 0, cap_e = 0, keep_n = N, keep_e = E;
+    gbl::arena_capacity(slot.ctx, &cap_n, &cap_e);
+    if (cap_n < N || cap_e < E) {
+      int64_t both = 0;
+      louvain_arena_bytes(std::max(cap_n, N), std::max(cap_e, E), &both);
+      if (S->reserved_total + std::max<int64_t>(0, both - slot.reserved) <= S->cfg.hbm_budget_bytes) {
+        keep_n = std::max(cap_n, N);
+        keep_e = std::max(cap_e, E);
+        need = both;
+      }
+    }
     for (;;) {
       if (need <= slot.reserved) break;   // the slot's arena already holds it
       const int64_t growth = need - slot.reserved;
@@ -293,6 +309,7 @@ void worker(louvain_server* S, int k) {
     const double start_s = now_s(S->t0);
     std::vector<louvain_server_result> res;
     std::vector<std::vector<int32_t>> membs;
+    if (cap_n < N || cap_e < E) gbl::reserve_arena(slot.ctx, keep_n, keep_e);   // a failure shows in the load
     run_batch(S, slot, batch, start_s, res, membs);
     int64_t bytes = 0;
     louvain_get_device_bytes(slot.ctx, &bytes);
