@@ -36,7 +36,7 @@ struct DevCounters {
   unsigned long long s_lo, s_hi;   // sum of the gains of the moves (u128)
   unsigned long long edges;        // CSR entries scanned
   unsigned long long visited;      // vertices visited
-  unsigned long long nmoves_list;  // entries in the synchronous move list
+  unsigned long long nmoves_list[2];  // entries in the synchronous move list, by class parity
   unsigned long long cands;        // distinct candidate communities evaluated (other than the own)
   int error;
   int pad;
@@ -404,11 +404,12 @@ struct LMArgs {
   int32_t* memb;             // community of each vertex
   long long* sig;            // community totals Sigma_c
   int32_t* csize;            // community sizes (for the singleton guard)
-  const int* d_iter;         // the iteration number, read from device memory so that one
+  const int* d_iter;         // the iteration number (-1: the phase has ended, do nothing), read from device memory so that one
                              // captured launch sequence serves every iteration of a pass
   int32_t* stamps[2];        // pruning: active in iteration t iff stamps[t & 1][i] == t;
                              // a move marks stamps[(t + 1) & 1] with t + 1
   int2* moves;               // synchronous: (vertex, target) of every move of the class
+  int odd;                   // synchronous: the class's parity (its counter of ctr->nmoves_list)
   DevCounters* ctr;
   long long M;
   // several graphs in one run (block-diagonal CSR); gid == nullptr means one graph

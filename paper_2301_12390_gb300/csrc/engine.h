@@ -154,6 +154,9 @@ void lm_launch_hub_mark(const LMArgs<W>& a, const int32_t* hubs, int nhubs, cons
                         cudaStream_t s);
 template <typename W>
 void lm_launch_commit(const LMArgs<W>& a, int64_t max_moves, cudaStream_t s);
+// One graph: the iteration's counters to hist[iteration mod 4] and the stop
+// test on the device (MM = M^2 as a double); *d_iter moves on or to -1.
+void lm_decide(const DevCounters* ctr, DevCounters* hist, int* d_iter, double MM, double tol, cudaStream_t s);
 
 // ------------------------------------------------------- graph_ops.cu
 

@@ -147,7 +147,7 @@ __device__ __forceinline__ bool commit_choice(const LMArgs<W>& a, BlockAcc& acc,
     atomicSub(a.csize + d, 1);
     atomicAdd(a.csize + c, 1);
   } else if (LIST) {
-    unsigned long long pos = atomicAdd(&a.ctr->nmoves_list, 1ull);
+    unsigned long long pos = atomicAdd(a.ctr->nmoves_list + a.odd, 1ull);
     a.moves[pos] = make_int2(i, c);
   }
   u128 gv = Arith<WIDE>::to_u128(g);   // g > 0 here
@@ -286,7 +286,7 @@ __device__ __forceinline__ void append_moves(const LMArgs<W>& a, bool moved, int
   if (!m) return;
   const int leader = __ffs(m) - 1;
   unsigned long long base = 0;
-  if ((int)(threadIdx.x & 31) == leader) base = atomicAdd(&a.ctr->nmoves_list, (unsigned long long)__popc(m));
+  if ((int)(threadIdx.x & 31) == leader) base = atomicAdd(a.ctr->nmoves_list + a.odd, (unsigned long long)__popc(m));
   base = __shfl_sync(0xffffffffu, base, leader);
   if (moved) a.moves[base + __popc(m & lanemask_lt_lm())] = make_int2(i, c);
 }
@@ -417,6 +417,7 @@ __device__ __forceinline__ void thread_vertex(const LMArgs<W>& a, const IterView
 template <typename W, bool WIDE, bool ASYNC>
 __global__ void __launch_bounds__(256, 3) lm_thread(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
   const IterView iv = iter_view(a);
+  if (iv.iter < 0) return;
   __shared__ BlockAcc acc;
   __shared__ int32_t queue[8][2 * kWarp];
   acc_init(acc);
@@ -581,6 +582,7 @@ __device__ __forceinline__ void thread_vertex_sorted(const LMArgs<W>& a, const I
 template <typename W, bool ASYNC, int D>
 __global__ void __launch_bounds__(128) lm_thread_sorted(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
   const IterView iv = iter_view(a);
+  if (iv.iter < 0) return;
   __shared__ BlockAcc acc;
   acc_init(acc);
   __syncthreads();
@@ -708,6 +710,7 @@ __device__ __forceinline__ void warp_vertex(const LMArgs<W>& a, const IterView& 
 template <typename W, bool WIDE, bool ASYNC, int CAP, int U>
 __global__ void __launch_bounds__(256, 4) lm_warp(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
   const IterView iv = iter_view(a);
+  if (iv.iter < 0) return;
   typedef typename TableVal<WIDE>::T V;
   constexpr int WPB = 8;
   __shared__ int32_t skeys[WPB][CAP];
@@ -754,6 +757,7 @@ template <typename W, bool WIDE, bool ASYNC>
 __global__ void __launch_bounds__(256, 3) lm_class(LMArgs<W> a, const int32_t* __restrict__ list,
                                                    const int64_t* __restrict__ ko, int P, int ch) {
   const IterView iv = iter_view(a);
+  if (iv.iter < 0) return;
   typedef typename TableVal<WIDE>::T V;
   constexpr int WPB = 8, CAP = 256, U = 4;
   __shared__ int32_t skeys[WPB][CAP];
@@ -1275,7 +1279,7 @@ __device__ __forceinline__ void flush_moves(const LMArgs<W>& a, const IterView& 
       atomicSub(a.csize + m.d, 1);
       atomicAdd(a.csize + m.c, 1);
     } else {
-      unsigned long long pos = atomicAdd(&a.ctr->nmoves_list, 1ull);
+      unsigned long long pos = atomicAdd(a.ctr->nmoves_list + a.odd, 1ull);
       a.moves[pos] = make_int2(m.i, m.c);
     }
   }
@@ -1329,6 +1333,7 @@ template <typename W, bool WIDE, bool ASYNC, int CAP, int THREADS, int U>
 __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ? 2 : 1)
     lm_block(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
   const IterView iv = iter_view(a);
+  if (iv.iter < 0) return;
   typedef typename Arith<WIDE>::S S;
   typedef typename TableVal<WIDE>::T V;
   constexpr int NW = THREADS / kWarp;
@@ -1468,6 +1473,7 @@ __global__ void __launch_bounds__(kHubThreads) lm_hub_insert(LMArgs<W> a, const 
                                                              const int64_t* __restrict__ chunk_pre) {
   typedef typename TableVal<WIDE>::T V;
   const IterView iv = iter_view(a);
+  if (iv.iter < 0) return;
   constexpr int CAP = 2 * kHubChunk;
   constexpr int U = kHubChunk / kHubThreads;
   static_assert(U >= 1 && kHubChunk % kHubThreads == 0, "a chunk covers whole rounds of the block");
@@ -1515,6 +1521,7 @@ __global__ void __launch_bounds__(kHubThreads) lm_hub_insert(LMArgs<W> a, const 
 template <typename W, bool WIDE, bool ASYNC>
 __global__ void __launch_bounds__(256) lm_hub_scan(LMArgs<W> a, const int32_t* __restrict__ hubs, int nhubs) {
   const IterView iv = iter_view(a);
+  if (iv.iter < 0) return;
   typedef typename Arith<WIDE>::S S;
   constexpr int NW = 256 / kWarp;
   __shared__ S red_g[NW];
@@ -1623,6 +1630,7 @@ template <typename W>
 __global__ void __launch_bounds__(256) lm_hub_mark(LMArgs<W> a, const int32_t* __restrict__ hubs, int nhubs,
                                                    const int64_t* __restrict__ chunk_pre) {
   const IterView iv = iter_view(a);
+  if (iv.iter < 0) return;
   __shared__ int64_t s_pre[kItemCache + 1];
   const int h = block_item<kItemCache>(chunk_pre, nhubs, blockIdx.x, s_pre);
   if (a.hmoved[h] != iv.iter + 1) return;
@@ -1636,9 +1644,12 @@ __global__ void __launch_bounds__(256) lm_hub_mark(LMArgs<W> a, const int32_t* _
 
 // ----------------------------------------------- synchronous commit step
 
+// It also clears the next class's counter (free: the class before this one,
+// which used it last, is committed).
 template <typename W>
 __global__ void __launch_bounds__(256) lm_commit(LMArgs<W> a) {
-  const unsigned long long n = a.ctr->nmoves_list;
+  const unsigned long long n = a.ctr->nmoves_list[a.odd];
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr->nmoves_list[a.odd ^ 1] = 0;
   for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < n;
        t += (unsigned long long)gridDim.x * blockDim.x) {
     int2 mv = a.moves[t];
@@ -1652,7 +1663,20 @@ __global__ void __launch_bounds__(256) lm_commit(LMArgs<W> a) {
   }
 }
 
-__global__ void reset_move_list(DevCounters* ctr) { ctr->nmoves_list = 0; }
+// The end of an iteration of one graph, on the device: its counters go to
+// slot (iteration mod 4) of hist, and the iteration number moves on, or to -1
+// when the phase ends (the stop test of the host, on the same roundings), which
+// makes the launches of an iteration queued behind it return at once.
+__global__ void lm_decide_k(const DevCounters* ctr, DevCounters* hist, int* d_iter, double MM, double tol) {
+  const int it = *d_iter;
+  if (it < 0) return;
+  hist[it & 3] = *ctr;
+  const u128 S = ((u128)ctr->s_hi << 64) | (u128)ctr->s_lo;
+  *d_iter = (2.0 * u128_to_double(S)) / MM <= tol ? -1 : it + 1;
+}
+void lm_decide(const DevCounters* ctr, DevCounters* hist, int* d_iter, double MM, double tol, cudaStream_t s) {
+  (count_launch(), lm_decide_k<<<1, 1, 0, s>>>(ctr, hist, d_iter, MM, tol));
+}
 
 // ---------------------------------------------------------------- launch
 
@@ -1815,7 +1839,6 @@ void lm_launch_commit(const LMArgs<W>& a, int64_t max_moves, cudaStream_t s) {
   int blocks = (int)((max_moves + 255) / 256);
   if (blocks > 152 * 16) blocks = 152 * 16;
   (count_launch(), lm_commit<W><<<blocks, 256, 0, s>>>(a));
-  (count_launch(), reset_move_list<<<1, 1, 0, s>>>(a.ctr));
 }
 
 template void lm_launch_bucket<int32_t>(const LMArgs<int32_t>&, bool, bool, int, const int32_t*, int, cudaStream_t);
