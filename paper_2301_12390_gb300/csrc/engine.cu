@@ -555,11 +555,11 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
     sa.count = (int64_t)small.size();   // the long ones first
     const int32_t* ids = sa.ids;
     if (multi) sa.ids = ids + tiny.size();
-    lm_launch_small<W>(a, sa, async, ss);
+    lm_launch_small<W>(a, sa, ss);
     sa.count = (int64_t)tiny.size();
     sa.tiny = true;
     sa.ids = ids;
-    lm_launch_small<W>(a, sa, async, ss);
+    lm_launch_small<W>(a, sa, ss);
     CKLAUNCH();
     if (beside) CK(cudaEventRecord(c->ev_side, ss));
   }

@@ -147,7 +147,7 @@ struct SmallArgs {
   unsigned long long* rec;
 };
 template <typename W>
-void lm_launch_small(const LMArgs<W>& a, const SmallArgs& sa, bool async, cudaStream_t s);
+void lm_launch_small(const LMArgs<W>& a, const SmallArgs& sa, cudaStream_t s);
 // Pruning marks of every hub of the pass's hub list that moved in this iteration.
 template <typename W>
 void lm_launch_hub_mark(const LMArgs<W>& a, const int32_t* hubs, int nhubs, const int64_t* chunk_pre, int64_t nchunks,
