@@ -57,6 +57,9 @@ constexpr double kFilterFraction = 0.1;
 // A pass with at least this many vertices per vertex with edges classifies
 // its later iterations over the vertices with edges only.
 constexpr int64_t kEdgeListRatio = 4;
+// A synchronous pass of up to this many entries is shorter on the GPU than its
+// launches on the host.
+constexpr int64_t kGraphEntries = 8 << 20;
 
 struct IterRec {
   int pass;
@@ -163,8 +166,8 @@ struct louvain_ctx {
   unsigned long long* acc = nullptr;   // 8 words of reduction scratch
   int* flags = nullptr;
   int* d_iter = nullptr;               // current local-moving iteration (device)
-  DevCounters* hist = nullptr;         // counters of the last four iterations queued ahead
-  DevCounters* h_hist = nullptr;       // pinned
+  DevCounters* h_hist = nullptr;       // pinned: counters of the last four iterations queued ahead
+  unsigned* draw = nullptr;            // draw_lists' scratch (zero between draws)
   cudaEvent_t ev_iter[4] = {};
   int* h_iter = nullptr;               // pinned staging for it
   int64_t* scal = nullptr;             // small device scalars
@@ -629,14 +632,13 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // sub_m > 0: the classes are drawn anew over the sub_m vertices with edges
   // kept in c->level (a small pass; its other vertices are isolated)
   int64_t sub_m = 0;
-  // the class lists of the vertices with edges only, all on the device (a
-  // small pass whose classes are drawn anew: part of its iteration)
-  auto reclassify_small = [&]() {
-    int32_t* idx = (int32_t*)c->moves;   // free in asynchronous mode
-    lm_keys_sub(g.off, c->level, sub_m, P, c->key, multi ? c->gid : nullptr, multi ? c->vo : nullptr, c->d_gcat,
-                cs, c->d_iter, thr, nullptr, nullptr, s);
-    stable_partition(c->key, sub_m, nkeys, idx, c->key_off, c->tmp, s);
-    gather_ids(idx, c->level, sub_m, c->list, s);
+  DrawArgs dr{g.off, nullptr, g.n, P, multi ? c->gid : nullptr, multi ? c->vo : nullptr, c->d_gcat, cs, c->d_iter,
+              thr, nullptr, nullptr, nullptr, klimit, (unsigned long long*)(c->key_off + nkeys + 1)};
+  uint16_t* const keys = (uint16_t*)c->key;
+  auto draw = [&](int64_t m, const int32_t* sub) {
+    dr.m = m;
+    dr.sub = sub;
+    draw_lists(dr, keys, c->list, c->key_off, c->draw, s);
   };
   // With pruning, once few vertices of a large pass are active (the last
   // iteration visited less than kFilterFraction of at least kFilterMinList
@@ -648,23 +650,23 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // A pass whose vertices are mostly isolated (the later passes of a
   // heavy-tailed graph: every isolated vertex stays a community of its own)
   // classifies again only its vertices with edges, kept in c->level (free
-  // until renumbering) after the first classification; c->newid (free too)
-  // takes the partition's positions.
+  // until renumbering) after the first classification.
   int64_t edge_m = 0;
   auto classify = [&](int iter, bool filter) -> int {
     const bool first = wide && iter == 0;
     if (first) CK(cudaMemsetAsync(c->key_off + nkeys + 1, 0, sizeof(int64_t), s));
-    if (edge_m > 0) {
-      lm_keys_sub(g.off, c->level, edge_m, P, c->key, multi ? c->gid : nullptr, multi ? c->vo : nullptr, c->d_gcat,
-                  cs, c->d_iter, thr, filter ? c->stamp[iter & 1] : nullptr, multi ? c->d_gon : nullptr, s);
-      stable_partition(c->key, edge_m, nkeys, c->newid, c->key_off, c->tmp, s);
-      gather_ids(c->newid, c->level, edge_m, c->list, s);
+    dr.K = first ? c->K : nullptr;
+    dr.active = filter ? c->stamp[iter & 1] : nullptr;
+    dr.g_on = multi ? c->d_gon : nullptr;
+    if (!reclass && !filter && edge_m == 0) {   // these lists serve the pass
+      dr.m = g.n;
+      dr.sub = nullptr;
+      draw_lists_stable(dr, c->key, c->list, c->key_off, c->tmp, s);
     } else {
-      lm_keys(g.off, g.n, P, c->key, multi ? c->gid : nullptr, multi ? c->vo : nullptr, c->d_gcat, cs, c->d_iter,
-              thr, filter ? c->stamp[iter & 1] : nullptr, multi ? c->d_gon : nullptr, first ? c->K : nullptr, klimit,
-              (unsigned long long*)(c->key_off + nkeys + 1), s);
-      stable_partition(c->key, g.n, nkeys, c->list, c->key_off, c->tmp, s);
+      draw(edge_m > 0 ? edge_m : g.n, edge_m > 0 ? c->level : nullptr);
     }
+    dr.K = nullptr;
+    dr.active = dr.g_on = nullptr;
     CKLAUNCH();
     if (int r = fetch(c, ko.data(), c->key_off, ko.size() * sizeof(int64_t))) return r;
     if (first) wmask = (unsigned long long)ko[nkeys + 1];
@@ -709,18 +711,35 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // first hub list; later lists are subsets of it)
   if (nhubs > 0) CK(cudaMemsetAsync(c->hmoved, 0, (size_t)nhubs * sizeof(int32_t), s));
 
+  const bool may_filter = c->opt.prune && !small_pass && full_len >= kFilterMinList;
   // One graph whose launches do not depend on the host from one iteration to
-  // the next (no new draw of large classes, no filtered lists): the iterations
+  // the next (no new draw of hubs, no filtered lists): the iterations
   // are queued one ahead of the host's reading (12-15 us an iteration saved; the
   // one iteration queued in vain costs 1-2 us a launch, so not with many classes).
-  const bool ahead = !multi && c->opt.stop_rule == 0 && (small_pass || !reclass) && P <= 16 &&
-                     !(c->opt.prune && !small_pass && full_len >= kFilterMinList);
+  const bool ahead = !multi && c->opt.stop_rule == 0 && (small_pass || !reclass || nhubs == 0) && P <= 16 &&
+                     !may_filter;
   // From this iteration on they are replayed as one captured CUDA graph: a
-  // small pass of several classes, others only with the cuda_graphs option and
-  // fixed classes.
+  // small pass of several classes; with fixed lists, a pass whose launches and
+  // stream joins (45 us) take the host longer than the GPU, once it has lasted
+  // four iterations (a graph costs about 150 us to build); others only with the
+  // cuda_graphs option and fixed classes.
   const int never = 1 << 30;
   const int graph_from = small_pass && P >= 4 ? (ahead ? 2 : 1)
+                         : !small_pass && !reclass && !may_filter && g.nnz <= kGraphEntries ? 4
                          : c->opt.cuda_graphs && !reclass && !c->opt.prune && !small_pass ? 2 : never;
+  // Classes drawn anew every iteration inside the iteration's sequence: a small
+  // pass (over its vertices with edges), or iterations queued ahead.
+  const bool redraw = reclass && (small_pass ? sub_m > 0 : ahead);
+  const int64_t redraw_m = small_pass ? sub_m : edge_m > 0 ? edge_m : g.n;
+  const int32_t* redraw_sub = small_pass || edge_m > 0 ? c->level : nullptr;
+  if (ahead) CK(cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), s));
+  // vertices of (bucket, class): exact after a classification read here, with
+  // classes drawn on the device an estimate for the grid
+  auto class_size = [&](int b, int ch) -> int64_t {
+    if (!redraw) return ko[b * P + ch + 1] - ko[b * P + ch];
+    const int64_t all = ko[(b + 1) * P] - ko[b * P];
+    return all ? all / P + all / (4 * P) + 64 : 0;
+  };
   // One iteration's launch sequence: counters cleared, every class's buckets
   // forked onto their streams and joined (synchronous: then committed), and
   // the counters copied to pinned host memory.  The sequence depends on the
@@ -732,14 +751,14 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // iteration 0, whose classes the first classification drew.
   bool drawn = true;
   auto iteration = [&]() -> int {
-    CK(cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), s));
+    if (!ahead) CK(cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), s));
     if (multi) {
       CK(cudaMemsetAsync(c->d_gmoves, 0, G * sizeof(unsigned long long), s));
       CK(cudaMemsetAsync(c->d_gs, 0, 2 * G * sizeof(unsigned long long), s));
     }
     // a small pass graph without vertices above degree 128: one launch per
     // class on the main stream (and the new draw of its classes first)
-    if (small_pass && sub_m > 0 && !drawn) reclassify_small();
+    if (redraw && !drawn) draw(redraw_m, redraw_sub);
     drawn = false;
     for (int ch = 0; ch < P && small_pass; ++ch) {
       a.odd = ch & 1;
@@ -757,10 +776,10 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
       for (int b = 0; b < kBuckets; ++b) CK(cudaStreamWaitEvent(c->aux[b], c->ev_fork, 0));
       for (int ch = 0; ch < P; ++ch) {
         for (int b = 0; b < kHubBucket; ++b) {
-          int64_t s0 = ko[b * P + ch], s1 = ko[b * P + ch + 1];
-          if (s1 <= s0) continue;
+          const int64_t m = class_size(b, ch);
+          if (m <= 0) continue;
           sused[b] = true;
-          lm_launch_bucket<W>(a, wide_bucket(b), async, b, c->list + s0, (int)(s1 - s0), c->aux[b]);
+          lm_launch_bucket<W>(a, wide_bucket(b), async, b, c->list, c->key_off + b * P + ch, m, c->aux[b]);
         }
         // hubs go in groups of consecutive classes (one launch sequence each)
         const int hstep = P / kHubGroups > 1 ? P / kHubGroups : 1;
@@ -792,11 +811,11 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
       bool used[kBuckets] = {};
       CK(cudaEventRecord(c->ev_fork, s));
       for (int b = 0; b < kHubBucket; ++b) {
-        int64_t s0 = ko[b * P + ch], s1 = ko[b * P + ch + 1];
-        if (s1 <= s0) continue;
+        const int64_t m = class_size(b, ch);
+        if (m <= 0) continue;
         used[b] = true;
         CK(cudaStreamWaitEvent(c->aux[b], c->ev_fork, 0));
-        lm_launch_bucket<W>(a, wide_bucket(b), async, b, c->list + s0, (int)(s1 - s0), c->aux[b]);
+        lm_launch_bucket<W>(a, wide_bucket(b), async, b, c->list, c->key_off + b * P + ch, m, c->aux[b]);
       }
       int64_t h0 = ko[kHubBucket * P + ch] - hub0, h1 = ko[kHubBucket * P + ch + 1] - hub0;
       if (h1 > h0) {
@@ -819,7 +838,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
       }
       if (!async) {
         int64_t cls = 0;
-        for (int b = 0; b <= kHubBucket; ++b) cls += ko[b * P + ch + 1] - ko[b * P + ch];
+        for (int b = 0; b <= kHubBucket; ++b) cls += class_size(b, ch);
         lm_launch_commit<W>(a, cls, s);
       }
       CKLAUNCH();
@@ -830,7 +849,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
       lm_launch_hub_mark<W>(am, c->list + hub0, (int)nhubs, c->chunk_pre, hchunks[nhubs], s);
     }
     if (ahead) {
-      lm_decide(c->ctr, c->hist, c->d_iter, dbl((i128)c->M * c->M), tol, s);
+      lm_decide(c->ctr, c->h_hist, c->d_iter, dbl((i128)c->M * c->M), tol, s);
       return 0;
     }
     CK(cudaMemcpyAsync(c->h_ctr, c->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s));
@@ -881,7 +900,6 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // launches into no-ops when the phase has ended.
   auto queue_ahead = [&](int k) -> int {
     if (int r = enqueue(k)) return r;
-    CK(cudaMemcpyAsync(c->h_hist + (k & 3), c->hist + (k & 3), sizeof(DevCounters), cudaMemcpyDeviceToHost, s));
     CK(cudaEventRecord(c->ev_iter[k & 3], s));
     return 0;
   };
@@ -1646,7 +1664,7 @@ static int arena_pieces(louvain_ctx* c, int64_t n, int64_t nnz) {
     ALLOC(c->tmp, (int64_t)c->tmp_bytes);
   }
   ALLOC(c->ctr, 1);
-  ALLOC(c->hist, 4);
+  ALLOC(c->draw, kDrawScratch);
   ALLOC(c->acc, 8);
   ALLOC(c->flags, 4);
   ALLOC(c->d_iter, 4);
@@ -1902,6 +1920,7 @@ int load_graphs(louvain_ctx* c, int64_t G, const int64_t* vo, int64_t n, int64_t
     CK(cudaMemsetAsync(c->gvals, 0, 2 * c->cap_nnz * sizeof(unsigned long long), s));
     CK(cudaMemsetAsync(c->hkid, 0, (c->cap_n + 1) * sizeof(unsigned long long), s));
     CK(cudaMemsetAsync(c->hdone, 0, (c->cap_n + 1) * sizeof(int32_t), s));
+    CK(cudaMemsetAsync(c->draw, 0, kDrawScratch * sizeof(unsigned), s));
     c->tables_dirty = false;
   }
   if (c->opt.validate) {

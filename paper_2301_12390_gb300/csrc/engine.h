@@ -104,9 +104,11 @@ __device__ __forceinline__ int vertex_class(int64_t i, const int32_t* gid, const
 }
 
 // ------------------------------------------------------ local_move.cu
+// The vertices list[ko[0] .. ko[1]) of a (bucket, class), offsets read on the
+// device; nverts: their number, or an estimate, for the size of the grid.
 template <typename W>
-void lm_launch_bucket(const LMArgs<W>& a, bool wide, bool async, int bucket, const int32_t* verts, int nverts,
-                      cudaStream_t s);
+void lm_launch_bucket(const LMArgs<W>& a, bool wide, bool async, int bucket, const int32_t* list, const int64_t* ko,
+                      int64_t nverts, cudaStream_t s);
 template <typename W>
 void lm_launch_hubs(const LMArgs<W>& a, bool wide, bool async, const int32_t* hubs, int nhubs,
                     const int64_t* chunk_pre, int64_t nchunks, const int64_t* spre, int64_t nslotchunks,
@@ -154,9 +156,10 @@ void lm_launch_hub_mark(const LMArgs<W>& a, const int32_t* hubs, int nhubs, cons
                         cudaStream_t s);
 template <typename W>
 void lm_launch_commit(const LMArgs<W>& a, int64_t max_moves, cudaStream_t s);
-// One graph: the iteration's counters to hist[iteration mod 4] and the stop
-// test on the device (MM = M^2 as a double); *d_iter moves on or to -1.
-void lm_decide(const DevCounters* ctr, DevCounters* hist, int* d_iter, double MM, double tol, cudaStream_t s);
+// One graph: the iteration's counters to hist[iteration mod 4] (pinned host
+// memory) and cleared, and the stop test on the device (MM = M^2 as a double);
+// *d_iter moves on or to -1.
+void lm_decide(DevCounters* ctr, DevCounters* hist, int* d_iter, double MM, double tol, cudaStream_t s);
 
 // ------------------------------------------------------- graph_ops.cu
 
@@ -173,23 +176,37 @@ size_t partition_tmp_bytes(int64_t n, int nkeys);
 void stable_partition(const int32_t* key, int64_t n, int nkeys, int32_t* out, int64_t* key_off, void* tmp,
                       cudaStream_t s);
 
-// Keys for the local-moving lists, bucket-major: key[i] = bucket * P + class
-// of vertex i (P >= Ps, Pb); vertices of degree 0 get the trailing key
-// kBuckets * P.
-// active (may be null): the stamps of this iteration; with it, vertices not
-// active in it get the trailing key, and so do those of a graph that does not
-// iterate (g_on, may be null).
-// K (may be null): bit b of *wmask is set when a vertex of bucket b has a
-// degree above klimit.
-void lm_keys(const int64_t* off, int64_t n, int P, int32_t* key, const int32_t* gid, const int64_t* vo,
-             const int32_t* gcat, ClassSpec cs, const int* d_iter, LMThresholds th, const int32_t* active,
-             const int32_t* g_on, const long long* K, long long klimit, unsigned long long* wmask, cudaStream_t s);
-// lm_keys for the m vertices sub[0..m) (with `active`, as lm_keys);
-// gather_ids: out[j] = sub[idx[j]].
-void lm_keys_sub(const int64_t* off, const int32_t* sub, int64_t m, int P, int32_t* key, const int32_t* gid,
-                 const int64_t* vo, const int32_t* gcat, ClassSpec cs, const int* d_iter, LMThresholds th,
-                 const int32_t* active, const int32_t* g_on, cudaStream_t s);
-void gather_ids(const int32_t* idx, const int32_t* sub, int64_t m, int32_t* out, cudaStream_t s);
+// The local-moving lists: list = the vertices by key = bucket * P + class
+// (P >= Ps, Pb), in no particular order within a key; key_off[nkeys + 1]
+// (nkeys = kBuckets * P + 1) their offsets, the vertices without a bucket
+// counted under the last key and not listed.  sub (may be null): the m vertices
+// sub[0..m) instead of [0, m).  active (may be null): the stamps of this
+// iteration; with it, vertices not active in it are not listed, and neither are
+// those of a graph that does not iterate (g_on, may be null).  K (may be null):
+// bit b of *wmask is set when a vertex of bucket b has a degree above klimit.
+// scratch: kDrawScratch words, zero before the first draw (left so).
+constexpr int kDrawKeys = kBuckets * 64 + 8, kDrawScratch = 2 * kDrawKeys + 8;
+struct DrawArgs {
+  const int64_t* off;
+  const int32_t* sub;
+  int64_t m;
+  int P;
+  const int32_t* gid;
+  const int64_t* vo;
+  const int32_t* gcat;
+  ClassSpec cs;
+  const int* d_iter;
+  LMThresholds th;
+  const int32_t* active;
+  const int32_t* g_on;
+  const long long* K;
+  long long klimit;
+  unsigned long long* wmask;
+};
+// draw_lists_stable: ascending within a key, the vertices without a bucket last
+// (sub null).
+void draw_lists_stable(const DrawArgs& d, int32_t* key, int32_t* list, int64_t* key_off, void* tmp, cudaStream_t s);
+void draw_lists(const DrawArgs& d, uint16_t* key, int32_t* list, int64_t* key_off, unsigned* scratch, cudaStream_t s);
 // For the hub list: per hub its table base (2 * degree slots), the prefix of
 // its insert chunks and the prefix of its slot chunks (each nhubs + 1 long).
 void hub_layout(const int64_t* off, const int32_t* hubs, int64_t nhubs, int64_t* hbase, int64_t* chunk_pre,

@@ -415,9 +415,12 @@ __device__ __forceinline__ void thread_vertex(const LMArgs<W>& a, const IterView
 // shared memory until 32 are there: with pruning most lanes of a warp would
 // otherwise idle through the others' rows.
 template <typename W, bool WIDE, bool ASYNC>
-__global__ void __launch_bounds__(256, 3) lm_thread(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
+__global__ void __launch_bounds__(256, 3) lm_thread(LMArgs<W> a, const int32_t* __restrict__ list,
+    const int64_t* __restrict__ ko) {
   const IterView iv = iter_view(a);
   if (iv.iter < 0) return;
+  const int32_t* __restrict__ verts = list + ko[0];
+  const int nverts = (int)(ko[1] - ko[0]);
   __shared__ BlockAcc acc;
   __shared__ int32_t queue[8][2 * kWarp];
   acc_init(acc);
@@ -580,9 +583,12 @@ __device__ __forceinline__ void thread_vertex_sorted(const LMArgs<W>& a, const I
 }
 
 template <typename W, bool ASYNC, int D>
-__global__ void __launch_bounds__(128) lm_thread_sorted(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
+__global__ void __launch_bounds__(128) lm_thread_sorted(LMArgs<W> a, const int32_t* __restrict__ list,
+    const int64_t* __restrict__ ko) {
   const IterView iv = iter_view(a);
   if (iv.iter < 0) return;
+  const int32_t* __restrict__ verts = list + ko[0];
+  const int nverts = (int)(ko[1] - ko[0]);
   __shared__ BlockAcc acc;
   acc_init(acc);
   __syncthreads();
@@ -708,9 +714,12 @@ __device__ __forceinline__ void warp_vertex(const LMArgs<W>& a, const IterView& 
 // U entries per lane cover the bucket's largest degree: the row is loaded and
 // gathered before any insert, so its memory latencies overlap.
 template <typename W, bool WIDE, bool ASYNC, int CAP, int U>
-__global__ void __launch_bounds__(256, 4) lm_warp(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
+__global__ void __launch_bounds__(256, 4) lm_warp(LMArgs<W> a, const int32_t* __restrict__ list,
+    const int64_t* __restrict__ ko) {
   const IterView iv = iter_view(a);
   if (iv.iter < 0) return;
+  const int32_t* __restrict__ verts = list + ko[0];
+  const int nverts = (int)(ko[1] - ko[0]);
   typedef typename TableVal<WIDE>::T V;
   constexpr int WPB = 8;
   __shared__ int32_t skeys[WPB][CAP];
@@ -1322,9 +1331,11 @@ __device__ __forceinline__ bool decide_move(const LMArgs<W>& a, BlockAcc& acc, i
 // 12288-degree instance in place of the hub chain and 4096-entry hub chunks.
 template <typename W, bool WIDE, bool ASYNC, int CAP, int THREADS, int U>
 __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ? 2 : 1)
-    lm_block(LMArgs<W> a, const int32_t* __restrict__ verts, int nverts) {
+    lm_block(LMArgs<W> a, const int32_t* __restrict__ list, const int64_t* __restrict__ ko) {
   const IterView iv = iter_view(a);
   if (iv.iter < 0) return;
+  const int32_t* __restrict__ verts = list + ko[0];
+  const int nverts = (int)(ko[1] - ko[0]);
   typedef typename Arith<WIDE>::S S;
   typedef typename TableVal<WIDE>::T V;
   constexpr int NW = THREADS / kWarp;
@@ -1655,17 +1666,19 @@ __global__ void __launch_bounds__(256) lm_commit(LMArgs<W> a) {
 }
 
 // The end of an iteration of one graph, on the device: its counters go to
-// slot (iteration mod 4) of hist, and the iteration number moves on, or to -1
+// slot (iteration mod 4) of hist (pinned host memory: no copy to queue) and are
+// cleared for the next one, and the iteration number moves on, or to -1
 // when the phase ends (the stop test of the host, on the same roundings), which
 // makes the launches of an iteration queued behind it return at once.
-__global__ void lm_decide_k(const DevCounters* ctr, DevCounters* hist, int* d_iter, double MM, double tol) {
+__global__ void lm_decide_k(DevCounters* ctr, DevCounters* hist, int* d_iter, double MM, double tol) {
   const int it = *d_iter;
   if (it < 0) return;
   hist[it & 3] = *ctr;
   const u128 S = ((u128)ctr->s_hi << 64) | (u128)ctr->s_lo;
   *d_iter = (2.0 * u128_to_double(S)) / MM <= tol ? -1 : it + 1;
+  memset(ctr, 0, sizeof(DevCounters));
 }
-void lm_decide(const DevCounters* ctr, DevCounters* hist, int* d_iter, double MM, double tol, cudaStream_t s) {
+void lm_decide(DevCounters* ctr, DevCounters* hist, int* d_iter, double MM, double tol, cudaStream_t s) {
   (count_launch(), lm_decide_k<<<1, 1, 0, s>>>(ctr, hist, d_iter, MM, tol));
 }
 
@@ -1674,7 +1687,7 @@ void lm_decide(const DevCounters* ctr, DevCounters* hist, int* d_iter, double MM
 namespace {
 
 template <typename K>
-int grid_for(K kernel, int threads, size_t smem, int work_blocks) {
+int grid_for(K kernel, int threads, size_t smem, int64_t work_blocks) {
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -1684,46 +1697,46 @@ int grid_for(K kernel, int threads, size_t smem, int work_blocks) {
   }
   const int per_sm = blocks_per_sm(kernel, threads, smem);
   int g = sms * per_sm;
-  if (work_blocks < g) g = work_blocks;
+  if (work_blocks < g) g = (int)work_blocks;
   return g < 1 ? 1 : g;
 }
 
 template <typename W, bool WIDE, bool ASYNC, int CAP, int THREADS, int U>
-void launch_block_t(const LMArgs<W>& a, const int32_t* verts, int nverts, cudaStream_t s) {
+void launch_block_t(const LMArgs<W>& a, const int32_t* list, const int64_t* ko, int64_t nverts, cudaStream_t s) {
   const size_t smem = (size_t)CAP * (sizeof(typename TableVal<WIDE>::T) + 4);
   auto k = lm_block<W, WIDE, ASYNC, CAP, THREADS, U>;
   static std::atomic<unsigned long long> attr{0};
   smem_limit_once(attr, k, smem);
-  (count_launch(), k<<<grid_for(k, THREADS, smem, nverts), THREADS, smem, s>>>(a, verts, nverts));
+  (count_launch(), k<<<grid_for(k, THREADS, smem, nverts), THREADS, smem, s>>>(a, list, ko));
 }
 
 template <typename W, bool WIDE, bool ASYNC>
-void launch_bucket_t(const LMArgs<W>& a, int bucket, const int32_t* verts, int nverts, cudaStream_t s) {
+void launch_bucket_t(const LMArgs<W>& a, int bucket, const int32_t* list, const int64_t* ko, int64_t nverts, cudaStream_t s) {
   if (nverts <= 0) return;
   switch (bucket) {
     case 0: {
       auto k = lm_thread<W, WIDE, ASYNC>;
-      (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 255) / 256), 256, 0, s>>>(a, verts, nverts));
+      (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 255) / 256), 256, 0, s>>>(a, list, ko));
       break;
     }
     case 1: {
       if (!WIDE) {   // narrow sums: a lane per vertex, its row sorted in registers
         auto k = lm_thread_sorted<W, ASYNC, 32>;
-        (count_launch(), k<<<grid_for(k, 128, 0, (nverts + 127) / 128), 128, 0, s>>>(a, verts, nverts));
+        (count_launch(), k<<<grid_for(k, 128, 0, (nverts + 127) / 128), 128, 0, s>>>(a, list, ko));
       } else {
         auto k = lm_warp<W, WIDE, ASYNC, 64, 1>;
-        (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 7) / 8), 256, 0, s>>>(a, verts, nverts));
+        (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 7) / 8), 256, 0, s>>>(a, list, ko));
       }
       break;
     }
     case 2: {
       auto k = lm_warp<W, WIDE, ASYNC, 256, 4>;
-      (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 7) / 8), 256, 0, s>>>(a, verts, nverts));
+      (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 7) / 8), 256, 0, s>>>(a, list, ko));
       break;
     }
-    case 3: launch_block_t<W, WIDE, ASYNC, 2048, 128, 8>(a, verts, nverts, s); break;
-    case 4: launch_block_t<W, WIDE, ASYNC, 8192, 512, 8>(a, verts, nverts, s); break;
-    case 5: launch_block_t<W, WIDE, ASYNC, 18432, 1024, 12>(a, verts, nverts, s); break;
+    case 3: launch_block_t<W, WIDE, ASYNC, 2048, 128, 8>(a, list, ko, nverts, s); break;
+    case 4: launch_block_t<W, WIDE, ASYNC, 8192, 512, 8>(a, list, ko, nverts, s); break;
+    case 5: launch_block_t<W, WIDE, ASYNC, 18432, 1024, 12>(a, list, ko, nverts, s); break;
     default: break;
   }
 }
@@ -1731,14 +1744,14 @@ void launch_bucket_t(const LMArgs<W>& a, int bucket, const int32_t* verts, int n
 }  // namespace
 
 template <typename W>
-void lm_launch_bucket(const LMArgs<W>& a, bool wide, bool async, int bucket, const int32_t* verts, int nverts,
-                      cudaStream_t s) {
+void lm_launch_bucket(const LMArgs<W>& a, bool wide, bool async, int bucket, const int32_t* list, const int64_t* ko,
+                      int64_t nverts, cudaStream_t s) {
   if (wide) {
-    if (async) launch_bucket_t<W, true, true>(a, bucket, verts, nverts, s);
-    else launch_bucket_t<W, true, false>(a, bucket, verts, nverts, s);
+    if (async) launch_bucket_t<W, true, true>(a, bucket, list, ko, nverts, s);
+    else launch_bucket_t<W, true, false>(a, bucket, list, ko, nverts, s);
   } else {
-    if (async) launch_bucket_t<W, false, true>(a, bucket, verts, nverts, s);
-    else launch_bucket_t<W, false, false>(a, bucket, verts, nverts, s);
+    if (async) launch_bucket_t<W, false, true>(a, bucket, list, ko, nverts, s);
+    else launch_bucket_t<W, false, false>(a, bucket, list, ko, nverts, s);
   }
 }
 
@@ -1826,8 +1839,10 @@ void lm_launch_commit(const LMArgs<W>& a, int64_t max_moves, cudaStream_t s) {
   (count_launch(), lm_commit<W><<<blocks, 256, 0, s>>>(a));
 }
 
-template void lm_launch_bucket<int32_t>(const LMArgs<int32_t>&, bool, bool, int, const int32_t*, int, cudaStream_t);
-template void lm_launch_bucket<int64_t>(const LMArgs<int64_t>&, bool, bool, int, const int32_t*, int, cudaStream_t);
+template void lm_launch_bucket<int32_t>(const LMArgs<int32_t>&, bool, bool, int, const int32_t*, const int64_t*,
+                                        int64_t, cudaStream_t);
+template void lm_launch_bucket<int64_t>(const LMArgs<int64_t>&, bool, bool, int, const int32_t*, const int64_t*,
+                                        int64_t, cudaStream_t);
 template void lm_launch_hubs<int32_t>(const LMArgs<int32_t>&, bool, bool, const int32_t*, int, const int64_t*,
                                       int64_t, const int64_t*, int64_t, cudaStream_t);
 template void lm_launch_hubs<int64_t>(const LMArgs<int64_t>&, bool, bool, const int32_t*, int, const int64_t*,
