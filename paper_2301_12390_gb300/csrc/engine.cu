@@ -375,6 +375,16 @@ int colour_pass(louvain_ctx* c, const PassState& g, int pass, int* ncls) {
   const int64_t* vo = multi ? c->vo : nullptr;
   const uint32_t salt = 0x9E3779B9u * (uint32_t)(pass + 1);
   int32_t* cls = c->members;
+  if (!multi && g.n <= kColourSmall && g.nnz <= kColourSmallEntries) {
+    colour_small(g.off, g.col, g.n, c->compacted ? c->isob[c->isob_cur] : nullptr, salt, cls, c->scal + 4, s);
+    CKLAUNCH();
+    int64_t got[3];
+    if (int e = fetch(c, got, c->scal + 4, sizeof(got))) return e;
+    if (got[0] != g.n || got[1])
+      return fail(c, LOUVAIN_ERR_INTERNAL, "colouring left a vertex without a class (asymmetric CSR?)");
+    *ncls = (int)got[2];
+    return 0;
+  }
   int32_t* cnt = c->inv;
   int32_t* front[2] = {(int32_t*)c->mdeg, (int32_t*)c->fill};
   const int64_t hslots = g.nnz / kColourHubDegree + 1;
@@ -382,12 +392,13 @@ int colour_pass(louvain_ctx* c, const PassState& g, int pass, int* ncls) {
   unsigned long long* hmask = (unsigned long long*)c->hpart;
   int32_t* hdone = c->hpart_c;
   if (hslots > c->npart) return fail(c, LOUVAIN_ERR_INTERNAL, "colouring: hub slots exceed the partial buffer");
-  // [0], [1]: frontier sizes; [2]: coloured; [3], [4]: hub frontier sizes (c->scal + 8)
+  // frontier sizes, hub frontier sizes (three of each in turn: read, filled,
+  // cleared), vertices coloured, largest class
   unsigned long long* sz = (unsigned long long*)(c->scal + 4);
-  unsigned long long* hsz = (unsigned long long*)(c->scal + 8);
-  int* cmax = (int*)(c->scal + 7);
-  CK(cudaMemsetAsync(sz, 0, 3 * sizeof(unsigned long long), s));
-  CK(cudaMemsetAsync(hsz, 0, 2 * sizeof(unsigned long long), s));
+  unsigned long long* hsz = (unsigned long long*)(c->scal + 7);
+  unsigned long long* ncoloured = (unsigned long long*)(c->scal + 10);
+  int* cmax = (int*)(c->scal + 11);
+  CK(cudaMemsetAsync(sz, 0, 8 * sizeof(unsigned long long), s));
   CK(cudaMemsetAsync(hmask, 0, hslots * sizeof(unsigned long long), s));
   CK(cudaMemsetAsync(hdone, 0, hslots * sizeof(int32_t), s));
   CK(cudaMemsetAsync(c->flags, 0, sizeof(int), s));
@@ -398,23 +409,19 @@ int colour_pass(louvain_ctx* c, const PassState& g, int pass, int* ncls) {
   for (;;) {
     for (int k = 0; k < kColourRoundsPerCheck; ++k, ++r) {
       const int a = (int)(r & 1), b = a ^ 1;
-      CK(cudaMemsetAsync(sz + b, 0, sizeof(unsigned long long), s));
-      CK(cudaMemsetAsync(hsz + b, 0, sizeof(unsigned long long), s));
-      colour_round(g.off, g.col, g.n, gid, vo, isob, zpre, salt, front[a], sz + a, hfront[a], hsz + a, cnt, cls,
-                   front[b],
-                   sz + b, hfront[b], hsz + b, sz + 2, hmask, hdone, c->flags, s);
+      const int ca = (int)(r % 3), cb = (int)((r + 1) % 3), cc = (int)((r + 2) % 3);
+      colour_round(g.off, g.col, g.n, gid, vo, isob, zpre, salt, front[a], sz + ca, hfront[a], hsz + ca, cnt, cls,
+                   front[b], sz + cb, hfront[b], hsz + cb, ncoloured, hmask, hdone, c->flags, sz + cc, hsz + cc, s);
     }
     CKLAUNCH();
-    unsigned long long left[2] = {0, 0};
-    if (int e = fetch(c, &left[0], sz + (r & 1), sizeof(unsigned long long))) return e;
-    if (int e = fetch(c, &left[1], hsz + (r & 1), sizeof(unsigned long long))) return e;
-    if (left[0] + left[1] == 0) break;
+    unsigned long long left[6];   // sz, hsz
+    if (int e = fetch(c, left, sz, sizeof(left))) return e;
+    if (left[r % 3] + left[3 + r % 3] == 0) break;
     if (r > g.n + kColourRoundsPerCheck) return fail(c, LOUVAIN_ERR_INTERNAL, "colouring did not end");
   }
   unsigned long long coloured = 0;
   int flags = 0;
-  if (int e = fetch(c, &coloured, sz + 2, sizeof(coloured))) return e;
-  if (int e = fetch(c, &flags, c->flags, sizeof(flags))) return e;
+  if (int e = fetch_pair(c, &coloured, ncoloured, sizeof(coloured), &flags, c->flags, sizeof(flags))) return e;
   if ((int64_t)coloured != g.n || (flags & 2))
     return fail(c, LOUVAIN_ERR_INTERNAL, "colouring left a vertex without a class (asymmetric CSR?)");
   CK(cudaMemsetAsync(cmax, 0, sizeof(int), s));

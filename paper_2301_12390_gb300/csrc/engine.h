@@ -352,7 +352,8 @@ void compact_vo(const int64_t* vo_full, int64_t G, const int32_t* pos, int64_t k
 // Colouring frontiers: vertices of degree above kColourHubDegree go to the
 // hub frontier (hfront / hnext), whose rows many blocks share; hmask / hdone
 // hold a zeroed mask and item counter per hub-frontier slot (at most
-// nnz / kColourHubDegree + 1 slots), left zeroed after every round.
+// nnz / kColourHubDegree + 1 slots), left zeroed after every round.  A round
+// clears the counters nclear / nhclear, which the round after next fills.
 constexpr int64_t kColourHubDegree = 2048;
 // isob / zpre: as in ClassSpec (priorities follow the full numbering).
 void colour_init(const int64_t* off, const int32_t* col, int64_t n, const int32_t* gid, const int64_t* vo,
@@ -363,7 +364,14 @@ void colour_round(const int64_t* off, const int32_t* col, int64_t n, const int32
                   const unsigned long long* nfront, const int32_t* hfront,
                   const unsigned long long* nhfront, int32_t* cnt, int32_t* cls, int32_t* next,
                   unsigned long long* nnext, int32_t* hnext, unsigned long long* nhnext, unsigned long long* total,
-                  unsigned long long* hmask, int32_t* hdone, int* flags, cudaStream_t s);
+                  unsigned long long* hmask, int32_t* hdone, int* flags, unsigned long long* nclear,
+                  unsigned long long* nhclear, cudaStream_t s);
+// The whole colouring of one graph of at most kColourSmall vertices, in one
+// launch (worth it up to kColourSmallEntries entries); out[0..2]: vertices
+// coloured, flags, classes.
+constexpr int64_t kColourSmall = 8192, kColourSmallEntries = 131072;
+void colour_small(const int64_t* off, const int32_t* col, int64_t n, const int32_t* isob, uint32_t salt, int32_t* cls,
+                  int64_t* out, cudaStream_t s);
 void class_max(const int32_t* cls, int64_t n, int* out, cudaStream_t s);
 void graph_ids(const int64_t* vo, int G, int64_t n, int64_t nnz, int32_t* gid, const int64_t* off, const int32_t* col,
                int32_t* crow /* merge-path scratch */, int* flags, cudaStream_t s);

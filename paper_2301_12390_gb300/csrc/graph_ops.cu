@@ -2113,8 +2113,10 @@ __global__ void colour_round_k(const int64_t* __restrict__ off, const int32_t* _
                                unsigned long long* __restrict__ nnext, int32_t* __restrict__ hnext,
                                unsigned long long* __restrict__ nhnext, unsigned long long* __restrict__ total,
                                unsigned long long* __restrict__ hmask, int32_t* __restrict__ hdone,
-                               int* __restrict__ flags) {
+                               int* __restrict__ flags, unsigned long long* __restrict__ nclear,
+                               unsigned long long* __restrict__ nhclear) {
   const int lane = threadIdx.x & 31;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *nclear = *nhclear = 0;   // the round after next counts there
   const int64_t nf = (int64_t)*nfront, nh = (int64_t)*nhfront;
   if (blockIdx.x == 0 && threadIdx.x == 0) *total += (unsigned long long)(nf + nh);
   const int64_t wblocks = (int64_t)gridDim.x - kColourHubBlocks;
@@ -2212,6 +2214,97 @@ __global__ void colour_round_k(const int64_t* __restrict__ off, const int32_t* _
   }
 }
 
+// A small graph's whole colouring by one block: counts, classes, priorities and
+// frontiers in shared memory, a round a block barrier, rows read through L1 and
+// L2.  The launches of a round cost 12-15 us whatever the frontier (road grid of
+// 4.2M vertices, last passes of about 860 vertices and 18,000 entries: 1.0 ms
+// each).  Same priorities and rule as above.  out: vertices coloured, flags
+// (as *flags above), classes.
+constexpr int kColourBlock = 1024;
+__global__ void __launch_bounds__(kColourBlock) colour_small_k(const int64_t* __restrict__ off,
+                                                               const int32_t* __restrict__ col, int n,
+                                                               const int32_t* __restrict__ isob, uint32_t salt,
+                                                               int32_t* __restrict__ cls, int64_t* __restrict__ out) {
+  extern __shared__ uint32_t csm[];
+  uint32_t* pri = csm;                                   // kColourSmall each
+  int32_t* cnt = (int32_t*)(pri + kColourSmall);
+  uint16_t* front = (uint16_t*)(cnt + kColourSmall);     // two lists
+  int8_t* c8 = (int8_t*)(front + 2 * kColourSmall);
+  __shared__ int s_n[2], s_bad, s_max;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  constexpr int NW = kColourBlock / kWarp;
+  if (tid == 0) s_n[0] = s_n[1] = s_bad = s_max = 0;
+  for (int v = tid; v < n; v += kColourBlock) {
+    pri[v] = hash32((uint32_t)(v + (isob ? isob[v] : 0)) ^ salt);
+    c8[v] = -1;
+  }
+  __syncthreads();
+  for (int v = wid; v < n; v += NW) {   // preceding neighbours
+    unsigned c = 0;
+    for (int64_t x = off[v] + lane; x < off[v + 1]; x += kWarp) {
+      const int u = __ldg(col + x);
+      if (u != v && (pri[u] > pri[v] || (pri[u] == pri[v] && u < v))) ++c;
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) {
+      cnt[v] = (int)c;
+      if (c == 0) front[atomicAdd(&s_n[0], 1)] = (uint16_t)v;
+    }
+  }
+  __syncthreads();
+  int done = 0, most = 0;
+  bool bad = false;
+  for (int r = 0;; r ^= 1) {
+    const int nf = s_n[r];
+    if (nf == 0) break;   // uniform
+    done += nf;
+    const uint16_t* f = front + r * kColourSmall;
+    uint16_t* g = front + (r ^ 1) * kColourSmall;
+    for (int t = wid; t < nf; t += NW) {
+      const int v = f[t];
+      const int64_t b = off[v], e = off[v + 1];
+      unsigned long long used = 0;
+      for (int64_t x = b + lane; x < e; x += kWarp) {
+        const int u = __ldg(col + x);
+        if (u == v || !(pri[u] > pri[v] || (pri[u] == pri[v] && u < v))) continue;
+        const int cu = c8[u];
+        if (cu >= 0) used |= 1ull << cu;
+        else bad = true;
+      }
+      const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)used);
+      const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(used >> 32));
+      const unsigned long long free_cls = ~(((unsigned long long)hi << 32) | lo) & 0x7fffffffffffffffull;
+      const int c = free_cls ? __ffsll((long long)free_cls) - 1 : 63;
+      most = max(most, c);
+      if (lane == 0) c8[v] = (int8_t)c;
+      for (int64_t x = b + lane; x < e; x += kWarp) {
+        const int u = __ldg(col + x);
+        if (u == v || !(pri[v] > pri[u] || (pri[v] == pri[u] && v < u))) continue;
+        if (atomicSub(cnt + u, 1) == 1) g[atomicAdd(&s_n[r ^ 1], 1)] = (uint16_t)u;
+      }
+    }
+    __syncthreads();
+    if (tid == 0) s_n[r] = 0;
+    __syncthreads();
+  }
+  if (bad) s_bad = 1;
+  if (lane == 0) atomicMax(&s_max, most);
+  for (int v = tid; v < n; v += kColourBlock) cls[v] = c8[v];
+  __syncthreads();
+  if (tid == 0) {
+    out[0] = done;
+    out[1] = s_bad ? 2 : 0;
+    out[2] = s_max + 1;
+  }
+}
+void colour_small(const int64_t* off, const int32_t* col, int64_t n, const int32_t* isob, uint32_t salt, int32_t* cls,
+                  int64_t* out, cudaStream_t s) {
+  const size_t smem = (size_t)kColourSmall * (4 + 4 + 2 * 2 + 1);
+  static std::atomic<unsigned long long> attr{0};
+  smem_limit_once(attr, colour_small_k, smem);
+  (count_launch(), colour_small_k<<<1, kColourBlock, smem, s>>>(off, col, (int)n, isob, salt, cls, out));
+}
+
 __global__ void class_max_k(const int32_t* __restrict__ cls, int64_t n, int* __restrict__ out) {
   int m = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -2236,10 +2329,11 @@ void colour_round(const int64_t* off, const int32_t* col, int64_t n, const int32
                   const unsigned long long* nfront, const int32_t* hfront,
                   const unsigned long long* nhfront, int32_t* cnt, int32_t* cls, int32_t* next,
                   unsigned long long* nnext, int32_t* hnext, unsigned long long* nhnext, unsigned long long* total,
-                  unsigned long long* hmask, int32_t* hdone, int* flags, cudaStream_t s) {
+                  unsigned long long* hmask, int32_t* hdone, int* flags, unsigned long long* nclear,
+                  unsigned long long* nhclear, cudaStream_t s) {
   (count_launch(), colour_round_k<<<warp_grid(n) + kColourHubBlocks, 256, 0, s>>>(
                        off, col, gid, vo, isob, zpre, salt, front, nfront, hfront, nhfront, cnt, cls, next, nnext,
-                       hnext, nhnext, total, hmask, hdone, flags));
+                       hnext, nhnext, total, hmask, hdone, flags, nclear, nhclear));
 }
 void class_max(const int32_t* cls, int64_t n, int* out, cudaStream_t s) {
   if (n > 0) (count_launch(), class_max_k<<<grid1d(n), kT, 0, s>>>(cls, n, out));
