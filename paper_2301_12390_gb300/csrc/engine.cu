@@ -1164,6 +1164,36 @@ int aggregate(louvain_ctx* c, const PassState& g, int64_t k, PassState* next, st
   return 0;
 }
 
+// The same for a small pass graph, renumbering included: *k communities.
+template <typename W, typename W2>
+int aggregate_small(louvain_ctx* c, const PassState& g, int64_t* k, PassState* next, std::vector<i128>& nafter) {
+  cudaStream_t s = c->stream;
+  const int dst = g.widx == 0 ? 1 : 0;
+  SmallAgg r{g.off, g.col, g.w, g.n, c->memb, c->sig, c->compacted ? c->isob[c->isob_cur] : nullptr,
+             c->compacted ? c->isob[c->isob_cur ^ 1] : nullptr, c->level, c->Knext, c->cstart, c->members, c->inv,
+             c->mpre, c->rlen, c->list, c->key_off, c->scal, c->tcol, c->tw, c->offX[dst], c->colX[dst], c->wX[dst],
+             c->acc, c->flags};
+  agg_small<W, W2>(r, c->tmp, s);
+  compose_top(c->top, c->n0, c->level, s);
+  CKLAUNCH();
+  if (c->compacted) c->isob_cur ^= 1;
+  int64_t nnz2 = 0;
+  int flag = 0;
+  if (int e = fetch_many(c, {{k, c->scal, sizeof(int64_t)}, {&nnz2, c->offX[dst] + g.n, sizeof(int64_t)},
+                             {&flag, c->flags, sizeof(int)}, {c->h_acc, c->acc, 8 * sizeof(unsigned long long)}}))
+    return e;
+  if (flag) return fail(c, LOUVAIN_ERR_INTERNAL, "aggregation: hash table overflow");
+  u128 SS = ((u128)c->h_acc[5] << 64) | (u128)c->h_acc[4];
+  nafter[0] = (i128)c->M * (i128)c->h_acc[6] - (i128)SS;
+  next->n = *k;
+  next->nnz = nnz2;
+  next->off = c->offX[dst];
+  next->col = c->colX[dst];
+  next->w = (void*)c->wX[dst];
+  next->widx = dst;
+  return 0;
+}
+
 template <typename W2>
 int record_coarse(louvain_ctx* c, PassRec& pr, const PassState& h) {
   pr.coff.resize(h.n + 1);
@@ -1359,45 +1389,51 @@ int run_pass(louvain_ctx* c, const PassState& g, int pass, double* tol, bool wid
     *stop = true;
     return 0;
   }
-  // renumber by ascending old id and compose the top level; with several
-  // graphs each graph's communities stay contiguous and in order
-  mark_used(c->memb, g.n, c->used, s);
-  scan_i32(c->used, c->newid, g.n, c->scal, c->tmp, s);
-  apply_level(c->memb, c->newid, g.n, c->level, s);
-  compose_top(c->top, c->n0, c->level, s);
-  if (multi) {
-    CK(cudaMemsetAsync(c->kcount, 0, (G + 1) * sizeof(int64_t), s));
-    graph_renumber(c->used, c->newid, c->gid, g.n, c->kcount, c->gid_next, s);
-    scan_i64(c->kcount, c->vo_next, G, c->vo_next + G, c->tmp, s);
-    CK(cudaMemcpyAsync(c->vo_top, c->vo_next, (G + 1) * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-  }
-  if (c->compacted) {
-    carry_isob(c->used, c->newid, c->isob[c->isob_cur], g.n, c->isob[c->isob_cur ^ 1], s);
-    c->isob_cur ^= 1;
-  }
-  CKLAUNCH();
   int64_t k = 0;
   std::vector<int64_t> vo_next;
-  if (multi) {
-    vo_next.resize(G + 1);
-    if (int r = fetch_pair(c, &k, c->scal, sizeof(int64_t), vo_next.data(), c->vo_next, (G + 1) * sizeof(int64_t)))
-      return r;
-  } else {
-    if (int r = fetch(c, &k, c->scal, sizeof(int64_t))) return r;
-  }
-  if (c->compacted) c->kc_top = k;
-  c->vo_host_next = vo_next;
-  // If another pass may follow, aggregate first: the coarse self-loops give
-  // sum_C L_C, so the pass's Q numerators cost no extra scan of the graph; a
-  // coarse graph built for a pass after which every graph stops is dropped.
   std::vector<i128> nafter(G, 0);
   bool built = false;
-  if (pass + 1 < c->opt.max_passes) {
-    if (int r = aggregate<W, W2>(c, g, k, next, nafter)) return r;
+  const bool another = pass + 1 < c->opt.max_passes;
+  if (!multi && another && g.n <= kAggSmall && g.nnz <= kAggSmallEntries) {
+    if (int r = aggregate_small<W, W2>(c, g, &k, next, nafter)) return r;
     built = true;
   } else {
-    if (int r = q_numerators<W>(c, g, nafter)) return r;
+    // renumber by ascending old id and compose the top level; with several
+    // graphs each graph's communities stay contiguous and in order
+    mark_used(c->memb, g.n, c->used, s);
+    scan_i32(c->used, c->newid, g.n, c->scal, c->tmp, s);
+    apply_level(c->memb, c->newid, g.n, c->level, s);
+    compose_top(c->top, c->n0, c->level, s);
+    if (multi) {
+      CK(cudaMemsetAsync(c->kcount, 0, (G + 1) * sizeof(int64_t), s));
+      graph_renumber(c->used, c->newid, c->gid, g.n, c->kcount, c->gid_next, s);
+      scan_i64(c->kcount, c->vo_next, G, c->vo_next + G, c->tmp, s);
+      CK(cudaMemcpyAsync(c->vo_top, c->vo_next, (G + 1) * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    }
+    if (c->compacted) {
+      carry_isob(c->used, c->newid, c->isob[c->isob_cur], g.n, c->isob[c->isob_cur ^ 1], s);
+      c->isob_cur ^= 1;
+    }
+    CKLAUNCH();
+    if (multi) {
+      vo_next.resize(G + 1);
+      if (int r = fetch_pair(c, &k, c->scal, sizeof(int64_t), vo_next.data(), c->vo_next, (G + 1) * sizeof(int64_t)))
+        return r;
+    } else {
+      if (int r = fetch(c, &k, c->scal, sizeof(int64_t))) return r;
+    }
+    c->vo_host_next = vo_next;
+    // If another pass may follow, aggregate first: the coarse self-loops give
+    // sum_C L_C, so the pass's Q numerators cost no extra scan of the graph; a
+    // coarse graph built for a pass after which every graph stops is dropped.
+    if (another) {
+      if (int r = aggregate<W, W2>(c, g, k, next, nafter)) return r;
+      built = true;
+    } else {
+      if (int r = q_numerators<W>(c, g, nafter)) return r;
+    }
   }
+  if (c->compacted) c->kc_top = k;
   CK(cudaEventRecord(c->ev[3], s));
   bool all_stopped = true;
   for (int64_t q = 0; q < G; ++q) {

@@ -319,6 +319,41 @@ template <typename W2>
 void agg_compact(const int64_t* cstart, const int64_t* mpre, const int64_t* coff, int64_t k, int64_t nnz2,
                  int32_t* crow, const int32_t* tcol, const W2* tw, int32_t* ocol, W2* ow, cudaStream_t s);
 
+// Renumbering and aggregation of one small pass graph, without a host read in
+// between (at most kAggSmall vertices and kAggSmallEntries entries): what
+// mark_used .. agg_compact do, in seven launches.  r.acc as in aggregate() ([4..5]
+// sum of Sigma^2, [6] coarse self-loops), r.k[0] the communities.
+constexpr int64_t kAggSmall = 8192, kAggSmallEntries = 131072;
+struct SmallAgg {
+  const int64_t* off;
+  const int32_t* col;
+  const void* wt;            // W
+  int64_t n;
+  const int32_t* memb;
+  const long long* sig;
+  const int32_t* isob;       // compact pass graph: isolated counts, carried to isob_next (else null)
+  int32_t* isob_next;
+  int32_t* level;
+  long long* Knext;
+  int64_t* cstart;
+  int32_t* members;
+  int32_t* inv;
+  int64_t* mpre;
+  int64_t* rlen;
+  int32_t* list;
+  int64_t* ko;               // 4: communities of at most 128 entries list[ko[0] .. ko[1]), larger ones [ko[2] .. ko[3])
+  int64_t* k;
+  int32_t* tcol;
+  void* tw;                  // W2
+  int64_t* coff;             // coarse CSR: n + 1 offsets (all of them written), columns, weights
+  int32_t* ocol;
+  void* ow;                  // W2
+  unsigned long long* acc;   // 8
+  int* flags;
+};
+template <typename W, typename W2>
+void agg_small(const SmallAgg& r, void* tmp, cudaStream_t s);
+
 // Several graphs in one CSR (contiguous vertex ranges per graph).
 void graph_totals(const long long* K, const int32_t* gid, int64_t n, unsigned long long* Mg, cudaStream_t s);
 template <typename W>

@@ -4,6 +4,8 @@
 // are merged with summed weights, edges inside one become a summed
 // self-loop).  No library primitives: scan and partition are our own.
 #include <type_traits>
+#include <algorithm>
+#include <cstring>
 #include "common.cuh"
 #include "engine.h"
 
@@ -1364,8 +1366,13 @@ __global__ void __launch_bounds__(256) agg_thread_k(AggArgs a, const int32_t* __
 // shared memory; the coarse row is written back over the community's tmp
 // entries (all of them are read before the first write).
 template <typename W2, int CAP>
-__global__ void __launch_bounds__(256) agg_warp_k(AggArgs a, const int32_t* __restrict__ comms, int ncomms) {
+__global__ void __launch_bounds__(256) agg_warp_k(AggArgs a, const int32_t* __restrict__ comms, int ncomms,
+                                                  const int64_t* __restrict__ ko) {
   typedef AggVal<W2> V;
+  if (ko) {   // the communities comms[ko[0] .. ko[1]) (agg_small: not known on the host)
+    comms += ko[0];
+    ncomms = (int)(ko[1] - ko[0]);
+  }
   constexpr int WPB = 8;
   constexpr int U = CAP / 2 / kWarp > 0 ? CAP / 2 / kWarp : 1;
   __shared__ int32_t skeys[WPB][CAP];
@@ -1659,7 +1666,7 @@ void agg_launch_bucket(const AggArgs& a, int bucket, const int32_t* comms, int n
     }
     case 2: {
       auto k = agg_warp_k<W2, 256>;
-      (count_launch(), k<<<agrid(k, 256, 0, (ncomms + 7) / 8), 256, 0, s>>>(a, comms, ncomms));
+      (count_launch(), k<<<agrid(k, 256, 0, (ncomms + 7) / 8), 256, 0, s>>>(a, comms, ncomms, nullptr));
       break;
     }
     case 3: {
@@ -2029,6 +2036,228 @@ __global__ void graph_entries_k(const int64_t* __restrict__ off, const int64_t* 
 void graph_entries(const int64_t* off, const int64_t* vo, int64_t G, int64_t* out, cudaStream_t s) {
   if (G > 0) (count_launch(), graph_entries_k<<<(unsigned)((G + kT - 1) / kT), kT, 0, s>>>(off, vo, G, out));
 }
+
+// ------------------------------------ small pass graphs: renumber, aggregate
+//
+// The later passes work on a few thousand vertices, and their renumbering and
+// aggregation took 35 launches and four host reads (0.19-0.25 ms) for work that
+// is microseconds.  One block does everything that is linear in the vertices
+// (renumbering, members grouped by community, prefixes, community lists); the
+// entries then take a launch each for relabelling, small and large communities,
+// and the rows' compaction, all sized on the device.
+
+constexpr int kRenumberThreads = 1024;
+
+// Exclusive scan of a[0 .. m) in shared memory by the whole block; returns the
+// sum, also left in a[m].
+__device__ __forceinline__ int small_scan(int* a, int m, int* warp_sums) {
+  constexpr int PER = (int)(kAggSmall / kRenumberThreads);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  __syncthreads();
+  int v[PER], sum = 0;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int i = tid * PER + j;
+    v[j] = i < m ? a[i] : 0;
+    sum += v[j];
+  }
+  int inc = sum;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= d) inc += u;
+  }
+  if (lane == 31) warp_sums[wid] = inc;
+  __syncthreads();
+  if (wid == 0) {
+    int w = warp_sums[lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, w, d);
+      if (lane >= d) w += u;
+    }
+    warp_sums[lane] = w;
+  }
+  __syncthreads();
+  int ex = inc - sum + (wid > 0 ? warp_sums[wid - 1] : 0);
+  const int total = warp_sums[31];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int i = tid * PER + j;
+    if (i < m) a[i] = ex;
+    ex += v[j];
+  }
+  if (tid == 0) a[m] = total;
+  __syncthreads();
+  return total;
+}
+
+__global__ void __launch_bounds__(kRenumberThreads) renumber_small_k(SmallAgg r) {
+  extern __shared__ int rsm[];
+  int* newid = rsm;                       // kAggSmall + 1 each
+  int* cnt = newid + kAggSmall + 1;
+  int* fill = cnt + kAggSmall + 1;
+  __shared__ int warp_sums[32];
+  __shared__ unsigned long long s_lo[32], s_hi[32];
+  __shared__ int s_c[2];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int n = (int)r.n;
+  for (int i = tid; i < n; i += kRenumberThreads) newid[i] = cnt[i] = fill[i] = 0;
+  if (tid < 2) s_c[tid] = 0;
+  __syncthreads();
+  for (int v = tid; v < n; v += kRenumberThreads) newid[r.memb[v]] = 1;
+  const int k = small_scan(newid, n, warp_sums);   // dense ids by ascending old id
+  u128 ss = 0;
+  for (int c = tid; c < n; c += kRenumberThreads) {
+    const unsigned long long sc = (unsigned long long)r.sig[c];
+    ss += (u128)sc * (u128)sc;
+    if (newid[c + 1] > newid[c]) {   // community c has members
+      r.Knext[newid[c]] = (long long)sc;
+      if (r.isob) r.isob_next[newid[c]] = r.isob[c];
+    }
+  }
+  for (int v = tid; v < n; v += kRenumberThreads) {
+    const int L = newid[r.memb[v]];
+    r.level[v] = L;
+    atomicAdd(&cnt[L], 1);
+  }
+  small_scan(cnt, k, warp_sums);
+  for (int c = tid; c <= k; c += kRenumberThreads) r.cstart[c] = cnt[c];
+  for (int v = tid; v < n; v += kRenumberThreads) {
+    const int L = r.level[v];   // this thread's own store
+    const int p = cnt[L] + atomicAdd(&fill[L], 1);
+    r.members[p] = v;
+    r.inv[v] = p;
+    newid[p] = (int)(r.off[v + 1] - r.off[v]);   // the renumbering is done: member degrees
+  }
+  small_scan(newid, n, warp_sums);
+  for (int p = tid; p <= n; p += kRenumberThreads) r.mpre[p] = newid[p];
+  for (int c = tid; c < n; c += kRenumberThreads) r.rlen[c] = 0;
+  for (int c = tid; c < k; c += kRenumberThreads) {
+    const int dsum = newid[cnt[c + 1]] - newid[cnt[c]];
+    if (dsum == 0) continue;
+    if (dsum <= 128) r.list[atomicAdd(&s_c[0], 1)] = c;
+    else r.list[n - 1 - atomicAdd(&s_c[1], 1)] = c;
+  }
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1)
+    ss += ((u128)__shfl_xor_sync(0xffffffffu, (unsigned long long)(ss >> 64), m) << 64) |
+          (u128)__shfl_xor_sync(0xffffffffu, (unsigned long long)ss, m);
+  if (lane == 0) {
+    s_lo[wid] = (unsigned long long)ss;
+    s_hi[wid] = (unsigned long long)(ss >> 64);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    u128 tot = 0;
+    for (int w = 0; w < 32; ++w) tot += ((u128)s_hi[w] << 64) | (u128)s_lo[w];
+    for (int j = 0; j < 8; ++j) r.acc[j] = 0;
+    r.acc[4] = (unsigned long long)tot;
+    r.acc[5] = (unsigned long long)(tot >> 64);
+    r.ko[0] = 0;
+    r.ko[1] = s_c[0];
+    r.ko[2] = n - s_c[1];
+    r.ko[3] = n;
+    r.k[0] = k;
+    *r.flags = 0;
+  }
+}
+
+// Relabelled member rows (as agg_relabel_k), a warp per row.
+template <typename W, typename W2>
+__global__ void __launch_bounds__(256) agg_relabel_rows_k(SmallAgg r) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < r.n; u += (int64_t)gridDim.x * 8) {
+    const int64_t b = r.off[u], e = r.off[u + 1], dst = r.mpre[r.inv[u]] - b;
+    for (int64_t x = b + lane; x < e; x += kWarp) {
+      r.tcol[dst + x] = r.level[r.col[x]];
+      ((W2*)r.tw)[dst + x] = (W2)((const W*)r.wt)[x];
+    }
+  }
+}
+
+// Communities of more than 128 entries, a block each: their sums indexed by
+// neighbour community (k values of shared memory), whatever their size.
+template <typename W2>
+__global__ void __launch_bounds__(256) agg_dense_k(AggArgs a, const int32_t* __restrict__ list,
+                                                   const int64_t* __restrict__ ko, const int64_t* __restrict__ kp) {
+  typedef AggVal<W2> V;
+  extern __shared__ unsigned long long ddyn[];
+  V* sums = (V*)ddyn;
+  __shared__ int scnt;
+  const int k = (int)*kp;
+  if (ko[0] + blockIdx.x >= ko[1]) return;
+  for (int t = threadIdx.x; t < k; t += 256) sums[t] = 0;
+  if (threadIdx.x == 0) scnt = 0;
+  __syncthreads();
+  SelfLoops sl;
+  for (int64_t ci = ko[0] + blockIdx.x; ci < ko[1]; ci += gridDim.x) {
+    const int32_t C = list[ci];
+    const int64_t vs = a.mpre[a.cstart[C]], ve = a.mpre[a.cstart[C + 1]];
+    for (int64_t x = vs + threadIdx.x; x < ve; x += 256) atomicAdd(&sums[a.tcol[x]], (V)((const W2*)a.tw)[x]);
+    __syncthreads();
+    for (int t = threadIdx.x; t < k; t += 256) {
+      const V v = sums[t];
+      if (!v) continue;
+      sums[t] = 0;
+      const int64_t pos = vs + atomicAdd(&scnt, 1);
+      a.tcol[pos] = t;
+      ((W2*)a.tw)[pos] = (W2)v;
+      if (t == C) sl.add(a, C, v);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      a.rlen[C] = scnt;
+      scnt = 0;
+    }
+    __syncthreads();
+  }
+  selfloops_finish(a, sl);
+}
+
+template <typename W2>
+__global__ void __launch_bounds__(256) agg_compact_rows_k(SmallAgg r) {
+  const int lane = threadIdx.x & 31;
+  const int64_t k = *r.k;
+  for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < k; c += (int64_t)gridDim.x * 8) {
+    const int64_t src = r.mpre[r.cstart[c]], dst = r.coff[c], len = r.coff[c + 1] - dst;
+    for (int64_t x = lane; x < len; x += kWarp) {
+      r.ocol[dst + x] = r.tcol[src + x];
+      ((W2*)r.ow)[dst + x] = ((const W2*)r.tw)[src + x];
+    }
+  }
+}
+
+template <typename W, typename W2>
+void agg_small(const SmallAgg& r, void* tmp, cudaStream_t s) {
+  const size_t smem = 3 * (kAggSmall + 1) * sizeof(int);
+  static std::atomic<unsigned long long> attr{0};
+  smem_limit_once(attr, renumber_small_k, smem);
+  (count_launch(), renumber_small_k<<<1, kRenumberThreads, smem, s>>>(r));
+  const unsigned rows = (unsigned)std::max<int64_t>(1, (r.n + 7) / 8);
+  (count_launch(), agg_relabel_rows_k<W, W2><<<rows, 256, 0, s>>>(r));
+  AggArgs a;
+  memset(&a, 0, sizeof(a));
+  a.cstart = r.cstart;
+  a.mpre = r.mpre;
+  a.tcol = r.tcol;
+  a.tw = r.tw;
+  a.rlen = r.rlen;
+  a.lsum = r.acc + 6;
+  a.error = r.flags;
+  auto kw = agg_warp_k<W2, 256>;
+  (count_launch(), kw<<<agrid(kw, 256, 0, (int)rows), 256, 0, s>>>(a, r.list, 0, r.ko));
+  auto kd = agg_dense_k<W2>;
+  const size_t dsmem = (size_t)kAggSmall * sizeof(AggVal<W2>);
+  static std::atomic<unsigned long long> dattr{0};
+  smem_limit_once(dattr, kd, dsmem);
+  (count_launch(), kd<<<agrid(kd, 256, dsmem, (int)(kAggSmallEntries / 128)), 256, dsmem, s>>>(a, r.list, r.ko + 2, r.k));
+  scan_i64(r.rlen, r.coff, r.n, r.coff + r.n, tmp, s);
+  (count_launch(), agg_compact_rows_k<W2><<<rows, 256, 0, s>>>(r));
+}
+template void agg_small<int32_t, int32_t>(const SmallAgg&, void*, cudaStream_t);
+template void agg_small<int32_t, int64_t>(const SmallAgg&, void*, cudaStream_t);
+template void agg_small<int64_t, int64_t>(const SmallAgg&, void*, cudaStream_t);
 
 // ------------------------------------------------------ colour classes
 //
