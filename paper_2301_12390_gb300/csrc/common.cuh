@@ -420,6 +420,9 @@ struct LMArgs {
   unsigned long long* g_s;      // per-graph S of the iteration (lo, hi)
   int prune;
   int guard;
+  // pruning by pull (see local_move.cu): this iteration's activity is found from
+  // the flags of the neighbours' memberships; its moves set flags, not stamps
+  int pull_check, pull_mark;
   // hub path: per-hub global tables (2 deg slots each, per class from slot 0)
   int32_t* hkeys;
   unsigned long long* hvals;
@@ -427,7 +430,7 @@ struct LMArgs {
   const int64_t* spre;       // first slot chunk of hub h (absolute within the pass)
   unsigned long long* hkid;  // K_{i->d} of hub h, looked up before the scan clears the table
   int32_t* hdone;            // scan blocks of hub h finished so far (back to 0 by the last one)
-  int32_t* hmoved;           // iteration + 1 when hub h moved in that iteration
+  int32_t* hmoved;           // iteration + 1 when hub h moved in that iteration (pull: minus that, a neighbour moved)
   long long* hpart;          // per slot chunk: best gain (lo, hi)
   int32_t* hpart_c;          // per slot chunk: its community
 };

@@ -156,6 +156,9 @@ void lm_launch_hub_mark(const LMArgs<W>& a, const int32_t* hubs, int nhubs, cons
                         cudaStream_t s);
 template <typename W>
 void lm_launch_commit(const LMArgs<W>& a, int64_t max_moves, cudaStream_t s);
+// Clears the flags of the moves of iteration iter (iter < 0: all flags) from the
+// membership words (pruning by pull).
+void lm_clear_flags(int32_t* memb, int64_t n, int iter, cudaStream_t s);
 // One graph: the iteration's counters to hist[iteration mod 4] (pinned host
 // memory) and cleared, and the stop test on the device (MM = M^2 as a double);
 // *d_iter moves on or to -1.

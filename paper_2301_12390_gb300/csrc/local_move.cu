@@ -20,6 +20,7 @@
 // list afterwards.  Asynchronous mode (Gauss-Seidel-like): a decision is
 // applied at once (memberships stored, totals and sizes updated with
 // atomics), so later decisions may see it.
+#include <algorithm>
 #include <climits>
 #include "common.cuh"
 #include "engine.h"
@@ -194,9 +195,29 @@ __device__ __forceinline__ IterView iter_view(const LMArgs<W>& a) {
   return IterView{it, a.stamps[it & 1], a.stamps[(it + 1) & 1]};
 }
 
-template <typename W>
+// Pruning by pull, while nearly every vertex is active (synchronous, one class).
+// A vertex is active when it or a neighbour moved in the iteration before.
+// Pushed, every mover rereads its row and stores a stamp per neighbour, twenty
+// stores for one vertex and most of them to the same hubs (R-MAT of 4.2M
+// vertices: 21 of 117 ms).  Instead a move sets a flag in the mover's own
+// membership word, one of two bits above the ids by the iteration's parity; a
+// vertex's row is gathered anyway, so it sees its neighbours' flags for nothing,
+// and only the few inactive vertices gather for nothing.  The flags are cleared
+// at the end of the iteration that read them.  Bound by the gathers of the
+// neighbours' words, as before; a run of the R-MAT graph went from 116.8 to
+// 100.5 ms, an incremental one of 1M vertices from 13.1 to 11.0, a 4096 x 4096
+// road grid from 36.1 to 34.6.
+constexpr int32_t kIdMask = 0x3fffffff;
+__device__ __forceinline__ int32_t moved_bit(int iter) { return (iter & 1) ? (int32_t)0x80000000 : 0x40000000; }
+// A membership word as a community id.
+template <bool PULL>
+__device__ __forceinline__ int32_t word_id(int32_t w) {
+  return PULL ? (w & kIdMask) : w;
+}
+
+template <bool PULL = false, typename W>
 __device__ __forceinline__ bool is_active(const LMArgs<W>& a, const IterView& iv, int32_t i) {
-  return !a.prune || iv.iter == 0 || iv.sr[i] == iv.iter;
+  return !a.prune || iv.iter == 0 || (PULL && a.pull_check) || iv.sr[i] == iv.iter;
 }
 
 // What a warp or block needs of a vertex before its row.
@@ -215,7 +236,7 @@ struct VertexRow {
 // nothing more.  Returns the lanes whose vertex is visited in this iteration.
 // A vertex's own community only changes by its own commit, so it may be read
 // ahead; its community's total and size are read when its row is.
-template <typename W, int LD>
+template <typename W, int LD, bool PULL = false>
 __device__ __forceinline__ unsigned vertex_window(const LMArgs<W>& a, const IterView& iv,
                                                   const int32_t* __restrict__ verts, int64_t nverts, int64_t first,
                                                   int64_t stride, int lane, VertexRow& r) {
@@ -224,7 +245,7 @@ __device__ __forceinline__ unsigned vertex_window(const LMArgs<W>& a, const Iter
   r = VertexRow{0, 0, 0, 0, 0, 0, 0};
   if (at < nverts) {
     r.i = verts[at];
-    if (is_active(a, iv, r.i) && (!a.gid || a.g_on[a.gid[r.i]])) {
+    if (is_active<PULL>(a, iv, r.i) && (!a.gid || a.g_on[a.gid[r.i]])) {
       on = true;
       r.b = a.off[r.i];
       r.deg = (int)(a.off[r.i + 1] - r.b);
@@ -295,10 +316,12 @@ __device__ __forceinline__ void append_moves(const LMArgs<W>& a, bool moved, int
 // row is loaded first and its neighbours' communities gathered with all loads
 // in flight; duplicates are then merged in registers.  gv: the gain of a move.
 // A synchronous move is left to the caller's append (to: its target).
-template <typename W, bool WIDE, bool ASYNC, int D>
+// *on is cleared when a vertex taken for active (PULL) is not.
+template <typename W, bool WIDE, bool ASYNC, bool PULL, int D>
 __device__ __forceinline__ bool thread_decide(const LMArgs<W>& a, const IterView& iv, BlockAcc& acc, int32_t i,
-                                              int64_t b, int deg, int32_t d, long long Ki, long long M, int graph,
-                                              int32_t* to, u128* gv, unsigned* n_cand) {
+                                              int64_t b, int deg, int32_t dw, long long Ki, long long M, int graph,
+                                              int32_t* to, u128* gv, unsigned* n_cand, bool* on) {
+  const int32_t d = word_id<PULL>(dw);
   typedef typename Arith<WIDE>::S S;
   typedef typename TableVal<WIDE>::T V;
   const long long sd = ld_sig<ASYNC>(a.sig + d);
@@ -313,6 +336,19 @@ __device__ __forceinline__ bool thread_decide(const LMArgs<W>& a, const IterView
   }
 #pragma unroll
   for (int k = 0; k < D; ++k) cc[k] = cc[k] != i ? ld_memb<ASYNC>(a.memb + cc[k]) : kEmpty;
+  if (PULL) {
+    int32_t seen = dw;
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+      if (cc[k] != kEmpty) {
+        seen |= cc[k];
+        cc[k] &= kIdMask;
+      }
+    if (a.pull_check && !(seen & moved_bit(iv.iter - 1))) {
+      *on = false;
+      return false;
+    }
+  }
 #pragma unroll
   for (int k = 1; k < D; ++k) {
     bool merged = false;
@@ -358,7 +394,7 @@ __device__ __forceinline__ bool thread_decide(const LMArgs<W>& a, const IterView
 // do) takes the instance that compares six pairs instead of 28.  Whole warps
 // sum their counters, moves and gains over the warp: per-lane atomics on the
 // block's counters serialise (measured: a third of the kernel's time).
-template <typename W, bool WIDE, bool ASYNC>
+template <typename W, bool WIDE, bool ASYNC, bool PULL = false>
 __device__ __forceinline__ void thread_vertices(const LMArgs<W>& a, const IterView& iv, BlockAcc& acc, int32_t i) {
   int64_t b = 0;
   int deg = 0, graph = 0;
@@ -375,21 +411,21 @@ __device__ __forceinline__ void thread_vertices(const LMArgs<W>& a, const IterVi
       M = a.Mg[graph];
     }
   }
-  bool moved = false;
+  bool moved = false, on = i >= 0;
   u128 gv = 0;
   unsigned n_cand = 0;
   const unsigned longest = __reduce_max_sync(0xffffffffu, (unsigned)deg);
   if (longest <= 4) {
     if (i >= 0)
-      moved = thread_decide<W, WIDE, ASYNC, 4>(a, iv, acc, i, b, deg, d, Ki, M, graph, &to, &gv, &n_cand);
+      moved = thread_decide<W, WIDE, ASYNC, PULL, 4>(a, iv, acc, i, b, deg, d, Ki, M, graph, &to, &gv, &n_cand, &on);
   } else {
     if (i >= 0)
-      moved = thread_decide<W, WIDE, ASYNC, 8>(a, iv, acc, i, b, deg, d, Ki, M, graph, &to, &gv, &n_cand);
+      moved = thread_decide<W, WIDE, ASYNC, PULL, 8>(a, iv, acc, i, b, deg, d, Ki, M, graph, &to, &gv, &n_cand, &on);
   }
-  if (moved && a.prune) mark_row<8>(a, iv, i, b, b + deg);
+  if (moved && a.prune && !(PULL && a.pull_mark)) mark_row<8>(a, iv, i, b, b + deg);
   if (!ASYNC) append_moves(a, moved, i, to);
-  const unsigned n_edges = __reduce_add_sync(0xffffffffu, (unsigned)deg);
-  const unsigned n_visited = (unsigned)__popc(__ballot_sync(0xffffffffu, i >= 0));
+  const unsigned n_edges = __reduce_add_sync(0xffffffffu, PULL && !on ? 0u : (unsigned)deg);
+  const unsigned n_visited = (unsigned)__popc(__ballot_sync(0xffffffffu, on));
   n_cand = __reduce_add_sync(0xffffffffu, n_cand);
   if ((threadIdx.x & 31) == 0 && n_visited) {
     atomicAdd(&acc.edges, (unsigned long long)n_edges);
@@ -414,7 +450,7 @@ __device__ __forceinline__ void thread_vertex(const LMArgs<W>& a, const IterView
 // The warp walks its list entries 32 at a time and queues the visited ones in
 // shared memory until 32 are there: with pruning most lanes of a warp would
 // otherwise idle through the others' rows.
-template <typename W, bool WIDE, bool ASYNC>
+template <typename W, bool WIDE, bool ASYNC, bool PULL>
 __global__ void __launch_bounds__(256, 3) lm_thread(LMArgs<W> a, const int32_t* __restrict__ list,
     const int64_t* __restrict__ ko) {
   const IterView iv = iter_view(a);
@@ -433,11 +469,11 @@ __global__ void __launch_bounds__(256, 3) lm_thread(LMArgs<W> a, const int32_t* 
     int32_t i = -1;
     if (base + lane < nverts) {
       i = verts[base + lane];
-      if (!is_active(a, iv, i) || (a.gid && !a.g_on[a.gid[i]])) i = -1;
+      if (!is_active<PULL>(a, iv, i) || (a.gid && !a.g_on[a.gid[i]])) i = -1;
     }
     const unsigned on = __ballot_sync(0xffffffffu, i >= 0);
     if (have == 0 && on == 0xffffffffu) {   // nothing to gather
-      thread_vertices<W, WIDE, ASYNC>(a, iv, acc, i);
+      thread_vertices<W, WIDE, ASYNC, PULL>(a, iv, acc, i);
       continue;
     }
     if (i >= 0) q[have + __popc(on & lanemask_lt_lm())] = i;
@@ -450,10 +486,10 @@ __global__ void __launch_bounds__(256, 3) lm_thread(LMArgs<W> a, const int32_t* 
       q[lane] = rest;
       have -= kWarp;
       __syncwarp();
-      thread_vertices<W, WIDE, ASYNC>(a, iv, acc, j);
+      thread_vertices<W, WIDE, ASYNC, PULL>(a, iv, acc, j);
     }
   }
-  if (have > 0) thread_vertices<W, WIDE, ASYNC>(a, iv, acc, lane < have ? q[lane] : -1);
+  if (have > 0) thread_vertices<W, WIDE, ASYNC, PULL>(a, iv, acc, lane < have ? q[lane] : -1);
   __syncthreads();
   acc_flush(acc, a.ctr);
 }
@@ -467,7 +503,7 @@ __global__ void __launch_bounds__(256, 3) lm_thread(LMArgs<W> a, const int32_t* 
 // runs' totals gathered in two halves (bounded registers).  Same decisions as
 // the warp kernel it replaces for narrow sums (K_{i->c} < 2^31).  All 32
 // lanes call it.
-template <typename W, bool ASYNC, int D>
+template <typename W, bool ASYNC, bool PULL, int D>
 __device__ __forceinline__ void thread_vertex_sorted(const LMArgs<W>& a, const IterView& iv, BlockAcc& acc,
                                                      const int32_t* __restrict__ verts, int64_t nverts, int64_t vi) {
   typedef typename Arith<false>::S S;
@@ -483,9 +519,9 @@ __device__ __forceinline__ void thread_vertex_sorted(const LMArgs<W>& a, const I
     if (vi >= nverts) break;
     const int32_t i = verts[vi];
     const int64_t b = a.off[i], e = a.off[i + 1];
-    const int32_t d = a.memb[i];
+    const int32_t dw = a.memb[i], d = word_id<PULL>(dw);
     const long long Ki = a.K[i];
-    if (!is_active(a, iv, i)) break;
+    if (!is_active<PULL>(a, iv, i)) break;
     long long M;
     if (!graph_of(a, i, &M, &graph)) break;
     const long long sd = ld_sig<ASYNC>(a.sig + d);
@@ -503,6 +539,16 @@ __device__ __forceinline__ void thread_vertex_sorted(const LMArgs<W>& a, const I
       const bool other = k[j] != i;   // a self-loop adds to no K_{i->c}
       k[j] = other ? ld_memb<ASYNC>(a.memb + k[j]) : kPast;
       if (!other) w[j] = 0u;
+    }
+    if (PULL) {
+      int32_t seen = dw;
+#pragma unroll
+      for (int j = 0; j < D; ++j)
+        if (k[j] != kPast) {
+          seen |= k[j];
+          k[j] &= kIdMask;
+        }
+      if (a.pull_check && !(seen & moved_bit(iv.iter - 1))) break;
     }
 #pragma unroll
     for (int kk = 2; kk <= D; kk <<= 1) {
@@ -568,7 +614,7 @@ __device__ __forceinline__ void thread_vertex_sorted(const LMArgs<W>& a, const I
                                                                    &gv, bsz);
     vert = i;
     to = bc;
-    if (moved && a.prune) mark_row<8>(a, iv, i, b, e);
+    if (moved && a.prune && !(PULL && a.pull_mark)) mark_row<8>(a, iv, i, b, e);
   } while (false);
   if (!ASYNC) append_moves(a, moved, vert, to);
   n_edges = __reduce_add_sync(0xffffffffu, n_edges);
@@ -582,7 +628,7 @@ __device__ __forceinline__ void thread_vertex_sorted(const LMArgs<W>& a, const I
   warp_move_totals(a, acc, moved, graph, gv);
 }
 
-template <typename W, bool ASYNC, int D>
+template <typename W, bool ASYNC, bool PULL, int D>
 __global__ void __launch_bounds__(128) lm_thread_sorted(LMArgs<W> a, const int32_t* __restrict__ list,
     const int64_t* __restrict__ ko) {
   const IterView iv = iter_view(a);
@@ -593,7 +639,7 @@ __global__ void __launch_bounds__(128) lm_thread_sorted(LMArgs<W> a, const int32
   acc_init(acc);
   __syncthreads();
   for (int base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < nverts; base += gridDim.x * blockDim.x)
-    thread_vertex_sorted<W, ASYNC, D>(a, iv, acc, verts, nverts, base + (int)(threadIdx.x & 31));
+    thread_vertex_sorted<W, ASYNC, PULL, D>(a, iv, acc, verts, nverts, base + (int)(threadIdx.x & 31));
   __syncthreads();
   acc_flush(acc, a.ctr);
 }
@@ -623,9 +669,10 @@ struct WarpTally {
 // The U entries of row v that this thread holds (entry u * step + lane0),
 // their communities gathered with all loads in flight; kEmpty for none and
 // for a self-loop.  Rounds from nu on hold nothing for any lane of the warp.
-template <int U, int LD, typename W, typename V>
-__device__ __forceinline__ void row_communities(const LMArgs<W>& a, const VertexRow& v, int lane0, int step, int nu,
-                                                int32_t (&cc)[U], V (&ww)[U]) {
+// PULL: returns the flags of the neighbours' words, or-ed.
+template <int U, int LD, bool PULL = false, typename W, typename V>
+__device__ __forceinline__ int32_t row_communities(const LMArgs<W>& a, const VertexRow& v, int lane0, int step, int nu,
+                                                   int32_t (&cc)[U], V (&ww)[U]) {
   const int32_t* __restrict__ col = a.col + v.b;
   const W* __restrict__ wt = a.wt + v.b;
 #pragma unroll
@@ -642,6 +689,16 @@ __device__ __forceinline__ void row_communities(const LMArgs<W>& a, const Vertex
   }
 #pragma unroll
   for (int u = 0; u < U; ++u) cc[u] = u < nu && cc[u] != v.i ? ld_state<LD>(a.memb + cc[u]) : kEmpty;
+  int32_t seen = 0;
+  if (PULL) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (cc[u] != kEmpty) {
+        seen |= cc[u];
+        cc[u] &= kIdMask;
+      }
+  }
+  return seen;
 }
 
 // One vertex of degree <= U * 32 by one warp: its neighbour communities summed
@@ -653,20 +710,23 @@ __device__ __forceinline__ void row_communities(const LMArgs<W>& a, const Vertex
 // table.  SIZES: a singleton under the guard loads its candidates' sizes with
 // their totals (one dependent load less before the decision; off where the
 // registers would spill).
-template <typename W, bool WIDE, bool ASYNC, int CAP, int U, int LD, bool SIZES>
-__device__ __forceinline__ void warp_vertex(const LMArgs<W>& a, const IterView& iv, BlockAcc& acc, int32_t* keys,
+// Returns whether the vertex was active (PULL: known only here).
+template <typename W, bool WIDE, bool ASYNC, int CAP, int U, int LD, bool SIZES, bool PULL = false>
+__device__ __forceinline__ bool warp_vertex(const LMArgs<W>& a, const IterView& iv, BlockAcc& acc, int32_t* keys,
                                             typename TableVal<WIDE>::T* vals, const VertexRow& v, int lane, bool& ok,
                                             unsigned& cands) {
   typedef typename Arith<WIDE>::S S;
   typedef typename TableVal<WIDE>::T V;
-  const long long sd = ld_state<LD>(a.sig + v.d);
-  const int32_t szd = ld_state<LD>(a.csize + v.d);
+  const int32_t d = word_id<PULL>(v.d);
+  const long long sd = ld_state<LD>(a.sig + d);
+  const int32_t szd = ld_state<LD>(a.csize + d);
   // rounds of 32 entries that hold at least one (the rest are skipped)
   const int nu = (v.deg + kWarp - 1) / kWarp;
   int32_t cc[U];
   V ww[U];
   int hs[U];
-  row_communities<U, LD>(a, v, lane, kWarp, nu, cc, ww);
+  const int32_t seen = row_communities<U, LD, PULL>(a, v, lane, kWarp, nu, cc, ww);
+  if (PULL && a.pull_check && !__any_sync(0xffffffffu, ((seen | v.d) & moved_bit(iv.iter - 1)) != 0)) return false;
   const unsigned fresh = table_add_row<CAP, U, V>(keys, vals, cc, ww, nu, hs, &ok);
   // one lane's reading for the whole warp: it decides which reduction below the
   // lanes take together, and an asynchronous size may change between two loads
@@ -675,9 +735,9 @@ __device__ __forceinline__ void warp_vertex(const LMArgs<W>& a, const IterView& 
   bool one[U];   // the candidate is a singleton (asked only for the guard)
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    const bool cand = ((fresh >> u) & 1u) && cc[u] != v.d;
+    const bool cand = ((fresh >> u) & 1u) && cc[u] != d;
     sg[u] = cand ? ld_state<LD>(a.sig + cc[u]) : 0;
-    one[u] = cand && want_size && cc[u] > v.d && ld_state<LD>(a.csize + cc[u]) == 1;
+    one[u] = cand && want_size && cc[u] > d && ld_state<LD>(a.csize + cc[u]) == 1;
   }
   __syncwarp();   // the sums are complete
   V kid = 0;
@@ -687,7 +747,7 @@ __device__ __forceinline__ void warp_vertex(const LMArgs<W>& a, const IterView& 
   for (int u = 0; u < U; ++u) {
     if (!((fresh >> u) & 1u)) continue;
     const V sum = vals[hs[u]];
-    if (cc[u] != v.d) {
+    if (cc[u] != d) {
       ++cands;
       const S g = Arith<WIDE>::score(v.M, (long long)sum, v.Ki, sg[u]);
       if (better(g, cc[u], bg, bc)) { bg = g; bc = cc[u]; bsz = one[u] ? 1 : 0; }
@@ -705,15 +765,16 @@ __device__ __forceinline__ void warp_vertex(const LMArgs<W>& a, const IterView& 
   }
   bool moved = false;
   if (lane == 0)
-    moved = commit_choice<W, WIDE, ASYNC, LD>(a, acc, v.i, v.d, v.Ki, sd, szd, bg, bc, kid, v.M, v.graph, nullptr,
+    moved = commit_choice<W, WIDE, ASYNC, LD>(a, acc, v.i, d, v.Ki, sd, szd, bg, bc, kid, v.M, v.graph, nullptr,
                                               want_size ? bsz : -1);
   moved = __shfl_sync(0xffffffffu, moved, 0);
-  if (moved && a.prune) mark_row<U>(a, iv, v.i, v.b, v.b + v.deg, lane, kWarp);
+  if (moved && a.prune && !(PULL && a.pull_mark)) mark_row<U>(a, iv, v.i, v.b, v.b + v.deg, lane, kWarp);
+  return true;
 }
 
 // U entries per lane cover the bucket's largest degree: the row is loaded and
 // gathered before any insert, so its memory latencies overlap.
-template <typename W, bool WIDE, bool ASYNC, int CAP, int U>
+template <typename W, bool WIDE, bool ASYNC, bool PULL, int CAP, int U>
 __global__ void __launch_bounds__(256, 4) lm_warp(LMArgs<W> a, const int32_t* __restrict__ list,
     const int64_t* __restrict__ ko) {
   const IterView iv = iter_view(a);
@@ -736,15 +797,19 @@ __global__ void __launch_bounds__(256, 4) lm_warp(LMArgs<W> a, const int32_t* __
   const int64_t stride = (int64_t)gridDim.x * WPB;
   for (int64_t w0 = (int64_t)blockIdx.x * WPB + wib; w0 < nverts; w0 += kWarp * stride) {
     VertexRow r;
-    unsigned live = vertex_window<W, (ASYNC ? 1 : 0)>(a, iv, verts, nverts, w0, stride, lane, r);
-    if ((live >> lane) & 1u) {
+    unsigned live = vertex_window<W, (ASYNC ? 1 : 0), PULL>(a, iv, verts, nverts, w0, stride, lane, r);
+    if (!(PULL && a.pull_check) && ((live >> lane) & 1u)) {
       tally.edges += (unsigned)r.deg;
       ++tally.visited;
     }
     for (; live; live &= live - 1) {
       const VertexRow v = window_row(a, r, __ffs(live) - 1);
-      warp_vertex<W, WIDE, ASYNC, CAP, U, (ASYNC ? 1 : 0), (CAP <= 64 && !WIDE)>(a, iv, acc, keys, vals, v, lane, ok,
-                                                                                   tally.cands);
+      const bool on = warp_vertex<W, WIDE, ASYNC, CAP, U, (ASYNC ? 1 : 0), (CAP <= 64 && !WIDE), PULL>(
+          a, iv, acc, keys, vals, v, lane, ok, tally.cands);
+      if (PULL && a.pull_check && on && lane == 0) {
+        tally.edges += (unsigned)v.deg;
+        ++tally.visited;
+      }
       __syncwarp();
     }
   }
@@ -1266,7 +1331,7 @@ struct PendingMove {
 };
 
 // Commit and mark the pending moves of a block (all threads take part).
-template <typename W, bool ASYNC>
+template <typename W, bool ASYNC, bool PULL>
 __device__ __forceinline__ void flush_moves(const LMArgs<W>& a, const IterView& iv, const PendingMove* q, int n,
                                             int tid, int nthr) {
   for (int t = tid; t < n; t += nthr) {
@@ -1283,7 +1348,7 @@ __device__ __forceinline__ void flush_moves(const LMArgs<W>& a, const IterView& 
       a.moves[pos] = make_int2(m.i, m.c);
     }
   }
-  if (!a.prune) return;
+  if (!a.prune || (PULL && a.pull_mark)) return;
   if (nthr >= 512) {   // long rows: the whole block marks one after the other
     for (int t = 0; t < n; ++t) mark_row<8>(a, iv, q[t].i, q[t].b, q[t].e, tid, nthr);
   } else {             // one warp per move, the warps' moves in parallel
@@ -1329,7 +1394,7 @@ __device__ __forceinline__ bool decide_move(const LMArgs<W>& a, BlockAcc& acc, i
 // with the touched-slot list and its scan, 48% of the issue slots).  R-MAT of
 // 4.2M vertices, synchronous: 143.4 -> 117.8 ms a run with this kernel, its
 // 12288-degree instance in place of the hub chain and 4096-entry hub chunks.
-template <typename W, bool WIDE, bool ASYNC, int CAP, int THREADS, int U>
+template <typename W, bool WIDE, bool ASYNC, bool PULL, int CAP, int THREADS, int U>
 __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ? 2 : 1)
     lm_block(LMArgs<W> a, const int32_t* __restrict__ list, const int64_t* __restrict__ ko) {
   const IterView iv = iter_view(a);
@@ -1366,8 +1431,8 @@ __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ?
   for (int64_t w0 = blockIdx.x; w0 < nverts; w0 += (int64_t)kWarp * gridDim.x, wp ^= 1) {
     if (wid == 0) {
       VertexRow r;
-      const unsigned on = vertex_window<W, LD>(a, iv, verts, nverts, w0, gridDim.x, lane, r);
-      if ((on >> lane) & 1u) {
+      const unsigned on = vertex_window<W, LD, PULL>(a, iv, verts, nverts, w0, gridDim.x, lane, r);
+      if (!(PULL && a.pull_check) && ((on >> lane) & 1u)) {
         tally.edges += (unsigned)r.deg;
         ++tally.visited;
       }
@@ -1380,8 +1445,8 @@ __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ?
       long long sd = 0;
       int32_t szd = 0;
       if (wid == 0) {   // for the decision
-        sd = ld_state<LD>(a.sig + v.d);
-        szd = ld_state<LD>(a.csize + v.d);
+        sd = ld_state<LD>(a.sig + word_id<PULL>(v.d));
+        szd = ld_state<LD>(a.csize + word_id<PULL>(v.d));
       }
       // this warp's rounds that hold at least one entry (the rest skipped)
       const int rem = v.deg - wid * kWarp;
@@ -1389,20 +1454,40 @@ __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ?
       int32_t cc[U];
       int hs[U];
       unsigned fresh;
+      int32_t seen = 0;
       {
         V ww[U];
-        row_communities<U, LD>(a, v, (int)threadIdx.x, THREADS, nu, cc, ww);
+        seen = row_communities<U, LD, PULL>(a, v, (int)threadIdx.x, THREADS, nu, cc, ww);
         fresh = table_add_row<CAP, U, V>(keys, vals, cc, ww, nu, hs, &ok);
       }
-      __syncthreads();   // B1: table complete; warp 0 has finished the previous vertex
+      // B1: table complete; warp 0 has finished the previous vertex
+      if (PULL && a.pull_check) {
+        const bool on = __syncthreads_or(((seen | v.d) & moved_bit(iv.iter - 1)) != 0);
+        if (!on) {   // not active after all: the table is cleared and nothing else done
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if ((fresh >> u) & 1u) {
+              keys[hs[u]] = kEmpty;
+              vals[hs[u]] = 0;
+            }
+          __syncthreads();
+          continue;
+        }
+        if (threadIdx.x == 0) {
+          tally.edges += (unsigned)v.deg;
+          ++tally.visited;
+        }
+      } else {
+        __syncthreads();
+      }
       if (q_n >= QCAP) {   // uniform: q_n was last written before this barrier
-        flush_moves<W, ASYNC>(a, iv, queue, q_n, threadIdx.x, THREADS);
+        flush_moves<W, ASYNC, PULL>(a, iv, queue, q_n, threadIdx.x, THREADS);
         __syncthreads();
         if (threadIdx.x == 0) q_n = 0;
       }
       if (threadIdx.x == 0) s_kid[p ^ 1] = 0;   // the next vertex's copy
       const long long M = a.gid ? a.Mg[a.gid[v.i]] : a.M, Ki = v.Ki;
-      const int32_t d = v.d;
+      const int32_t d = word_id<PULL>(v.d);
       S bg = Arith<WIDE>::lowest();
       int32_t bc = -1;
 #pragma unroll
@@ -1444,7 +1529,7 @@ __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ?
   }
   tally.add(acc);
   __syncthreads();
-  flush_moves<W, ASYNC>(a, iv, queue, q_n, threadIdx.x, THREADS);
+  flush_moves<W, ASYNC, PULL>(a, iv, queue, q_n, threadIdx.x, THREADS);
   if (!ok) atomicOr(&acc.error, kErrProbe);
   __syncthreads();
   acc_flush(acc, a.ctr);
@@ -1470,7 +1555,7 @@ constexpr int kItemCache = 512;   // hub prefix entries a block copies to shared
 
 constexpr int kHubThreads = 512;
 
-template <typename W, bool WIDE, bool ASYNC>
+template <typename W, bool WIDE, bool ASYNC, bool PULL>
 __global__ void __launch_bounds__(kHubThreads) lm_hub_insert(LMArgs<W> a, const int32_t* __restrict__ hubs, int nhubs,
                                                              const int64_t* __restrict__ chunk_pre) {
   typedef typename TableVal<WIDE>::T V;
@@ -1486,7 +1571,7 @@ __global__ void __launch_bounds__(kHubThreads) lm_hub_insert(LMArgs<W> a, const 
   const int h = block_item<kItemCache>(chunk_pre, nhubs, blockIdx.x, s_pre);
   VertexRow v;
   v.i = hubs[h];
-  if (!is_active(a, iv, v.i)) return;   // uniform across the block
+  if (!is_active<PULL>(a, iv, v.i)) return;   // uniform across the block
   if (!graph_of(a, v.i, &v.M, &v.graph)) return;
   const int64_t q = (int64_t)blockIdx.x - (chunk_pre[h] - chunk_pre[0]);
   for (int t = threadIdx.x; t < CAP; t += kHubThreads) { skeys[t] = kEmpty; svals[t] = 0; }
@@ -1500,7 +1585,10 @@ __global__ void __launch_bounds__(kHubThreads) lm_hub_insert(LMArgs<W> a, const 
   int32_t cc[U];
   V ww[U];
   int hs[U];
-  row_communities<U, (ASYNC ? 1 : 0)>(a, v, (int)threadIdx.x, kHubThreads, U, cc, ww);
+  const int32_t seen = row_communities<U, (ASYNC ? 1 : 0), PULL>(a, v, (int)threadIdx.x, kHubThreads, U, cc, ww);
+  // a neighbour moved: the scan finds the hub active
+  if (PULL && a.pull_check && __any_sync(0xffffffffu, (seen & moved_bit(iv.iter - 1)) != 0) && (threadIdx.x & 31) == 0)
+    a.hmoved[h] = -(iv.iter + 1);
   const unsigned fresh = table_add_row<CAP, U, V>(skeys, svals, cc, ww, U, hs, &ok);
   __syncthreads();
   // the thread that claimed a slot adds its sum to the hub's table
@@ -1520,7 +1608,7 @@ __global__ void __launch_bounds__(kHubThreads) lm_hub_insert(LMArgs<W> a, const 
 // best; the block that finishes a hub's last chunk (a per-hub counter after a
 // fence) reduces the hub's chunk bests and commits the hub's move, so the
 // decision needs no launch of its own.  No block waits for another.
-template <typename W, bool WIDE, bool ASYNC>
+template <typename W, bool WIDE, bool ASYNC, bool PULL>
 __global__ void __launch_bounds__(256) lm_hub_scan(LMArgs<W> a, const int32_t* __restrict__ hubs, int nhubs) {
   const IterView iv = iter_view(a);
   if (iv.iter < 0) return;
@@ -1535,7 +1623,7 @@ __global__ void __launch_bounds__(256) lm_hub_scan(LMArgs<W> a, const int32_t* _
   __shared__ int64_t s_pre[kItemCache + 1];
   const int h = block_item<kItemCache>(a.spre, nhubs, blockIdx.x, s_pre);
   const int32_t i = hubs[h];
-  if (!is_active(a, iv, i)) return;   // uniform across the block
+  if (!is_active<PULL>(a, iv, i)) return;   // uniform across the block
   long long M;
   int graph;
   if (!graph_of(a, i, &M, &graph)) return;
@@ -1544,7 +1632,8 @@ __global__ void __launch_bounds__(256) lm_hub_scan(LMArgs<W> a, const int32_t* _
   const int64_t b = a.off[i], e = a.off[i + 1];
   const int64_t cap = 2 * (e - b);
   const int64_t base = a.hbase[h] - a.hbase[0];
-  const int32_t d = a.memb[i];
+  const int32_t dw = a.memb[i], d = word_id<PULL>(dw);
+  const bool on = !(PULL && a.pull_check) || (dw & moved_bit(iv.iter - 1)) || a.hmoved[h] == -(iv.iter + 1);
   const long long Ki = a.K[i];
   const int64_t t0 = q * kSlotChunk, t1 = min(cap, t0 + kSlotChunk);
   S bg = Arith<WIDE>::lowest();
@@ -1567,7 +1656,8 @@ __global__ void __launch_bounds__(256) lm_hub_scan(LMArgs<W> a, const int32_t* _
     for (int u = 0; u < U; ++u) {
       if (cs[u] == kEmpty) continue;
       const int64_t t = y + u * 256 + threadIdx.x;
-      if (cs[u] != d) {
+      if (PULL && !on) {   // inactive after all: only cleared
+      } else if (cs[u] != d) {
         ++ncand;
         S g = Arith<WIDE>::score(M, (long long)vs[u], Ki, sg[u]);
         if (better(g, cs[u], bg, bc)) { bg = g; bc = cs[u]; }
@@ -1611,14 +1701,16 @@ __global__ void __launch_bounds__(256) lm_hub_scan(LMArgs<W> a, const int32_t* _
     }
     warp_argmax(hg, hc);
     if (lane == 0) {
-      atomicAdd(&acc.edges, (unsigned long long)(e - b));
-      atomicAdd(&acc.visited, 1ull);
-      const bool moved = commit_choice<W, WIDE, ASYNC>(a, acc, i, d, Ki, ld_sig<ASYNC>(a.sig + d),
+      if (on) {
+        atomicAdd(&acc.edges, (unsigned long long)(e - b));
+        atomicAdd(&acc.visited, 1ull);
+      }
+      const bool moved = on && commit_choice<W, WIDE, ASYNC>(a, acc, i, d, Ki, ld_sig<ASYNC>(a.sig + d),
                                                        ld_size<ASYNC>(a.csize + d), hg, hc, __ldcg(a.hkid + h), M,
                                                        graph);
       a.hkid[h] = 0;
       a.hdone[h] = 0;
-      if (moved && a.prune) a.hmoved[h] = iv.iter + 1;   // lm_hub_mark marks its neighbours
+      if (moved && a.prune && !(PULL && a.pull_mark)) a.hmoved[h] = iv.iter + 1;   // lm_hub_mark marks its neighbours
     }
   }
   __syncthreads();
@@ -1651,18 +1743,33 @@ __global__ void __launch_bounds__(256) lm_hub_mark(LMArgs<W> a, const int32_t* _
 template <typename W>
 __global__ void __launch_bounds__(256) lm_commit(LMArgs<W> a) {
   const unsigned long long n = a.ctr->nmoves_list[a.odd];
+  const bool pull = a.pull_check || a.pull_mark;
+  const int32_t flag = a.pull_mark ? moved_bit(*a.d_iter) : 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr->nmoves_list[a.odd ^ 1] = 0;
   for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < n;
        t += (unsigned long long)gridDim.x * blockDim.x) {
     int2 mv = a.moves[t];
-    int32_t i = mv.x, c = mv.y, d = a.memb[i];
+    int32_t i = mv.x, c = mv.y, d = pull ? a.memb[i] & kIdMask : a.memb[i];
     long long Ki = a.K[i];
-    a.memb[i] = c;
+    a.memb[i] = c | flag;
     atomicAdd((unsigned long long*)(a.sig + d), (unsigned long long)(-Ki));
     atomicAdd((unsigned long long*)(a.sig + c), (unsigned long long)Ki);
     atomicSub(a.csize + d, 1);
     atomicAdd(a.csize + c, 1);
   }
+}
+
+// memb &= keep (flags that have been read; both at the end of a phase).
+__global__ void clear_flags_k(int32_t* __restrict__ memb, int64_t n, int32_t keep) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t w = memb[i];
+    if ((w & keep) != w) memb[i] = w & keep;
+  }
+}
+void lm_clear_flags(int32_t* memb, int64_t n, int iter, cudaStream_t s) {
+  const int32_t keep = iter < 0 ? kIdMask : (iter & 1) ? 0x7fffffff : (int32_t)0xbfffffff;
+  const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16));
+  (count_launch(), clear_flags_k<<<blocks, 256, 0, s>>>(memb, n, keep));
 }
 
 // The end of an iteration of one graph, on the device: its counters go to
@@ -1701,42 +1808,42 @@ int grid_for(K kernel, int threads, size_t smem, int64_t work_blocks) {
   return g < 1 ? 1 : g;
 }
 
-template <typename W, bool WIDE, bool ASYNC, int CAP, int THREADS, int U>
+template <typename W, bool WIDE, bool ASYNC, bool PULL, int CAP, int THREADS, int U>
 void launch_block_t(const LMArgs<W>& a, const int32_t* list, const int64_t* ko, int64_t nverts, cudaStream_t s) {
   const size_t smem = (size_t)CAP * (sizeof(typename TableVal<WIDE>::T) + 4);
-  auto k = lm_block<W, WIDE, ASYNC, CAP, THREADS, U>;
+  auto k = lm_block<W, WIDE, ASYNC, PULL, CAP, THREADS, U>;
   static std::atomic<unsigned long long> attr{0};
   smem_limit_once(attr, k, smem);
   (count_launch(), k<<<grid_for(k, THREADS, smem, nverts), THREADS, smem, s>>>(a, list, ko));
 }
 
-template <typename W, bool WIDE, bool ASYNC>
+template <typename W, bool WIDE, bool ASYNC, bool PULL>
 void launch_bucket_t(const LMArgs<W>& a, int bucket, const int32_t* list, const int64_t* ko, int64_t nverts, cudaStream_t s) {
   if (nverts <= 0) return;
   switch (bucket) {
     case 0: {
-      auto k = lm_thread<W, WIDE, ASYNC>;
+      auto k = lm_thread<W, WIDE, ASYNC, PULL>;
       (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 255) / 256), 256, 0, s>>>(a, list, ko));
       break;
     }
     case 1: {
       if (!WIDE) {   // narrow sums: a lane per vertex, its row sorted in registers
-        auto k = lm_thread_sorted<W, ASYNC, 32>;
+        auto k = lm_thread_sorted<W, ASYNC, PULL, 32>;
         (count_launch(), k<<<grid_for(k, 128, 0, (nverts + 127) / 128), 128, 0, s>>>(a, list, ko));
       } else {
-        auto k = lm_warp<W, WIDE, ASYNC, 64, 1>;
+        auto k = lm_warp<W, WIDE, ASYNC, PULL, 64, 1>;
         (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 7) / 8), 256, 0, s>>>(a, list, ko));
       }
       break;
     }
     case 2: {
-      auto k = lm_warp<W, WIDE, ASYNC, 256, 4>;
+      auto k = lm_warp<W, WIDE, ASYNC, PULL, 256, 4>;
       (count_launch(), k<<<grid_for(k, 256, 0, (nverts + 7) / 8), 256, 0, s>>>(a, list, ko));
       break;
     }
-    case 3: launch_block_t<W, WIDE, ASYNC, 2048, 128, 8>(a, list, ko, nverts, s); break;
-    case 4: launch_block_t<W, WIDE, ASYNC, 8192, 512, 8>(a, list, ko, nverts, s); break;
-    case 5: launch_block_t<W, WIDE, ASYNC, 18432, 1024, 12>(a, list, ko, nverts, s); break;
+    case 3: launch_block_t<W, WIDE, ASYNC, PULL, 2048, 128, 8>(a, list, ko, nverts, s); break;
+    case 4: launch_block_t<W, WIDE, ASYNC, PULL, 8192, 512, 8>(a, list, ko, nverts, s); break;
+    case 5: launch_block_t<W, WIDE, ASYNC, PULL, 18432, 1024, 12>(a, list, ko, nverts, s); break;
     default: break;
   }
 }
@@ -1746,23 +1853,27 @@ void launch_bucket_t(const LMArgs<W>& a, int bucket, const int32_t* list, const 
 template <typename W>
 void lm_launch_bucket(const LMArgs<W>& a, bool wide, bool async, int bucket, const int32_t* list, const int64_t* ko,
                       int64_t nverts, cudaStream_t s) {
+  const bool pull = a.pull_check || a.pull_mark;   // synchronous only
   if (wide) {
-    if (async) launch_bucket_t<W, true, true>(a, bucket, list, ko, nverts, s);
-    else launch_bucket_t<W, true, false>(a, bucket, list, ko, nverts, s);
+    if (async) launch_bucket_t<W, true, true, false>(a, bucket, list, ko, nverts, s);
+    else if (pull) launch_bucket_t<W, true, false, true>(a, bucket, list, ko, nverts, s);
+    else launch_bucket_t<W, true, false, false>(a, bucket, list, ko, nverts, s);
   } else {
-    if (async) launch_bucket_t<W, false, true>(a, bucket, list, ko, nverts, s);
-    else launch_bucket_t<W, false, false>(a, bucket, list, ko, nverts, s);
+    if (async) launch_bucket_t<W, false, true, false>(a, bucket, list, ko, nverts, s);
+    else if (pull) launch_bucket_t<W, false, false, true>(a, bucket, list, ko, nverts, s);
+    else launch_bucket_t<W, false, false, false>(a, bucket, list, ko, nverts, s);
   }
 }
 
-template <typename W, bool WIDE, bool ASYNC>
-static void launch_hub_insert(const LMArgs<W>& a, const int32_t* hubs, int nhubs, const int64_t* chunk_pre,
-                              int64_t nchunks, cudaStream_t s) {
+template <typename W, bool WIDE, bool ASYNC, bool PULL>
+static void launch_hubs_t(const LMArgs<W>& a, const int32_t* hubs, int nhubs, const int64_t* chunk_pre,
+                          int64_t nchunks, int64_t nslotchunks, cudaStream_t s) {
   const size_t smem = (size_t)(2 * kHubChunk) * (sizeof(typename TableVal<WIDE>::T) + 4);
-  auto k = lm_hub_insert<W, WIDE, ASYNC>;
+  auto k = lm_hub_insert<W, WIDE, ASYNC, PULL>;
   static std::atomic<unsigned long long> attr{0};
   smem_limit_once(attr, k, smem);
   (count_launch(), k<<<(unsigned)nchunks, kHubThreads, smem, s>>>(a, hubs, nhubs, chunk_pre));
+  (count_launch(), lm_hub_scan<W, WIDE, ASYNC, PULL><<<(unsigned)nslotchunks, 256, 0, s>>>(a, hubs, nhubs));
 }
 
 template <typename W>
@@ -1770,19 +1881,15 @@ void lm_launch_hubs(const LMArgs<W>& a, bool wide, bool async, const int32_t* hu
                     const int64_t* chunk_pre, int64_t nchunks, const int64_t* spre, int64_t nslotchunks,
                     cudaStream_t s) {
   if (nhubs <= 0 || nchunks <= 0) return;
+  const bool pull = a.pull_check || a.pull_mark;   // synchronous only
   if (wide) {
-    if (async) launch_hub_insert<W, true, true>(a, hubs, nhubs, chunk_pre, nchunks, s);
-    else launch_hub_insert<W, true, false>(a, hubs, nhubs, chunk_pre, nchunks, s);
+    if (async) launch_hubs_t<W, true, true, false>(a, hubs, nhubs, chunk_pre, nchunks, nslotchunks, s);
+    else if (pull) launch_hubs_t<W, true, false, true>(a, hubs, nhubs, chunk_pre, nchunks, nslotchunks, s);
+    else launch_hubs_t<W, true, false, false>(a, hubs, nhubs, chunk_pre, nchunks, nslotchunks, s);
   } else {
-    if (async) launch_hub_insert<W, false, true>(a, hubs, nhubs, chunk_pre, nchunks, s);
-    else launch_hub_insert<W, false, false>(a, hubs, nhubs, chunk_pre, nchunks, s);
-  }
-  if (wide) {
-    if (async) (count_launch(), lm_hub_scan<W, true, true><<<(unsigned)nslotchunks, 256, 0, s>>>(a, hubs, nhubs));
-    else (count_launch(), lm_hub_scan<W, true, false><<<(unsigned)nslotchunks, 256, 0, s>>>(a, hubs, nhubs));
-  } else {
-    if (async) (count_launch(), lm_hub_scan<W, false, true><<<(unsigned)nslotchunks, 256, 0, s>>>(a, hubs, nhubs));
-    else (count_launch(), lm_hub_scan<W, false, false><<<(unsigned)nslotchunks, 256, 0, s>>>(a, hubs, nhubs));
+    if (async) launch_hubs_t<W, false, true, false>(a, hubs, nhubs, chunk_pre, nchunks, nslotchunks, s);
+    else if (pull) launch_hubs_t<W, false, false, true>(a, hubs, nhubs, chunk_pre, nchunks, nslotchunks, s);
+    else launch_hubs_t<W, false, false, false>(a, hubs, nhubs, chunk_pre, nchunks, nslotchunks, s);
   }
 }
 
@@ -1827,7 +1934,7 @@ void lm_launch_small(const LMArgs<W>& a, const SmallArgs& sa, cudaStream_t s) {
 template <typename W>
 void lm_launch_hub_mark(const LMArgs<W>& a, const int32_t* hubs, int nhubs, const int64_t* chunk_pre, int64_t nchunks,
                         cudaStream_t s) {
-  if (nhubs <= 0 || nchunks <= 0 || !a.prune) return;
+  if (nhubs <= 0 || nchunks <= 0 || !a.prune || a.pull_mark) return;
   (count_launch(), lm_hub_mark<W><<<(unsigned)nchunks, 256, 0, s>>>(a, hubs, nhubs, chunk_pre));
 }
 
