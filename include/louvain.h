@@ -87,7 +87,10 @@ typedef struct {
                                  louvain_get_coarse (copies them to host memory) */
   int32_t cuda_graphs;        /* 1: from the third iteration of a pass, replay that pass's iteration
                                  as one captured CUDA graph instead of individual launches (default 0:
-                                 measured slower on the benchmark graphs) */
+                                 measured slower on the benchmark graphs).  Either way the engine
+                                 captures the iterations that last less than their launches: small
+                                 passes of several classes, and synchronous passes of at most 8M
+                                 entries from their fifth iteration */
   int32_t reclass;            /* asynchronous mode with P > 1: 0 = classes id mod P; 1 = each
                                  iteration draws the classes anew, class = hash(id, pass, iteration)
                                  mod P (breaks the repeated same-class swaps of structured ids such
@@ -220,8 +223,9 @@ int louvain_batch_get_iterations(louvain_ctx *ctx, int64_t g, int64_t *out, int6
  * largest degrees handled by, in order, a thread per vertex (register table,
  * at most 8), a warp with a 64-slot table (at most 32), a warp with a 256-slot
  * table (at most 128), a block with a 2048-slot table (at most 1024) and a
- * block with an 8192-slot table (at most 4096); larger degrees go to the hub
- * path (global tables).  They must increase.  Lowering one moves vertices to
+ * block with an 8192-slot table (at most 4096); degrees of 4097 to
+ * 12288 (asynchronous mode: 6144) go to a block with an 18432-slot table, other
+ * degrees above the thresholds to the hub path (global tables).  They must increase.  Lowering one moves vertices to
  * a wider mapping whose table is emptier.  NULL restores the defaults (the
  * maxima).  The mapping never changes results: only which kernel computes
  * them.  Errors: INVALID_ARG. */

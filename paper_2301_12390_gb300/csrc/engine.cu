@@ -60,7 +60,8 @@ constexpr int64_t kEdgeListRatio = 4;
 // Pruning by pull while an iteration visits at least this share of a pass's
 // vertices with edges (the others gather their rows for nothing).  A 4096 x 4096
 // road grid: 34.6 ms a run at 0.75 and 0.5, 35.4 at 0.25, 36.1 always pushed;
-// R-MAT visits nearly all, any share gives 100.5 (116.8 pushed).
+// R-MAT visits nearly all, any share gives 100.5 (116.8 pushed); a 2048 x 2048
+// grid in colour classes 14.0 (14.25).
 constexpr double kPullFraction = 0.75;
 // A synchronous pass of up to this many entries is shorter on the GPU than its
 // launches on the host.
@@ -634,8 +635,9 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // |K_i Sigma_c| stay at or below 2^61, a gain at or below 2^62 and every
   // K_{i->c} below 2^31.  ko[nkeys + 1] receives the buckets that do not (found
   // by the pass's first classification; degrees do not change within a pass).
-  // Road grid of 16.8M vertices (M = 3e9): degrees 1-8 913 -> 560 us an
-  // iteration.  Only vertices holding more than 2^61 / M^2 of all weight stay wide.
+  // Road grid of 16.8M vertices (M = 3e9): 54.2 -> 48.2 ms a run, R-MAT of 1M
+  // vertices with weights to 10,000: 13.3 -> 11.8.  Only vertices holding more
+  // than 2^61 / M^2 of all weight stay wide.
   const long long klimit = wide ? (long long)((1ull << 61) / (unsigned long long)c->M) : 0;
   unsigned long long wmask = 0;
   auto wide_bucket = [&](int b) { return ((wmask >> b) & 1ull) != 0; };
@@ -742,7 +744,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // Pruning by pull (local_move.cu): iteration k's moves set flags when the last
   // iteration known visited nearly every vertex.  A captured graph's launches are
   // fixed, so its iterations neither read flags nor set them.
-  const bool may_pull = c->opt.prune && !async && !multi && !colour && P == 1 && !small_pass &&
+  const bool may_pull = c->opt.prune && !async && !multi && !small_pass &&
                         c->opt.stop_rule == 0 && g.n < (1ll << 30) - 1;
   bool pull_now = false, pulled = false;
   int cur_iter = 0;

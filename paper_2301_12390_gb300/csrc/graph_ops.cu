@@ -335,8 +335,9 @@ void stable_partition(const int32_t* key, int64_t n, int nkeys, int32_t* out, in
 // sorted stably: the first launch counts the keys per block in shared memory
 // and adds them up with atomics, its last block scans the totals; the second
 // ranks a tile's vertices per key in shared memory and reserves the tile's
-// range of each key with one atomic.  A redraw of 4.2M vertices into 8 classes
-// took 80 us in six launches (keys, counts, three scan steps, stable scatter).
+// range of each key with one atomic, instead of six launches (keys, counts,
+// three scan steps, stable scatter) with a host read before the classes' first
+// one: asynchronous road grid of 4.2M vertices, eight tolerances, 89 -> 79 ms.
 // Vertices without a key (no entries; inactive, with `active`; of a graph that
 // does not iterate, with g_on) are counted as the last key and not listed.
 // Lists that serve a whole pass are worth the stable partition instead

@@ -195,7 +195,7 @@ __device__ __forceinline__ IterView iter_view(const LMArgs<W>& a) {
   return IterView{it, a.stamps[it & 1], a.stamps[(it + 1) & 1]};
 }
 
-// Pruning by pull, while nearly every vertex is active (synchronous, one class).
+// Pruning by pull, while nearly every vertex is active (synchronous).
 // A vertex is active when it or a neighbour moved in the iteration before.
 // Pushed, every mover rereads its row and stores a stamp per neighbour, twenty
 // stores for one vertex and most of them to the same hubs (R-MAT of 4.2M
@@ -1758,14 +1758,16 @@ template <typename W>
 __global__ void __launch_bounds__(256) lm_commit(LMArgs<W> a) {
   const unsigned long long n = a.ctr->nmoves_list[a.odd];
   const bool pull = a.pull_check || a.pull_mark;
-  const int32_t flag = a.pull_mark ? moved_bit(*a.d_iter) : 0;
+  // the flag of this iteration's moves, and the last one's, which later classes read
+  const int it = *a.d_iter;
+  const int32_t flag = a.pull_mark ? moved_bit(it) : 0, kept = a.pull_check ? moved_bit(it - 1) : 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr->nmoves_list[a.odd ^ 1] = 0;
   for (unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; t < n;
        t += (unsigned long long)gridDim.x * blockDim.x) {
     int2 mv = a.moves[t];
-    int32_t i = mv.x, c = mv.y, d = pull ? a.memb[i] & kIdMask : a.memb[i];
-    long long Ki = a.K[i];
-    a.memb[i] = c | flag;
+    const int32_t i = mv.x, c = mv.y, w = a.memb[i], d = pull ? w & kIdMask : w;
+    const long long Ki = a.K[i];
+    a.memb[i] = c | flag | (w & kept);
     atomicAdd((unsigned long long*)(a.sig + d), (unsigned long long)(-Ki));
     atomicAdd((unsigned long long*)(a.sig + c), (unsigned long long)Ki);
     atomicSub(a.csize + d, 1);

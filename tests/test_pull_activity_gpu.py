@@ -37,13 +37,14 @@ class _Stars:
 DEGREES = [[1, 4, 5, 8, 9, 32, 33], [64, 128, 129, 1024, 1025], [4096, 4097, 12288, 12289, 20000]]
 
 
+@pytest.mark.parametrize("classes", [{}, {"subrounds": 4}, {"colour_classes": 1}], ids=["one", "four", "colour"])
 @pytest.mark.parametrize("wmax", [3, 1 << 29])
 @pytest.mark.parametrize("degrees", DEGREES, ids=["-%d" % max(d) for d in DEGREES])
-def test_flagged_and_stamped_iterations_visit_the_same_vertices(degrees, wmax):
+def test_flagged_and_stamped_iterations_visit_the_same_vertices(degrees, wmax, classes):
     g = _Stars(degrees, 30000, wmax, 5)
-    assert_sync_parity(g, prune=1, max_passes=1, max_iterations=8)
+    assert_sync_parity(g, prune=1, max_passes=1, max_iterations=8, **classes)
     # stop rule 1 keeps the stamps, and its modularity rises in the first four iterations
-    opt = dict(mode=0, prune=1, max_passes=1, max_iterations=4, tolerance=0.0)
+    opt = dict(mode=0, prune=1, max_passes=1, max_iterations=4, tolerance=0.0, **classes)
     got, ref = engine_run(g, **opt), engine_run(g, stop_rule=1, **opt)
     assert len(ref["iters"]) == 4 and ref["iters"] == got["iters"]
     for f in ("lm_vertices", "lm_edges", "lm_bytes"):
