@@ -35,18 +35,13 @@ __device__ __forceinline__ unsigned lanemask_lt_lm() {
   return m;
 }
 
-// Synchronous launches never write memberships, totals or sizes, so they
-// read them through the read-only path; asynchronous launches use plain
-// loads, which may return a value that another vertex has since changed —
-// exactly the staleness the asynchronous variant allows.
 // Loads of memberships, community totals and sizes.  LD 0: read-only path
 // (nothing writes them while the kernel runs: a synchronous class); 1: plain
-// (asynchronous in-place updates, any recent value will do); 2: L2 only (the
-// kernel itself updates them between its classes and must see the result).
+// (asynchronous in-place updates, any recent value will do: exactly the
+// staleness that mode allows).
 template <int LD, typename T>
 __device__ __forceinline__ T ld_state(const T* p) {
   if (LD == 0) return __ldg(p);
-  if (LD == 2) return __ldcg(p);
   return *p;
 }
 template <bool ASYNC>
@@ -236,7 +231,7 @@ struct VertexRow {
 // nothing more.  Returns the lanes whose vertex is visited in this iteration.
 // A vertex's own community only changes by its own commit, so it may be read
 // ahead; its community's total and size are read when its row is.
-template <typename W, int LD, bool PULL = false>
+template <typename W, bool PULL = false>
 __device__ __forceinline__ unsigned vertex_window(const LMArgs<W>& a, const IterView& iv,
                                                   const int32_t* __restrict__ verts, int64_t nverts, int64_t first,
                                                   int64_t stride, int lane, VertexRow& r) {
@@ -249,7 +244,7 @@ __device__ __forceinline__ unsigned vertex_window(const LMArgs<W>& a, const Iter
       on = true;
       r.b = a.off[r.i];
       r.deg = (int)(a.off[r.i + 1] - r.b);
-      r.d = ld_state<LD == 2 ? 2 : 1>(a.memb + r.i);
+      r.d = ld_state<1>(a.memb + r.i);
       r.Ki = a.K[r.i];
     }
   }
@@ -811,7 +806,7 @@ __global__ void __launch_bounds__(256, 4) lm_warp(LMArgs<W> a, const int32_t* __
   const int64_t stride = (int64_t)gridDim.x * WPB;
   for (int64_t w0 = (int64_t)blockIdx.x * WPB + wib; w0 < nverts; w0 += kWarp * stride) {
     VertexRow r;
-    unsigned live = vertex_window<W, (ASYNC ? 1 : 0), PULL>(a, iv, verts, nverts, w0, stride, lane, r);
+    unsigned live = vertex_window<W, PULL>(a, iv, verts, nverts, w0, stride, lane, r);
     if (!(PULL && a.pull_check) && ((live >> lane) & 1u)) {
       tally.edges += (unsigned)r.deg;
       ++tally.visited;
@@ -874,7 +869,7 @@ __global__ void __launch_bounds__(256, 3) lm_class(LMArgs<W> a, const int32_t* _
     const int64_t u = t - m0;
     const int64_t idx = u < n1 ? r1 + u : r2 + (u - n1);
     VertexRow r;
-    if (!vertex_window<W, (ASYNC ? 1 : 0)>(a, iv, list + idx, 1, 0, 1, lane, r)) continue;
+    if (!vertex_window<W>(a, iv, list + idx, 1, 0, 1, lane, r)) continue;
     if (lane == 0) {
       tally.edges += (unsigned)r.deg;
       ++tally.visited;
@@ -1445,7 +1440,7 @@ __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ?
   for (int64_t w0 = blockIdx.x; w0 < nverts; w0 += (int64_t)kWarp * gridDim.x, wp ^= 1) {
     if (wid == 0) {
       VertexRow r;
-      const unsigned on = vertex_window<W, LD, PULL>(a, iv, verts, nverts, w0, gridDim.x, lane, r);
+      const unsigned on = vertex_window<W, PULL>(a, iv, verts, nverts, w0, gridDim.x, lane, r);
       if (!(PULL && a.pull_check) && ((on >> lane) & 1u)) {
         tally.edges += (unsigned)r.deg;
         ++tally.visited;
