@@ -135,9 +135,10 @@ constexpr int64_t kSmallVerts = 8192, kTinyVerts = 1024;   // vertices whose sta
 // With this line, against launches only: 512 planted partitions 43.8 -> 22.4 ms,
 // one of 8,192 vertices 1.69 -> 1.48 (136,000 entries: its later passes), the
 // later passes of an R-MAT of 75,879 vertices 5.9 -> 5.5 a run.
+constexpr int64_t kSmallEntries = 131072;
 __host__ __device__ inline int64_t small_entries(int classes) {
   const int64_t e = 16384 + 4096 * (int64_t)classes;
-  return e < 131072 ? e : 131072;
+  return e < kSmallEntries ? e : kSmallEntries;
 }
 struct SmallArgs {
   const int64_t* vo;

@@ -904,6 +904,9 @@ __global__ void __launch_bounds__(256, 3) lm_class(LMArgs<W> a, const int32_t* _
 // degrees up to 128, and the block together takes larger ones, its warps'
 // values forming one such array.
 
+// Vertices of degree above 128 that a graph within the entry limit can hold.
+constexpr int kSmallLong = (int)(kSmallEntries / 129) + 1;
+
 // One vertex's best candidate so far.
 struct SmallBest {
   long long g;
@@ -960,7 +963,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
   extern __shared__ unsigned long long sdyn[];
   const SG s(sdyn);
   __shared__ int s_start[66], s_fill[64];
-  __shared__ int s_stop, s_moved;
+  __shared__ int s_stop, s_moved, s_nlong;
+  __shared__ uint16_t s_long[SG::kDense ? 1 : kSmallLong];
   __shared__ unsigned s_kid;
   __shared__ long long r_g[NW];
   __shared__ int32_t r_c[NW];
@@ -998,6 +1002,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
     s.vals[t] = 0;
   }
   for (int t = tid; t < 2 * NMAX / 32; t += THREADS) s.act[t] = 0;
+  if (tid == 0) s_nlong = 0;
   const double MM = u128_to_double((u128)M * (u128)M);
   int32_t* keys = s.keys + wid * SG::CAP;
   unsigned* vals = s.vals + wid * SG::CAP;
@@ -1039,7 +1044,6 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
     for (int ch = 0; ch < P; ++ch) {
       const int l0 = s_start[ch], m = s_start[ch + 1] - l0;
       if (m == 0) continue;   // uniform
-      bool left = false;
       // warp w takes entries w, w + NW, ...: 32 of them at a time, a lane each
       for (int j0 = wid; j0 < m; j0 += kWarp * NW) {
         const int j = j0 + lane * NW;
@@ -1109,7 +1113,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
           const int64_t bb = __shfl_sync(0xffffffffu, b, src);
           const long long kk = __shfl_sync(0xffffffffu, Ki, src);
           if (dg > 128 && !SG::kDense) {   // for the block, after the class's other vertices
-            left = true;
+            if (lane == 0) s_long[atomicAdd(&s_nlong, 1)] = (uint16_t)vv;
             continue;
           }
           int cl[4], cc[4];
@@ -1200,14 +1204,18 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
           __syncwarp();
         }
       }
-      const bool nbig = __syncthreads_or(left);
-      if (nbig) {   // uniform: vertices of degree above 128, the block together
+      __syncthreads();
+      // The vertices of degree above 128, queued above, the block together on each.
+      // (Finding them by walking the class again cost all 32 warps a list entry
+      // and two offsets a vertex: 3,300 pairs beside one vertex of degree 200,
+      // one class, 1.07 ms an iteration; with the queue 0.02.)
+      const int nlong = s_nlong;
+      if (nlong) {   // uniform
         unsigned* dense = s.vals;
-        for (int j = 0; j < m; ++j) {
-          const int v = s.list[l0 + j];
+        for (int j = 0; j < nlong; ++j) {
+          const int v = s_long[j];
           const int64_t b = off[v];
           const int deg = (int)(off[v + 1] - b);
-          if (deg <= 128 || (a.prune && it > 0 && !((cur[v >> 5] >> (v & 31)) & 1u))) continue;   // uniform
           const int d = s.memb[v];
           const long long Ki = a.K[v0 + v];
           if (tid == 0) s_kid = 0;
@@ -1254,6 +1262,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
           }
         }
         __syncthreads();
+        if (tid == 0) s_nlong = 0;   // for the next class, after the barrier that ends this one
       }
       // the class's moves
       for (int j = tid; j < m; j += THREADS) {

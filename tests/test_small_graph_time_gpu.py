@@ -1,0 +1,42 @@
+"""Time of the one-block local-moving phase on graphs whose shape could make it slow."""
+import numpy as np
+import pytest
+
+from engine_util import assert_sync_parity
+from paper_2301_12390_gb300 import SYNC, Louvain
+from test_degree_edges_gpu import _Csr
+
+pytestmark = pytest.mark.gpu
+
+
+def _pairs(n, links, leaves):
+    """`links` disjoint pairs among n vertices; with leaves, vertex 0 also joined to that many of the others."""
+    u, v = 1 + 2 * np.arange(links), 2 + 2 * np.arange(links)
+    if leaves:
+        leaf = 1 + np.random.default_rng(1).choice(2 * links, leaves, replace=False)
+        u, v = np.concatenate([u, np.zeros(leaves, np.int64)]), np.concatenate([v, leaf])
+    return _Csr(n, u, v, np.ones(len(u), np.int64))
+
+
+def _star(leaves):
+    return _Csr(leaves + 1, np.zeros(leaves, np.int64), 1 + np.arange(leaves), np.ones(leaves, np.int64))
+
+
+def _iteration_ms(g, runs=7, **opt):
+    """Local-moving time of an iteration of pass 0, the shortest of several runs."""
+    best = float("inf")
+    with Louvain(device=0, mode=SYNC, prune=1, max_passes=1, **opt) as lv:
+        lv.load_csr(g.off, g.col, g.w)
+        for _ in range(runs):
+            lv.run()
+            p = lv.passes()[0]
+            best = min(best, p.lm_ms / p.iterations)
+    return best
+
+
+def test_a_long_row_does_not_slow_the_other_vertices():
+    # the same 3,300 pairs with and without one vertex of degree 200: searching the class for it by the
+    # whole block took ten times the rest of the iteration
+    plain, hub = _pairs(7000, 3300, 0), _pairs(7000, 3300, 200)
+    assert_sync_parity(hub, prune=1)
+    assert _iteration_ms(hub) < 3 * _iteration_ms(plain)
