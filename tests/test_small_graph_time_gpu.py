@@ -40,3 +40,24 @@ def test_a_long_row_does_not_slow_the_other_vertices():
     plain, hub = _pairs(7000, 3300, 0), _pairs(7000, 3300, 200)
     assert_sync_parity(hub, prune=1)
     assert _iteration_ms(hub) < 3 * _iteration_ms(plain)
+
+
+def test_moves_into_one_community_do_not_queue_up():
+    # the leaves of a star all leave and join the same communities: four times the time of as many pairs
+    # when each of their updates waits for the others'
+    star, plain = _star(3400), _pairs(7000, 3300, 0)
+    assert_sync_parity(star, prune=1)
+    assert _iteration_ms(star) < 2 * _iteration_ms(plain)
+
+
+@pytest.mark.parametrize("classes", [1, 3])
+def test_totals_carry_across_32_bits(classes):
+    # two communities whose totals pass 2^32 while every degree still suits 64-bit gains
+    rng = np.random.default_rng(2)
+    u, v = np.triu_indices(64, 1)
+    keep = rng.random(len(u)) < np.where(u // 32 == v // 32, 0.7, 0.03)
+    g = _Csr(64, u[keep], v[keep], rng.integers(5_000_000, 8_000_000, int(keep.sum())))
+    K = np.add.reduceat(g.w.astype(np.int64), g.off[:-1])
+    assert int(K.max()) <= (1 << 61) // int(K.sum())
+    _, ref = assert_sync_parity(g, prune=1, subrounds=classes)
+    assert np.bincount(ref.top, weights=K).min() > 1 << 32
