@@ -130,15 +130,31 @@ constexpr int kSmallIters = 32;   // a larger max_iterations takes the launches
 constexpr int kSmallRec = 4 + 3 * kSmallIters;
 constexpr unsigned long long kSmallNot = ~0ull, kSmallErr = ~1ull;
 constexpr int64_t kSmallVerts = 8192, kTinyVerts = 1024;   // vertices whose state fits a block's shared memory
-// Entries up to which one block is taken instead of the launches of an
-// iteration, which cost 5-7 us a class whatever the size: more with more classes.
-// With this line, against launches only: 512 planted partitions 43.8 -> 22.4 ms,
-// one of 8,192 vertices 1.69 -> 1.48 (136,000 entries: its later passes), the
-// later passes of an R-MAT of 75,879 vertices 5.9 -> 5.5 a run.
-constexpr int64_t kSmallEntries = 131072;
-__host__ __device__ inline int64_t small_entries(int classes) {
-  const int64_t e = 16384 + 4096 * (int64_t)classes;
-  return e < kSmallEntries ? e : kSmallEntries;
+constexpr int64_t kSmallEntries = 131072;   // entries of a graph that one block takes at most
+// Whether one block pays.  Its iteration costs about 10 us, 3-4 a class, one for
+// each round of its warps over the vertices of more than 8 entries (at most
+// min(n, e / 9), a warp each) and the long rows that the whole block takes one by
+// one (e / 1000 allows for them; of a tiny graph a warp takes them too).  The
+// launches' iteration costs about 13 us and 7 a class (15 with a long row), and a
+// phase 100 to set up, which weighs as the later passes have one to five
+// iterations.  Iteration of one block / of the launches, us: planted partition of
+// 1,000 vertices, 18,000 entries: 1 class 109 / 19, 8 classes 110 / 72, 32
+// classes 149 / 205; of 8,000, 118,000: 1 class 284 / 24, 32 classes 377 / 239;
+// grid of 7,225: 1 class 36 / 18, 8 classes 62 / 65; R-MAT of 4,096, 28,900: 1
+// class 100 / 28, 32 classes 229 / 483.  The last passes of a road grid (830
+// vertices, 18,000 entries, 8 classes), one or two iterations with the set-up,
+// 90 / 175 us.
+// The graphs of a batch run beside each other, while its launches wait for the
+// host every iteration and serve all graphs: one block pays three times as long
+// (300 graphs of 8,000 vertices, 111,000 entries, 32 classes: 10.0 ms against
+// 13.9 with the line of a single graph).
+inline bool small_pays(int64_t n, int64_t entries, int classes, bool batch) {
+  if (n > kSmallVerts || entries > kSmallEntries || entries > 16384 + 4096 * (int64_t)classes) return false;
+  const bool tiny = n <= kTinyVerts;
+  const int64_t warp_rows = n < entries / 9 ? n : entries / 9;
+  const int64_t cost = warp_rows / (tiny ? 8 : 32) + entries / (tiny ? 2000 : 1000);
+  const int64_t line = 20 + 14 * (int64_t)classes;
+  return cost <= (line < 160 ? line : 160) * (batch ? 3 : 1);
 }
 struct SmallArgs {
   const int64_t* vo;

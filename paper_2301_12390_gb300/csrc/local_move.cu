@@ -994,7 +994,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
   const long long M = single ? a.M : a.Mg[g];
   // 64-bit gains and 32-bit sums must hold every vertex (as for the buckets)
   const long long klimit = M < (1ll << 31) ? M : (long long)((1ull << 61) / (unsigned long long)M);
-  int unfit = ng > NMAX || nnz > small_entries(P);
+  int unfit = ng > NMAX || nnz > kSmallEntries;
   if (!unfit)
     for (int v = tid; v < ng; v += THREADS) unfit |= a.K[v0 + v] > klimit;
   if (__syncthreads_or(unfit)) {

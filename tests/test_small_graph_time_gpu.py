@@ -2,6 +2,7 @@
 import numpy as np
 import pytest
 
+import graphgen as gg
 from engine_util import assert_sync_parity
 from paper_2301_12390_gb300 import SYNC, Louvain
 from test_degree_edges_gpu import _Csr
@@ -61,3 +62,18 @@ def test_totals_carry_across_32_bits(classes):
     assert int(K.max()) <= (1 << 61) // int(K.sum())
     _, ref = assert_sync_parity(g, prune=1, subrounds=classes)
     assert np.bincount(ref.top, weights=K).min() > 1 << 32
+
+
+def _blocks(n, degree):
+    """Blocks of about 60 vertices, three quarters of a vertex's entries inside its block."""
+    return gg.sbm(1, n, max(2, n // 60), min(1.0, 0.75 * degree / 60), 0.25 * degree / n)
+
+
+@pytest.mark.parametrize("n,degree,classes", [(1000, 19, 1), (1000, 19, 4), (600, 12, 1), (1500, 12, 1), (8000, 2.5, 1)])
+def test_one_block_only_where_it_pays(n, degree, classes):
+    # more than 32 iterations allowed: always the launches.  The first two graphs and the last took a
+    # block 2.3 to 5.8 times as long
+    g = _blocks(n, degree)
+    chosen = _iteration_ms(g, subrounds=classes, max_iterations=20)
+    launches = _iteration_ms(g, subrounds=classes, max_iterations=33)
+    assert chosen < 2 * launches
