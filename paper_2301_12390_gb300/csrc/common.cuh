@@ -69,6 +69,19 @@ __device__ __forceinline__ void atomic_add_u128(unsigned long long* lo, unsigned
   if (vhi) atomicAdd(hi, vhi);
 }
 
+// *p += v in shared memory; of 64 bits by two 32-bit atomics, the carry between
+// them (the halves agree again once every addition is done, at the next barrier).
+// A 64-bit shared atomic retries as long as others hit the same address, and the
+// leaves of a star all move to one community: 3,400 leaves 153 -> 26 us an
+// iteration of local moving, 7,900 333 -> 51.
+__device__ __forceinline__ void shared_add(unsigned* p, unsigned v) { atomicAdd(p, v); }
+__device__ __forceinline__ void shared_add(unsigned long long* p, unsigned long long v) {
+  const unsigned lo = (unsigned)v;
+  unsigned hi = (unsigned)(v >> 32);
+  if (atomicAdd((unsigned*)p, lo) > ~lo) ++hi;
+  if (hi) atomicAdd((unsigned*)p + 1, hi);
+}
+
 // The double nearest to v (ties to even): the same value as the host's
 // conversion of a 128-bit integer.  The top 64 bits keep a sticky bit for the
 // rest, so the one rounding is that of the 64-bit conversion.

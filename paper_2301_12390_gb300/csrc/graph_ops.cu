@@ -2178,7 +2178,10 @@ __global__ void __launch_bounds__(256) agg_relabel_rows_k(SmallAgg r) {
 }
 
 // Communities of more than 128 entries, a block each: their sums indexed by
-// neighbour community (k values of shared memory), whatever their size.
+// neighbour community (k values of shared memory), whatever their size.  Bound by
+// the additions to one sum when a community's entries nearly all stay inside it:
+// two blocks of 250 vertices fully joined, 64-bit sums, 2.52 -> 0.14 ms of
+// aggregation with shared_add in place of 64-bit atomics (32-bit sums 0.09).
 template <typename W2>
 __global__ void __launch_bounds__(256) agg_dense_k(AggArgs a, const int32_t* __restrict__ list,
                                                    const int64_t* __restrict__ ko, const int64_t* __restrict__ kp) {
@@ -2195,7 +2198,7 @@ __global__ void __launch_bounds__(256) agg_dense_k(AggArgs a, const int32_t* __r
   for (int64_t ci = ko[0] + blockIdx.x; ci < ko[1]; ci += gridDim.x) {
     const int32_t C = list[ci];
     const int64_t vs = a.mpre[a.cstart[C]], ve = a.mpre[a.cstart[C + 1]];
-    for (int64_t x = vs + threadIdx.x; x < ve; x += 256) atomicAdd(&sums[a.tcol[x]], (V)((const W2*)a.tw)[x]);
+    for (int64_t x = vs + threadIdx.x; x < ve; x += 256) shared_add(&sums[a.tcol[x]], (V)((const W2*)a.tw)[x]);
     __syncthreads();
     for (int t = threadIdx.x; t < k; t += 256) {
       const V v = sums[t];

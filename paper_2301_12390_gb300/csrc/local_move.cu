@@ -907,18 +907,6 @@ __global__ void __launch_bounds__(256, 3) lm_class(LMArgs<W> a, const int32_t* _
 // Vertices of degree above 128 that a graph within the entry limit can hold.
 constexpr int kSmallLong = (int)(kSmallEntries / 129) + 1;
 
-// *p += v in shared memory by two 32-bit atomics, the carry between them (the
-// halves agree again once every addition is done, at the next barrier).  A
-// 64-bit shared atomic retries as long as others hit the same address, and the
-// leaves of a star all move to one community: 3,400 leaves 153 -> 26 us an
-// iteration, 7,900 333 -> 51.
-__device__ __forceinline__ void shared_add_i64(long long* p, long long v) {
-  const unsigned lo = (unsigned)v;
-  unsigned hi = (unsigned)((unsigned long long)v >> 32);
-  if (atomicAdd((unsigned*)p, lo) > ~lo) ++hi;
-  if (hi) atomicAdd((unsigned*)p + 1, hi);
-}
-
 // One vertex's best candidate so far.
 struct SmallBest {
   long long g;
@@ -1285,8 +1273,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
         const int d = s.memb[v];
         const long long Ki = a.K[v0 + v];
         s.memb[v] = c;
-        shared_add_i64(s.sig + d, -Ki);
-        shared_add_i64(s.sig + c, Ki);
+        shared_add((unsigned long long*)(s.sig + d), (unsigned long long)(-Ki));
+        shared_add((unsigned long long*)(s.sig + c), (unsigned long long)Ki);
         atomicSub(s.size + d, 1);
         atomicAdd(s.size + c, 1);
       }

@@ -77,3 +77,20 @@ def test_one_block_only_where_it_pays(n, degree, classes):
     chosen = _iteration_ms(g, subrounds=classes, max_iterations=20)
     launches = _iteration_ms(g, subrounds=classes, max_iterations=33)
     assert chosen < 2 * launches
+
+
+def test_wide_weights_do_not_slow_the_aggregation():
+    # two blocks of 250 fully joined: their entries fall on a handful of sums, of 64 bits with large weights
+    # (27 times the time of 32-bit ones while each addition waited for the others)
+    ms = []
+    for wmax in (1, 1_000_000):
+        g = gg.sbm(1, 500, 2, 1.0, 0.002, 1, wmax)
+        with Louvain(device=0, mode=SYNC, prune=1, subrounds=4) as lv:
+            lv.load_csr(g.off, g.col, g.w)
+            best = float("inf")
+            for _ in range(7):
+                lv.run()
+                best = min(best, lv.passes()[0].agg_ms)
+            ms.append(best)
+        assert_sync_parity(g, prune=1, subrounds=4)
+    assert ms[1] < 4 * ms[0]
