@@ -539,8 +539,9 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
       const int Pg = cat == kCatSmall ? cs.Ps : cat == kCatSparse ? cs.Pl : cs.Pb;
       const int64_t nq = multi ? c->vo_host[q + 1] - c->vo_host[q] : g.n, eq = multi ? c->ent_host[q] : g.nnz;
       // of several graphs only those whose every degree suits 64-bit gains
-      // (the launch finds out for a single one)
-      if (small_pays(nq, eq, Pg, multi) && (!multi || c->gst[q].M < (1ll << 31)))
+      // (the launch finds out for a single one); asynchronous with one class, a
+      // class's moves committed together would be the synchronous schedule
+      if (!(async && Pg == 1) && small_pays(nq, eq, Pg, multi) && (!multi || c->gst[q].M < (1ll << 31)))
         (nq <= kTinyVerts ? tiny : small).push_back((int32_t)q);
       else
         any_left = true;
