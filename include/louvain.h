@@ -328,7 +328,7 @@ int louvain_get_level(louvain_ctx *ctx, int pass, int32_t *out, int64_t n);
 int louvain_get_coarse(louvain_ctx *ctx, int pass, int64_t *off, int64_t k, int32_t *col, int64_t *w,
                        int64_t nnz);
 
-/* Device bytes the context holds (arena). */
+/* Device bytes the context holds (arena; 800 bytes a graph of the largest batch loaded come on top). */
 int louvain_get_device_bytes(louvain_ctx *ctx, int64_t *bytes);
 
 /* Device bytes a context's arena needs for a graph (or a batch) of n

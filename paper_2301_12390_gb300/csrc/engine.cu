@@ -221,7 +221,10 @@ struct louvain_ctx {
   unsigned long long* d_gs = nullptr;
   unsigned long long* d_gL = nullptr;
   unsigned long long* d_gSS = nullptr;
-  int64_t hcap = 0;                    // pinned per-graph host buffers below hold hcap graphs
+  int64_t hcap = 0;                    // per-graph buffers below hold hcap graphs
+  unsigned long long* d_rec = nullptr;       // lm_launch_small's records (kSmallRec words a graph)
+  std::vector<unsigned long long> h_rec;     // as many of them as a pass needed
+  // pinned
   int32_t* h_gon = nullptr;
   int32_t* h_ids = nullptr;
   unsigned long long* h_gmoves = nullptr;
@@ -529,8 +532,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   std::vector<int32_t> tiny, small;   // the graphs done in one launch
   bool any_left = true;
   {
-    bool on = c->opt.stop_rule == 0 && c->opt.max_iterations <= kSmallIters && !c->tuning &&
-              G * kSmallRec <= c->cap_nnz;
+    bool on = c->opt.stop_rule == 0 && c->opt.max_iterations <= kSmallIters && !c->tuning;
     for (int b = 0; b < 5; ++b) on = on && c->thr.t[b] == kLMCap[b];
     if (on) any_left = false;
     for (int64_t q = 0; q < G && on; ++q) {
@@ -547,8 +549,8 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
         any_left = true;
     }
   }
-  SmallArgs sa{multi ? c->vo : nullptr, nullptr, c->d_gcat, g.n, 0, false, cs, tol, c->opt.max_iterations,
-               (unsigned long long*)c->tw};   // c->tw: free until the pass aggregates
+  SmallArgs sa{multi ? c->vo : nullptr, nullptr, c->d_gcat, g.n, 0, G, false, cs, tol, c->opt.max_iterations,
+               c->d_rec};
   const bool any_block = !tiny.empty() || !small.empty();   // some graph is done in one launch
   const bool beside = any_block && any_left;
   if (any_block) {
@@ -584,11 +586,24 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // single graph did not fit after all.
   std::vector<IterRec> small_iters;   // per iteration, summed over these graphs
   auto small_results = [&](bool* left) -> int {
-    std::vector<unsigned long long> rec(G * kSmallRec);
-    if (int r = fetch_many(c, {{rec.data(), c->tw, rec.size() * sizeof(unsigned long long)}})) return r;
+    // the first iterations' records with the counts, the others if there were more
+    std::vector<unsigned long long>& rec = c->h_rec;
+    const int64_t first = 4 + 3 * std::min(c->opt.max_iterations, 8);
+    if ((int64_t)rec.size() < first * G) rec.resize(first * G);
+    if (int r = fetch_many(c, {{rec.data(), c->d_rec, first * G * sizeof(unsigned long long)}})) return r;
+    int64_t longest = 0;
+    for (const std::vector<int32_t>* v : {&tiny, &small})
+      for (int32_t q : *v)
+        if (rec[q] <= (unsigned long long)kSmallIters) longest = std::max(longest, (int64_t)rec[q]);
+    if (4 + 3 * longest > first) {
+      if ((int64_t)rec.size() < (4 + 3 * longest) * G) rec.resize((4 + 3 * longest) * G);
+      if (int r = fetch_many(c, {{rec.data() + first * G, c->d_rec + first * G,
+                                  (4 + 3 * longest - first) * G * sizeof(unsigned long long)}}))
+        return r;
+    }
     for (const std::vector<int32_t>* v : {&tiny, &small})
       for (int32_t q : *v) {
-        const unsigned long long* r = rec.data() + q * kSmallRec;
+        const unsigned long long* r = rec.data() + q;   // word w at r[w * G]
         if (r[0] == kSmallNot && !multi) {
           *left = true;
           return 0;
@@ -596,11 +611,12 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
         if (r[0] > (unsigned long long)kSmallIters)
           return fail(c, LOUVAIN_ERR_INTERNAL, "local-moving: a small graph's launch failed");
         GraphState& st = c->gst[q];
-        edges_total += (int64_t)r[1];
-        visited_total += (int64_t)r[2];
-        cands_total += (int64_t)r[3];
+        edges_total += (int64_t)r[G];
+        visited_total += (int64_t)r[2 * G];
+        cands_total += (int64_t)r[3 * G];
         for (int64_t t = 0; t < (int64_t)r[0]; ++t) {
-          const IterRec x{pass, (int64_t)r[4 + 3 * t], ((u128)r[6 + 3 * t] << 64) | (u128)r[5 + 3 * t]};
+          const IterRec x{pass, (int64_t)r[(4 + 3 * t) * G],
+                          ((u128)r[(6 + 3 * t) * G] << 64) | (u128)r[(5 + 3 * t) * G]};
           if (multi) st.iters.push_back(x);
           st.pass_moves += x.moves;
           st.pass_iters++;
@@ -1801,6 +1817,8 @@ void arena_capacity(const louvain_ctx* c, int64_t* n, int64_t* nnz) {
 }  // namespace gbl
 
 void free_host_graph_buffers(louvain_ctx* c) {
+  if (c->d_rec) cudaFree(c->d_rec);
+  c->d_rec = nullptr;
   if (c->h_gon) cudaFreeHost(c->h_gon);
   if (c->h_ids) cudaFreeHost(c->h_ids);
   c->h_ids = nullptr;
@@ -1816,6 +1834,11 @@ void free_host_graph_buffers(louvain_ctx* c) {
 int host_graph_buffers(louvain_ctx* c, int64_t G) {
   if (c->hcap >= G) return 0;
   free_host_graph_buffers(c);
+  if (cudaMalloc(&c->d_rec, G * kSmallRec * sizeof(unsigned long long)) != cudaSuccess) {
+    cudaGetLastError();
+    c->d_rec = nullptr;
+    return fail(c, LOUVAIN_ERR_OOM, "cudaMalloc of the graphs' records failed");
+  }
   if (cudaMallocHost(&c->h_gon, G * sizeof(int32_t)) != cudaSuccess ||
       cudaMallocHost(&c->h_ids, G * sizeof(int32_t)) != cudaSuccess ||
       cudaMallocHost(&c->h_gmoves, G * sizeof(unsigned long long)) != cudaSuccess ||

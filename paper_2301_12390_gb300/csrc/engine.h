@@ -122,10 +122,11 @@ constexpr int64_t kSmallPassEntries = 1 << 21;   // CSR entries up to which a pa
 // Small graphs: the whole local-moving phase of a graph by one block, its
 // state in shared memory.  One graph (vo null: vertices [0, n)) or the `count`
 // graphs ids[0..count) of several (graph g: vertices [vo[g], vo[g + 1])); tiny:
-// all of them have at most kTinyVerts vertices.  rec: per graph kSmallRec
-// words: iterations run (kSmallNot: the graph does not fit and nothing was
-// done; kSmallErr: a table overflowed), entries scanned, vertices visited,
-// candidates, then per iteration its moves and the sum of their gains (lo, hi).
+// all of them have at most kTinyVerts vertices.  rec: kSmallRec words of each of
+// the `graphs` graphs, word w of graph g at rec[w * graphs + g]: iterations run
+// (kSmallNot: the graph does not fit and nothing was done; kSmallErr: a table
+// overflowed), entries scanned, vertices visited, candidates, then per iteration
+// its moves and the sum of their gains (lo, hi).
 constexpr int kSmallIters = 32;   // a larger max_iterations takes the launches
 constexpr int kSmallRec = 4 + 3 * kSmallIters;
 constexpr unsigned long long kSmallNot = ~0ull, kSmallErr = ~1ull;
@@ -160,7 +161,7 @@ struct SmallArgs {
   const int64_t* vo;
   const int32_t* ids;
   const int32_t* gcat;
-  int64_t n, count;
+  int64_t n, count, graphs;
   bool tiny;
   ClassSpec cs;
   double tol;

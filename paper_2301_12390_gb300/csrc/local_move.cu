@@ -975,7 +975,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
   const int64_t v0 = single ? 0 : sa.vo[g];
   const int64_t ng = (single ? sa.n : sa.vo[g + 1]) - v0;
   const int64_t nnz = a.off[v0 + ng] - a.off[v0];
-  unsigned long long* rec = sa.rec + g * kSmallRec;
+  unsigned long long* rec = sa.rec + g;   // word w at rec[w * rs]
+  const int64_t rs = sa.graphs;
   const int cat = single ? sa.cs.single_cat : sa.gcat[g];
   const int P = cat == kCatSmall ? sa.cs.Ps : cat == kCatSparse ? sa.cs.Pl : sa.cs.Pb;
   const int mode = cat == kCatSmall ? sa.cs.mode_s : sa.cs.mode_b;
@@ -1296,9 +1297,9 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
         tot += ((u128)r_hi[w] << 64) | (u128)r_lo[w];
         mv += r_moves[w];
       }
-      rec[4 + 3 * it] = mv;
-      rec[5 + 3 * it] = (unsigned long long)tot;
-      rec[6 + 3 * it] = (unsigned long long)(tot >> 64);
+      rec[(4 + 3 * it) * rs] = mv;
+      rec[(5 + 3 * it) * rs] = (unsigned long long)tot;
+      rec[(6 + 3 * it) * rs] = (unsigned long long)(tot >> 64);
       s_stop = (2.0 * u128_to_double(tot)) / MM <= sa.tol;
     }
     __syncthreads();
@@ -1333,9 +1334,9 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
       c += r_moves[w];
     }
     rec[0] = failed ? kSmallErr : (unsigned long long)it;
-    rec[1] = e;
-    rec[2] = vs;
-    rec[3] = c;
+    rec[rs] = e;
+    rec[2 * rs] = vs;
+    rec[3 * rs] = c;
   }
 }
 
