@@ -535,6 +535,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
     bool on = c->opt.stop_rule == 0 && c->opt.max_iterations <= kSmallIters && !c->tuning;
     for (int b = 0; b < 5; ++b) on = on && c->thr.t[b] == kLMCap[b];
     if (on) any_left = false;
+    int64_t steps = 0;
     for (int64_t q = 0; q < G && on; ++q) {
       if (!c->h_gon[q]) continue;
       const int cat = multi ? c->hgcat[q] : cs.single_cat;
@@ -543,10 +544,17 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
       // of several graphs only those whose every degree suits 64-bit gains
       // (the launch finds out for a single one); asynchronous with one class, a
       // class's moves committed together would be the synchronous schedule
-      if (!(async && Pg == 1) && small_pays(nq, eq, Pg, multi) && (!multi || c->gst[q].M < (1ll << 31)))
+      if (!(async && Pg == 1) && small_pays(nq, eq, Pg, multi) && (!multi || c->gst[q].M < (1ll << 31))) {
         (nq <= kTinyVerts ? tiny : small).push_back((int32_t)q);
-      else
+        steps += std::min<int64_t>(Pg, nq);
+      } else {
         any_left = true;
+      }
+    }
+    if (steps > kSmallSteps) {
+      tiny.clear();
+      small.clear();
+      any_left = true;
     }
   }
   SmallArgs sa{multi ? c->vo : nullptr, nullptr, c->d_gcat, g.n, 0, G, false, cs, tol, c->opt.max_iterations,
@@ -587,8 +595,9 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   std::vector<IterRec> small_iters;   // per iteration, summed over these graphs
   auto small_results = [&](bool* left) -> int {
     // the first iterations' records with the counts, the others if there were more
+    // (of many graphs the copy costs more than a second wait)
     std::vector<unsigned long long>& rec = c->h_rec;
-    const int64_t first = 4 + 3 * std::min(c->opt.max_iterations, 8);
+    const int64_t first = 4 + 3 * std::min(c->opt.max_iterations, G > 4096 ? 2 : 8);
     if ((int64_t)rec.size() < first * G) rec.resize(first * G);
     if (int r = fetch_many(c, {{rec.data(), c->d_rec, first * G * sizeof(unsigned long long)}})) return r;
     int64_t longest = 0;

@@ -157,6 +157,13 @@ inline bool small_pays(int64_t n, int64_t entries, int classes, bool batch) {
   const int64_t line = 20 + 14 * (int64_t)classes;
   return cost <= (line < 160 ? line : 160) * (batch ? 3 : 1);
 }
+// Classes that the blocks of a batch may walk in one iteration in all: more graphs
+// than that fill the chip either way, and the launches walk their classes
+// together.  Pass 0, one block / launches: 30,000 graphs of 150 vertices, 32
+// classes 22.1 / 21.5 ms (its pass 1 12.1 / 18.6), 50,000 of 24 14.2 / 14.3,
+// 100,000 of 24 28.7 / 25.2, 100,000 of 60 51.3 / 36.5; with one class
+// 100,000 of 60 53 / 86.
+constexpr int64_t kSmallSteps = 1500000;
 struct SmallArgs {
   const int64_t* vo;
   const int32_t* ids;
