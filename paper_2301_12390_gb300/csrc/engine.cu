@@ -805,7 +805,16 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // are drawn anew every iteration draws them inside the sequence, except in
   // iteration 0, whose classes the first classification drew.
   bool drawn = true;
+  // A synchronous class's moves (at most m).  The commit clears the next class's
+  // counter, so the counters change hands with it: a class without vertices has
+  // no commit, and the class after it goes on with the same counter.
+  auto commit = [&](int64_t m) {
+    if (m <= 0) return;
+    lm_launch_commit<W>(a, m, s);
+    a.odd ^= 1;
+  };
   auto iteration = [&]() -> int {
+    a.odd = 0;   // both counters are zero
     if (!ahead) CK(cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), s));
     if (multi) {
       CK(cudaMemsetAsync(c->d_gmoves, 0, G * sizeof(unsigned long long), s));
@@ -816,9 +825,8 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
     if (redraw && !drawn) draw(redraw_m, redraw_sub);
     drawn = false;
     for (int ch = 0; ch < P && small_pass; ++ch) {
-      a.odd = ch & 1;
       lm_launch_class<W>(a, wide_bucket(0) || wide_bucket(1) || wide_bucket(2), async, c->list, c->key_off, P, ch, class_grid_verts, s);
-      if (!async) lm_launch_commit<W>(a, ko[3 * P], s);
+      if (!async) commit(ko[3 * P]);
       CKLAUNCH();
     }
     // Asynchronous, with bucket_streams: every degree bucket runs the classes
@@ -861,7 +869,6 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
       }
     }
     for (int ch = 0; ch < P && !small_pass && !streams; ++ch) {
-      a.odd = ch & 1;
       // fork: every non-empty bucket of the class on its own stream
       bool used[kBuckets] = {};
       CK(cudaEventRecord(c->ev_fork, s));
@@ -894,7 +901,7 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
       if (!async) {
         int64_t cls = 0;
         for (int b = 0; b <= kHubBucket; ++b) cls += class_size(b, ch);
-        lm_launch_commit<W>(a, cls, s);
+        commit(cls);
       }
       CKLAUNCH();
     }
