@@ -813,7 +813,7 @@ __global__ void __launch_bounds__(256, 4) lm_warp(LMArgs<W> a, const int32_t* __
     }
     for (; live; live &= live - 1) {
       const VertexRow v = window_row(a, r, __ffs(live) - 1);
-      const bool on = warp_vertex<W, WIDE, ASYNC, CAP, U, (ASYNC ? 1 : 0), (CAP <= 64 && !WIDE), PULL>(
+      const bool on = warp_vertex<W, WIDE, ASYNC, CAP, U, (ASYNC ? 1 : 0), false, PULL>(
           a, iv, acc, keys, vals, v, lane, ok, tally.cands);
       if (PULL && a.pull_check && on && lane == 0) {
         tally.edges += (unsigned)v.deg;
@@ -1850,7 +1850,7 @@ void launch_bucket_t(const LMArgs<W>& a, int bucket, const int32_t* list, const 
       break;
     }
     case 1: {
-      if (!WIDE) {   // narrow sums: a lane per vertex, its row sorted in registers
+      if constexpr (!WIDE) {   // narrow sums: a lane per vertex, its row sorted in registers
         auto k = lm_thread_sorted<W, ASYNC, PULL, 32>;
         (count_launch(), k<<<grid_for(k, 128, 0, (nverts + 127) / 128), 128, 0, s>>>(a, list, ko));
       } else {
