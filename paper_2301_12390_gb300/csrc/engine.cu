@@ -594,10 +594,10 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
   // single graph did not fit after all.
   std::vector<IterRec> small_iters;   // per iteration, summed over these graphs
   auto small_results = [&](bool* left) -> int {
-    // the first iterations' records with the counts, the others if there were more
-    // (of many graphs the copy costs more than a second wait)
+    // the records of all iterations with the counts; of many graphs, where the copy
+    // costs more than a second wait, the first iterations' and the others if they ran
     std::vector<unsigned long long>& rec = c->h_rec;
-    const int64_t first = 4 + 3 * std::min(c->opt.max_iterations, G > 4096 ? 2 : 8);
+    const int64_t first = 4 + 3 * std::min(c->opt.max_iterations, G > 4096 ? 2 : G > 256 ? 8 : kSmallIters);
     if ((int64_t)rec.size() < first * G) rec.resize(first * G);
     if (int r = fetch_many(c, {{rec.data(), c->d_rec, first * G * sizeof(unsigned long long)}})) return r;
     int64_t longest = 0;

@@ -975,8 +975,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
   const int64_t v0 = single ? 0 : sa.vo[g];
   const int64_t ng = (single ? sa.n : sa.vo[g + 1]) - v0;
   const int64_t nnz = a.off[v0 + ng] - a.off[v0];
-  unsigned long long* rec = sa.rec + g;   // word w at rec[w * rs]
-  const int64_t rs = sa.graphs;
+  auto rec = [&](int w) -> unsigned long long& { return sa.rec[w * sa.graphs + g]; };
   const int cat = single ? sa.cs.single_cat : sa.gcat[g];
   const int P = cat == kCatSmall ? sa.cs.Ps : cat == kCatSparse ? sa.cs.Pl : sa.cs.Pb;
   const int mode = cat == kCatSmall ? sa.cs.mode_s : sa.cs.mode_b;
@@ -987,7 +986,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
   if (!unfit)
     for (int v = tid; v < ng; v += THREADS) unfit |= a.K[v0 + v] > klimit;
   if (__syncthreads_or(unfit)) {
-    if (tid == 0) rec[0] = kSmallNot;
+    if (tid == 0) rec(0) = kSmallNot;
     return;
   }
   const int n = (int)ng;
@@ -1297,9 +1296,9 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
         tot += ((u128)r_hi[w] << 64) | (u128)r_lo[w];
         mv += r_moves[w];
       }
-      rec[(4 + 3 * it) * rs] = mv;
-      rec[(5 + 3 * it) * rs] = (unsigned long long)tot;
-      rec[(6 + 3 * it) * rs] = (unsigned long long)(tot >> 64);
+      rec(4 + 3 * it) = mv;
+      rec(5 + 3 * it) = (unsigned long long)tot;
+      rec(6 + 3 * it) = (unsigned long long)(tot >> 64);
       s_stop = (2.0 * u128_to_double(tot)) / MM <= sa.tol;
     }
     __syncthreads();
@@ -1333,10 +1332,10 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 4 : 1) lm_small(LMAr
       vs += r_hi[w];
       c += r_moves[w];
     }
-    rec[0] = failed ? kSmallErr : (unsigned long long)it;
-    rec[rs] = e;
-    rec[2 * rs] = vs;
-    rec[3 * rs] = c;
+    rec(0) = failed ? kSmallErr : (unsigned long long)it;
+    rec(1) = e;
+    rec(2) = vs;
+    rec(3) = c;
   }
 }
 
