@@ -81,7 +81,9 @@ typedef struct {
                                  the other in each iteration; 1 = every vertex at once; 0 = automatic
                                  (synchronous 1; asynchronous, per graph: 32 for a graph of fewer than
                                  65,536 vertices, else 8 for a graph of fewer than 8 entries per vertex,
-                                 else 16) */
+                                 else 16).  Synchronous moves take effect when their class is done,
+                                 asynchronous ones at once, except that a pass graph of a few thousand
+                                 vertices may apply those of a class together (P >= 2) */
   int32_t validate;           /* 1: louvain_load_csr checks symmetry and CSR form (costs a pass) */
   int32_t record_levels;      /* 1: keep each pass's membership and coarse CSR for louvain_get_level /
                                  louvain_get_coarse (copies them to host memory) */
@@ -89,8 +91,8 @@ typedef struct {
                                  as one captured CUDA graph instead of individual launches (default 0:
                                  measured slower on the benchmark graphs).  Either way the engine
                                  captures the iterations that last less than their launches: small
-                                 passes of several classes, and synchronous passes of at most 8M
-                                 entries from their fifth iteration */
+                                 passes of several classes, and, from their fifth iteration, passes of
+                                 at most 8M entries whose classes are not drawn anew every iteration */
   int32_t reclass;            /* asynchronous mode with P > 1: 0 = classes id mod P; 1 = each
                                  iteration draws the classes anew, class = hash(id, pass, iteration)
                                  mod P (breaks the repeated same-class swaps of structured ids such

@@ -63,8 +63,9 @@ constexpr int64_t kEdgeListRatio = 4;
 // R-MAT visits nearly all, any share gives 100.5 (116.8 pushed); a 2048 x 2048
 // grid in colour classes 14.0 (14.25).
 constexpr double kPullFraction = 0.75;
-// A synchronous pass of up to this many entries is shorter on the GPU than its
-// launches on the host.
+// A pass of up to this many entries whose lists are drawn once (synchronous; or
+// asynchronous with classes fixed for the pass, as by default below 65,536
+// vertices) is shorter on the GPU than its launches on the host.
 constexpr int64_t kGraphEntries = 8 << 20;
 
 struct IterRec {
