@@ -133,18 +133,18 @@ constexpr unsigned long long kSmallNot = ~0ull, kSmallErr = ~1ull;
 constexpr int64_t kSmallVerts = 8192, kTinyVerts = 1024;   // vertices whose state fits a block's shared memory
 constexpr int64_t kSmallEntries = 131072;   // entries of a graph that one block takes at most
 // Whether one block pays.  Its iteration costs about 10 us, 3-4 a class, one for
-// each round of its warps over the vertices of more than 8 entries (at most
-// min(n, e / 9), a warp each) and the long rows that the whole block takes one by
-// one (e / 1000 allows for them; of a tiny graph a warp takes them too).  The
-// launches' iteration costs about 13 us and 7 a class (15 with a long row), and a
-// phase 100 to set up, which weighs as the later passes have one to five
-// iterations.  Iteration of one block / of the launches, us: planted partition of
-// 1,000 vertices, 18,000 entries: 1 class 109 / 19, 8 classes 110 / 72, 32
-// classes 149 / 205; of 8,000, 118,000: 1 class 284 / 24, 32 classes 377 / 239;
-// grid of 7,225: 1 class 36 / 18, 8 classes 62 / 65; R-MAT of 4,096, 28,900: 1
-// class 100 / 28, 32 classes 229 / 483.  The last passes of a road grid (830
-// vertices, 18,000 entries, 8 classes), one or two iterations with the set-up,
-// 90 / 175 us.
+// each round of its warps over the rows of more than 8 entries (a warp each; of n
+// rows about (e - 4 n) / 10 are that long, and e / 50 of a heavy tail), one for
+// each 256 vertices (64 of a tiny graph's fewer threads), and the long rows that
+// the whole block takes one by one (e / 1000 allows for them).  The launches'
+// iteration costs about 13 us and 7 a class (15 with a long row), and a phase 100
+// to set up, which weighs as the later passes have one to five iterations.
+// Iteration of one block / of the launches, us: planted partition of 1,000
+// vertices, 18,000 entries: 1 class 109 / 19, 8 classes 110 / 72, 32 classes 149 /
+// 205; of 8,000, 118,000: 1 class 284 / 24, 32 classes 377 / 239; grid of 7,225: 1
+// class 36 / 18, 8 classes 62 / 65; R-MAT of 4,096, 28,900: 1 class 100 / 28, 32
+// classes 229 / 483.  The last passes of a road grid (830 vertices, 18,000
+// entries, 8 classes), one or two iterations with the set-up, 90 / 175 us.
 // The graphs of a batch run beside each other, while its launches wait for the
 // host every iteration and serve all graphs: one block pays three times as long
 // (300 graphs of 8,000 vertices, 111,000 entries, 32 classes: 10.0 ms against
@@ -152,10 +152,12 @@ constexpr int64_t kSmallEntries = 131072;   // entries of a graph that one block
 inline bool small_pays(int64_t n, int64_t entries, int classes, bool batch) {
   if (n > kSmallVerts || entries > kSmallEntries || entries > 16384 + 4096 * (int64_t)classes) return false;
   const bool tiny = n <= kTinyVerts;
-  const int64_t warp_rows = n < entries / 9 ? n : entries / 9;
-  const int64_t cost = warp_rows / (tiny ? 8 : 32) + entries / (tiny ? 2000 : 1000);
-  const int64_t line = 20 + 14 * (int64_t)classes;
-  return cost <= (line < 160 ? line : 160) * (batch ? 3 : 1);
+  int64_t rows = (entries > 4 * n ? (entries - 4 * n) / 10 : 0) + entries / 50;
+  if (rows > n) rows = n;
+  const int64_t listed = n < entries ? n : entries;
+  const int64_t cost = rows / (tiny ? 8 : 32) + listed / (tiny ? 64 : 256) + entries / (tiny ? 2000 : 1000);
+  const int64_t few = 20 + 16 * (int64_t)classes, many = 152 + classes;
+  return cost <= (few < many ? few : many) * (batch ? 3 : 1);
 }
 // Classes that the blocks of a batch may walk in one iteration in all: more graphs
 // than that fill the chip either way, and the launches walk their classes
