@@ -48,9 +48,10 @@ L2_BYTES = 126 << 20   # GB300 L2 (about 126 MB)
 # DRAM bytes the local-moving phase moves per algorithmic byte, from one ncu
 # capture (dram__bytes_read.sum + dram__bytes_write.sum) of every
 # local-moving launch of an asynchronous R-MAT s22 run with L2 kept between
-# launches: 13.07 GB for 4.66 GB of algorithmic bytes.  Taken on the current
-# kernels; None where no capture was taken.
-LM_TRAFFIC_PER_BYTE = {("rmat22", "async"): 1.94}
+# launches: 9.41 GB for 5.11 GB of algorithmic bytes in pass 0
+# (profiles/lm_traffic_rmat22_async_run.md names the commit); null where no
+# capture was taken.
+LM_TRAFFIC_PER_BYTE = {("rmat22", "async"): 1.84}
 UNIT = "edges/s"
 
 
