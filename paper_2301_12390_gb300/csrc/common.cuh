@@ -437,6 +437,7 @@ struct LMArgs {
   // the flags of the neighbours' memberships; its moves set flags, not stamps
   int pull_check, pull_mark;
   // hub path: per-hub global tables (2 deg slots each, per class from slot 0)
+  int hchunk;                // entries per insert chunk
   int32_t* hkeys;
   unsigned long long* hvals;
   const int64_t* hbase;      // table offset of hub h (the class's first hub at hbase[0])

@@ -715,7 +715,10 @@ int local_moving(louvain_ctx* c, const PassState& g, int pass, double tol, bool 
     hub1 = ko[kHubBucket * P + P];
     nhubs = hub1 - hub0;
     if (nhubs > 0) {
-      hub_layout(g.off, c->list + hub0, nhubs, c->gbase, c->chunk_pre, c->spre, c->tmp, s);
+      const int launches = async ? std::min(P, kHubGroups) : 1;
+      const int64_t least = thr.t[4] < kBlockDegree ? thr.t[4] : thr.big;
+      a.hchunk = hub_chunk(nhubs, least, launches);
+      hub_layout(g.off, c->list + hub0, nhubs, a.hchunk, c->gbase, c->chunk_pre, c->spre, c->tmp, s);
       CKLAUNCH();
       hchunks.resize(nhubs + 1);
       hschunks.resize(nhubs + 1);

@@ -40,7 +40,17 @@ __host__ __device__ inline int lm_bucket_of(int64_t deg, const LMThresholds& th)
     if (deg <= th.t[b]) return b;
   return deg > kBlockDegree && deg <= th.big ? kBigBucket : kHubBucket;
 }
-constexpr int64_t kHubChunkEntries = 4096;   // entries per insert block of a hub
+// Entries per insert block of a hub: long chunks where the hubs fill the chip with
+// them (kHubLongBlocks, of an asynchronous iteration's `launches`), else short
+// ones, whose blocks finish sooner: the hubs' launches are the longest chain of an
+// asynchronous iteration.  Asynchronous R-MAT, pass 0 of three iterations, long /
+// short: scale 17 1.69 / 1.46 ms, 18 1.92 / 1.67, 19 2.92 / 2.43, 20 3.08 / 2.83, 21
+// 4.14 / 4.12; synchronous runs of 4.2M vertices 98.8 / 99.6, of 1M with four
+// classes 11.43 / 11.54, of 75,879 4.54 / 4.49.
+constexpr int kHubShortChunk = 1024, kHubLongChunk = 4096, kHubLongBlocks = 48;
+inline int hub_chunk(int64_t nhubs, int64_t least_degree, int launches) {
+  return nhubs * least_degree >= (int64_t)kHubLongBlocks * kHubLongChunk * launches ? kHubLongChunk : kHubShortChunk;
+}
 constexpr int64_t kSlotChunk = 4096;         // table slots per scan block (hubs and large communities)
 
 // Community classes of the aggregation phase by total member degree.
@@ -240,8 +250,9 @@ struct DrawArgs {
 void draw_lists_stable(const DrawArgs& d, int32_t* key, int32_t* list, int64_t* key_off, void* tmp, cudaStream_t s);
 void draw_lists(const DrawArgs& d, uint16_t* key, int32_t* list, int64_t* key_off, unsigned* scratch, cudaStream_t s);
 // For the hub list: per hub its table base (2 * degree slots), the prefix of
-// its insert chunks and the prefix of its slot chunks (each nhubs + 1 long).
-void hub_layout(const int64_t* off, const int32_t* hubs, int64_t nhubs, int64_t* hbase, int64_t* chunk_pre,
+// its insert chunks (of `chunk` entries) and the prefix of its slot chunks (each
+// nhubs + 1 long).
+void hub_layout(const int64_t* off, const int32_t* hubs, int64_t nhubs, int chunk, int64_t* hbase, int64_t* chunk_pre,
                 int64_t* spre, void* tmp, cudaStream_t s);
 
 // Row sums K (int64) of a CSR, the total M (u128 lo/hi) and the self-loop

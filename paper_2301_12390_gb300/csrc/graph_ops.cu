@@ -478,17 +478,17 @@ void draw_lists(const DrawArgs& d, uint16_t* key, int32_t* list, int64_t* key_of
   (count_launch(), draw_scatter_k<<<(unsigned)((d.m + kDrawTile - 1) / kDrawTile), kT, smem, s>>>(d, key, cursor, list));
 }
 
-__global__ void hub_sizes_k(const int64_t* off, const int32_t* hubs, int64_t nhubs, int64_t* cap, int64_t* chunks,
-                            int64_t* schunks) {
+__global__ void hub_sizes_k(const int64_t* off, const int32_t* hubs, int64_t nhubs, int chunk, int64_t* cap,
+                            int64_t* chunks, int64_t* schunks) {
   for (int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; h < nhubs; h += (int64_t)gridDim.x * blockDim.x) {
     int64_t d = off[hubs[h] + 1] - off[hubs[h]];
     cap[h] = 2 * d;
-    chunks[h] = (d + kHubChunkEntries - 1) / kHubChunkEntries;
+    chunks[h] = (d + chunk - 1) / chunk;
     schunks[h] = (2 * d + kSlotChunk - 1) / kSlotChunk;
   }
 }
 
-void hub_layout(const int64_t* off, const int32_t* hubs, int64_t nhubs, int64_t* hbase, int64_t* chunk_pre,
+void hub_layout(const int64_t* off, const int32_t* hubs, int64_t nhubs, int chunk, int64_t* hbase, int64_t* chunk_pre,
                 int64_t* spre, void* tmp, cudaStream_t s) {
   if (nhubs <= 0) {
     cudaMemsetAsync(hbase, 0, sizeof(int64_t), s);
@@ -500,7 +500,7 @@ void hub_layout(const int64_t* off, const int32_t* hubs, int64_t nhubs, int64_t*
   int64_t* chunks = cap + nhubs;
   int64_t* schunks = chunks + nhubs;
   void* stmp = (void*)(schunks + nhubs);
-  (count_launch(), hub_sizes_k<<<grid1d(nhubs), kT, 0, s>>>(off, hubs, nhubs, cap, chunks, schunks));
+  (count_launch(), hub_sizes_k<<<grid1d(nhubs), kT, 0, s>>>(off, hubs, nhubs, chunk, cap, chunks, schunks));
   scan_i64(cap, hbase, nhubs, hbase + nhubs, stmp, s);
   scan_i64(chunks, chunk_pre, nhubs, chunk_pre + nhubs, stmp, s);
   scan_i64(schunks, spre, nhubs, spre + nhubs, stmp, s);

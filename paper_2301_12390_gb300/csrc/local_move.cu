@@ -1565,7 +1565,7 @@ __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ?
 // Hub h of a class owns global table slots [hbase[h] - hbase[0], + 2 deg):
 // every class's tables start at slot 0, so a class reuses the slots the
 // previous class's scan just cleared, which are still in L2.
-// 1. insert: blocks are (hub, kHubChunkEntries-entry chunk) pairs; each sums its chunk
+// 1. insert: blocks are (hub, a.hchunk-entry chunk) pairs; each sums its chunk
 //    per community in shared memory, then adds each distinct community once
 //    to the hub's global table;
 // 2. scan: blocks are (hub, 4096-slot chunk) pairs; each evaluates the gain
@@ -1574,21 +1574,17 @@ __global__ void __launch_bounds__(THREADS, THREADS <= 128 ? 8 : THREADS <= 512 ?
 //    chunk bests and commits;
 // 3. mark (once per iteration, all classes): neighbours of the hubs that moved.
 
-constexpr int kHubChunk = (int)kHubChunkEntries;
-
 constexpr int kItemCache = 512;   // hub prefix entries a block copies to shared memory
 
-constexpr int kHubThreads = 512;
-
-template <typename W, bool WIDE, bool ASYNC, bool PULL>
-__global__ void __launch_bounds__(kHubThreads) lm_hub_insert(LMArgs<W> a, const int32_t* __restrict__ hubs, int nhubs,
-                                                             const int64_t* __restrict__ chunk_pre) {
+template <typename W, bool WIDE, bool ASYNC, bool PULL, int CHUNK, int THREADS>
+__global__ void __launch_bounds__(THREADS) lm_hub_insert(LMArgs<W> a, const int32_t* __restrict__ hubs, int nhubs,
+                                                         const int64_t* __restrict__ chunk_pre) {
   typedef typename TableVal<WIDE>::T V;
   const IterView iv = iter_view(a);
   if (iv.iter < 0) return;
-  constexpr int CAP = 2 * kHubChunk;
-  constexpr int U = kHubChunk / kHubThreads;
-  static_assert(U >= 1 && kHubChunk % kHubThreads == 0, "a chunk covers whole rounds of the block");
+  constexpr int CAP = 2 * CHUNK;
+  constexpr int U = CHUNK / THREADS;
+  static_assert(U >= 1 && CHUNK % THREADS == 0, "a chunk covers whole rounds of the block");
   extern __shared__ unsigned long long hdyn[];
   V* svals = (V*)hdyn;
   int32_t* skeys = (int32_t*)(svals + CAP);
@@ -1599,18 +1595,18 @@ __global__ void __launch_bounds__(kHubThreads) lm_hub_insert(LMArgs<W> a, const 
   if (!is_active<PULL>(a, iv, v.i)) return;   // uniform across the block
   if (!graph_of(a, v.i, &v.M, &v.graph)) return;
   const int64_t q = (int64_t)blockIdx.x - (chunk_pre[h] - chunk_pre[0]);
-  for (int t = threadIdx.x; t < CAP; t += kHubThreads) { skeys[t] = kEmpty; svals[t] = 0; }
+  for (int t = threadIdx.x; t < CAP; t += THREADS) { skeys[t] = kEmpty; svals[t] = 0; }
   __syncthreads();
   const int64_t b = a.off[v.i], e = a.off[v.i + 1];
   const int64_t base = a.hbase[h] - a.hbase[0];   // the class's tables start at slot 0
   const uint32_t cap = (uint32_t)(2 * (e - b));
-  v.b = b + q * kHubChunk;
-  v.deg = (int)min((int64_t)kHubChunk, e - v.b);
+  v.b = b + q * CHUNK;
+  v.deg = (int)min((int64_t)CHUNK, e - v.b);
   bool ok = true;
   int32_t cc[U];
   V ww[U];
   int hs[U];
-  const int32_t seen = row_communities<U, (ASYNC ? 1 : 0), PULL>(a, v, (int)threadIdx.x, kHubThreads, U, cc, ww);
+  const int32_t seen = row_communities<U, (ASYNC ? 1 : 0), PULL>(a, v, (int)threadIdx.x, THREADS, U, cc, ww);
   // a neighbour moved: the scan finds the hub active
   if (PULL && a.pull_check && __any_sync(0xffffffffu, (seen & moved_bit(iv.iter - 1)) != 0) && (threadIdx.x & 31) == 0)
     a.hmoved[h] = -(iv.iter + 1);
@@ -1744,7 +1740,7 @@ __global__ void __launch_bounds__(256) lm_hub_scan(LMArgs<W> a, const int32_t* _
 
 // Pruning marks of the hubs that moved in this iteration (all classes at
 // once; the marks only feed the next iteration's active set): blocks are
-// (hub, kHubChunkEntries-entry chunk) pairs of the pass's whole hub list.
+// (hub, a.hchunk-entry chunk) pairs of the pass's whole hub list.
 template <typename W>
 __global__ void __launch_bounds__(256) lm_hub_mark(LMArgs<W> a, const int32_t* __restrict__ hubs, int nhubs,
                                                    const int64_t* __restrict__ chunk_pre) {
@@ -1756,7 +1752,7 @@ __global__ void __launch_bounds__(256) lm_hub_mark(LMArgs<W> a, const int32_t* _
   const int32_t i = hubs[h];
   const int64_t q = (int64_t)blockIdx.x - (chunk_pre[h] - chunk_pre[0]);
   const int64_t b = a.off[i], e = a.off[i + 1];
-  const int64_t x0 = b + q * kHubChunk, x1 = min(e, x0 + kHubChunk);
+  const int64_t x0 = b + q * a.hchunk, x1 = min(e, x0 + a.hchunk);
   if (q == 0 && threadIdx.x == 0) iv.sw[i] = iv.iter + 1;
   mark_row<4>(a, iv, i, x0, x1, (int)threadIdx.x, 256, false);   // the hub itself: marked above
 }
@@ -1894,14 +1890,23 @@ void lm_launch_bucket(const LMArgs<W>& a, bool wide, bool async, int bucket, con
   }
 }
 
+template <typename W, bool WIDE, bool ASYNC, bool PULL, int CHUNK, int THREADS>
+static void launch_hub_insert_t(const LMArgs<W>& a, const int32_t* hubs, int nhubs, const int64_t* chunk_pre,
+                                int64_t nchunks, cudaStream_t s) {
+  const size_t smem = (size_t)(2 * CHUNK) * (sizeof(typename TableVal<WIDE>::T) + 4);
+  auto k = lm_hub_insert<W, WIDE, ASYNC, PULL, CHUNK, THREADS>;
+  static std::atomic<unsigned long long> attr{0};
+  smem_limit_once(attr, k, smem);
+  (count_launch(), k<<<(unsigned)nchunks, THREADS, smem, s>>>(a, hubs, nhubs, chunk_pre));
+}
+
 template <typename W, bool WIDE, bool ASYNC, bool PULL>
 static void launch_hubs_t(const LMArgs<W>& a, const int32_t* hubs, int nhubs, const int64_t* chunk_pre,
                           int64_t nchunks, int64_t nslotchunks, cudaStream_t s) {
-  const size_t smem = (size_t)(2 * kHubChunk) * (sizeof(typename TableVal<WIDE>::T) + 4);
-  auto k = lm_hub_insert<W, WIDE, ASYNC, PULL>;
-  static std::atomic<unsigned long long> attr{0};
-  smem_limit_once(attr, k, smem);
-  (count_launch(), k<<<(unsigned)nchunks, kHubThreads, smem, s>>>(a, hubs, nhubs, chunk_pre));
+  if (a.hchunk == kHubLongChunk)
+    launch_hub_insert_t<W, WIDE, ASYNC, PULL, kHubLongChunk, 512>(a, hubs, nhubs, chunk_pre, nchunks, s);
+  else
+    launch_hub_insert_t<W, WIDE, ASYNC, PULL, kHubShortChunk, 256>(a, hubs, nhubs, chunk_pre, nchunks, s);
   (count_launch(), lm_hub_scan<W, WIDE, ASYNC, PULL><<<(unsigned)nslotchunks, 256, 0, s>>>(a, hubs, nhubs));
 }
 

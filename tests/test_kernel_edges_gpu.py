@@ -78,3 +78,12 @@ def test_one_block_with_large_totals(n):
     assert int(K.sum()) > 1 << 32 and int(K.max()) <= (1 << 61) // int(K.sum())
     for opt in ({}, {"prune": 1, "subrounds": 4}, {"colour_classes": 1}):
         assert_sync_parity(g, **opt)
+
+
+@pytest.mark.parametrize("hubs", [6, 30])   # insert chunks of 1,024 entries; from 16 hubs of one class on, of 4,096
+@pytest.mark.parametrize("wmax", [3, 1 << 29])
+@pytest.mark.parametrize("opt", [{"prune": 0}, {"prune": 1}, {"prune": 1, "subrounds": 3}], ids=str)
+def test_hub_chunks(hubs, wmax, opt):
+    # degrees at the ends of both chunk lengths
+    degrees = np.resize([12289, 13312, 13313, 16383, 16384, 16385], hubs)
+    assert_sync_parity(_edges(degrees, 1, wmax, pool=20000), max_iterations=4, max_passes=2, **opt)
